@@ -117,50 +117,80 @@ struct TileInfo {
   int v, k, x, y, W, H, tx, ty;
 };
 
-// Compacts the staged entries [0, cnt) whose rectangle meets the warp's region (origin RX,
-// RY; 8 x 8 pixels for PPT = 2, 16 x 8 for PPT = 4) into list[], in entry order, as
-// entry | (region columns the rectangle spans) << 8 | (region rows it spans) << 24: bit c
-// of the column mask for column RX + c, bit r of the row mask for row RY + r.  A lane's
-// slot test is then two bit extractions (slot_mask).  One lane tests one entry, 32 at a
-// time; returns the number listed.
-template <int PPT>
-__device__ __forceinline__ int compact_entries(const float4* sB, const float4* sC, int cnt,
-                                               int RX, int RY, int lane, uint32_t* list) {
-  constexpr int RW = PPT == 4 ? 16 : 8;  // region width
-  int nl = 0;
-  for (int g0 = 0; g0 < cnt; g0 += 32) {
-    const int e = g0 + lane;
-    uint32_t item = 0;
-    if (e < cnt) {
-      const uint32_t rx = __float_as_uint(sB[e].w), ry = __float_as_uint(sC[e].w);
-      const int c0 = max((int)(rx & 0xFFFFu) - RX, 0), c1 = min((int)(rx >> 16) - RX, RW - 1);
-      const int r0 = max((int)(ry & 0xFFFFu) - RY, 0), r1 = min((int)(ry >> 16) - RY, 7);
-      if (c0 <= c1 && r0 <= r1) {
-        const uint32_t cm = ((2u << (c1 - c0)) - 1u) << c0;
-        const uint32_t rm = ((2u << (r1 - r0)) - 1u) << r0;
-        item = (uint32_t)e | (cm << 8) | (rm << 24);
-      }
-    }
-    const unsigned hit = __ballot_sync(0xffffffffu, item != 0u);
-    if (item) list[nl + __popc(hit & ((1u << lane) - 1u))] = item;
-    nl += __popc(hit);
-  }
-  __syncwarp();
-  return nl;
+// ---- the forward's warp lists -----------------------------------------------------------
+// A warp copies the staged entries that can reach a pixel of its region (8 x 8 pixels for
+// PPT = 2, 16 x 8 for PPT = 4), in entry order, into a ring of kRingItems items of shared
+// memory, laid out two entries side by side (kPairWords words per pair):
+//   [u0 u1 v0 v1] [qa0 qa1 qb0 qb1] [qc0 qc1 o0 o1] [r0 g0 b0 d0] [r1 g1 b1 d1] [m0 m1 j0 j1]
+// so that the conic of both entries is evaluated by packed FP32 instructions without moving
+// a register.  m: the region's columns (bits 8 and up) and rows (bits 24 and up) that the
+// entry's rectangle spans; j: the entry's position in the tile's list.
+constexpr int kRingItems = 64;
+constexpr int kPairWords = 28;  // 24 used; the stride spreads the pairs over the banks
+constexpr uint32_t kDeadPixel = 1u;  // a pixel's mask once it takes nothing more (bit 0 of m is 0)
+
+// Whether an entry with conic (qa, qb, qc), opacity o and centre (u, v) may reach alpha >=
+// alpha_min in the box [X0, X1] x [Y0, Y1] (offsets from the centre): its exponent's maximum
+// over the box, with a margin above the rounding of this evaluation and of pixel_alpha's
+// (at most a few 1e-7 of the terms' sum, and |qb x y| <= |qa| x^2 + |qc| y^2), against
+// lg_amin - log2(o).  The form is concave: its maximum over the box is 0 if that holds the
+// centre and else lies on an edge facing the centre, at the edge's clamped stationary point;
+// the other candidate is some point of the box and so never above it.  NaN keeps the entry.
+__device__ __forceinline__ bool box_reached(float qa, float qb, float qc, float o, float X0,
+                                            float X1, float Y0, float Y1, float lg_amin) {
+  const float x1 = fminf(fmaxf(0.0f, X0), X1), y2 = fminf(fmaxf(0.0f, Y0), Y1);
+  const float y1 = fminf(fmaxf(-0.5f * qb * rcp_approx(qc) * x1, Y0), Y1);
+  const float x2 = fminf(fmaxf(-0.5f * qb * rcp_approx(qa) * y2, X0), X1);
+  const float p1 = fmaf(fmaf(qa, x1, qb * y1), x1, qc * y1 * y1);
+  const float p2 = fmaf(fmaf(qa, x2, qb * y2), x2, qc * y2 * y2);
+  const float best = p1 > p2 ? p1 : p2;
+  const float xm = fmaxf(fabsf(X0), fabsf(X1)), ym = fmaxf(fabsf(Y0), fabsf(Y1));
+  const float margin = fmaf(-8e-6f, fmaf(qa * xm, xm, qc * ym * ym), 2e-3f);
+  return !(best + margin < lg_amin - __log2f(o));
 }
 
-// Slots of the lane at column lx, row ly of its 8 x 4 blocks whose pixel lies in the
-// rectangle of a compacted list item: bit i for slot i (pixel column lx + 8 col(i), row
-// ly + 4 row(i) of the region).
+// Tests the staged entries e0 + lane (< cnt) of one group of 32 against the warp's region
+// (its origin RX, RY on the image, rx0, ry0 in the tile) and appends those that may reach it
+// at ring position `tail`; returns the new tail.  Staged: a, b, c of the record with the
+// rectangle's words replaced by the tile's columns (b.w) and rows (c.w) that it spans.
+// pos0: list position of staged entry 0.
 template <int PPT>
-__device__ __forceinline__ unsigned slot_mask(uint32_t item, int lx, int ly) {
-  const uint32_t cs = item >> (8 + lx), rs = item >> (24 + ly);
-  const uint32_t c0 = cs & 1u, r0 = rs & 1u, r1 = (rs >> 4) & 1u;
-  if (PPT == 4) {
-    const uint32_t c1 = (cs >> 8) & 1u;
-    return (c0 & r0) | ((c1 & r0) << 1) | ((c0 & r1) << 2) | ((c1 & r1) << 3);
+__device__ __forceinline__ unsigned append_group(const float4* sA, const float4* sB,
+                                                 const float4* sC, int e0, int cnt, int pos0,
+                                                 int RX, int RY, int rx0, int ry0, int lane,
+                                                 float lg_amin, float* ring, unsigned tail) {
+  constexpr int RW = PPT == 4 ? 16 : 8;  // region width
+  const int e = e0 + lane;
+  uint32_t m = 0;
+  float4 A, B, C;
+  if (e < cnt) {
+    B = sB[e];
+    C = sC[e];
+    const uint32_t cm = (__float_as_uint(B.w) >> rx0) & ((1u << RW) - 1u);
+    const uint32_t rm = (__float_as_uint(C.w) >> ry0) << 24;
+    if (cm != 0u && rm != 0u) {
+      A = sA[e];
+      const float X0 = ((float)RX + 0.5f) - A.x, Y0 = ((float)RY + 0.5f) - A.y;
+      if (box_reached(A.z, A.w, B.x, B.y, X0, X0 + (float)(RW - 1), Y0, Y0 + 7.0f, lg_amin))
+        m = (cm << 8) | rm;
+    }
   }
-  return (c0 & r0) | ((c0 & r1) << 1);
+  const unsigned hit = __ballot_sync(0xffffffffu, m != 0u);
+  if (m) {
+    const unsigned pos = (tail + __popc(hit & ((1u << lane) - 1u))) & (kRingItems - 1);
+    float* q = ring + (pos >> 1) * kPairWords;
+    const unsigned h = pos & 1u;
+    q[h] = A.x;
+    q[2 + h] = A.y;
+    q[4 + h] = A.z;
+    q[6 + h] = A.w;
+    q[8 + h] = B.x;
+    q[10 + h] = B.y;
+    reinterpret_cast<float4*>(q + 12)[h] = make_float4(C.x, C.y, C.z, B.z);
+    q[20 + h] = __uint_as_float(m);
+    q[22 + h] = __int_as_float(pos0 + e);
+  }
+  return tail + (unsigned)__popc(hit);
 }
 
 template <int PPT>
@@ -178,11 +208,12 @@ __device__ __forceinline__ TileInfo decode_tile(const BatchDev& b, int64_t id) {
   TileInfo ti;
   ti.v = view_of(b.tile_base, b.V, id);
   const ViewDev& cam = b.views[ti.v];
-  const int64_t nt = (int64_t)cam.tiles_x * cam.tiles_y;
-  const int64_t rem = id - b.tile_base[ti.v];
+  // (a launch has fewer than 2^31 items, so an item's place in its view fits 32 bits)
+  const uint32_t nt = (uint32_t)cam.tiles_x * (uint32_t)cam.tiles_y;
+  const uint32_t rem = (uint32_t)(id - b.tile_base[ti.v]);
   ti.k = (int)(rem / nt);
-  const int64_t t = rem - (int64_t)ti.k * nt;
-  const int tx = (int)(t % cam.tiles_x), ty = (int)(t / cam.tiles_x);
+  const uint32_t t = rem - (uint32_t)ti.k * nt;
+  const int ty = (int)(t / (uint32_t)cam.tiles_x), tx = (int)(t - (uint32_t)ty * cam.tiles_x);
   ti.tx = tx;
   ti.ty = ty;
   const int w = (int)(threadIdx.x >> 5), l = (int)(threadIdx.x & 31);
@@ -209,8 +240,11 @@ __device__ __forceinline__ TileInfo decode_tile(const BatchDev& b, int64_t id) {
 
 // kCount variants (eager runs only) also count the work for the roofline: thread-entries
 // examined, (pixel, entry) alpha evaluations and blends / contributions.
-constexpr int kNB = 256;  // list entries staged in shared memory per batch
-static_assert(kNB <= 256, "a compacted list item holds the entry in 8 bits");
+// List entries the forward stages in shared memory per batch: one per thread.
+template <int TS>
+constexpr int kNBFwd = TS == 8 ? 32 : 128;
+template <int TS, int PPT>
+constexpr int kRingWords = TS * TS / PPT / 32 * (kRingItems / 2) * kPairWords;  // all warps' rings
 // the backward stages fewer at a time where its threads allow (one entry per thread at
 // least); one-warp CTAs stage 64, which keeps their shared memory at 7.4 KB
 template <int TS, int PPT>
@@ -223,11 +257,24 @@ constexpr int kMinBlocksBwd = TS == 16 ? (PPT == 8 ? 28 : 16) : 1;
 // atomics); measured on the 10M step: 3 -> 18.58 ms, 12 -> 17.95, 20 -> 17.55, 32 -> 19.19
 constexpr int kDirectLanes = 20;
 
+// The forward of one work item.  It is bound by instruction issue (80 % of the issue slots,
+// 40 % of the FMA pipe, 3 % of HBM), so everything here is there to issue fewer: a warp sees
+// only the entries that can reach its region (box_reached leaves 27.7M of 36.7M
+// warp-entries of the 2M-Gaussian, 4-view step), and it takes them two at a time with the
+// exponents of both in packed FP32 instructions, without a branch per pixel.  Measured on
+// that step (8 subsets, no skipping, 16x16 tiles): 2.89 -> 2.12 ms, 3.07e9 -> 2.06e9 warp
+// instructions; 8x8 tiles 3.39 -> 1.96 ms, 32x32 4.14 -> 3.91 ms; the 10M step 58.4
+// -> 55.5 ms.  Packing the colours too (channel pairs, with w moved into both halves) took
+// 2.37 ms, a branch per stopping pair 2.46 ms, 10 CTAs per SM at 48 registers (spilling)
+// and 7 at 72 1-2 % more than 8 at 64.
 template <int TS, int PPT, bool kCount>
 __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, float4* sA,
-                                         float4* sB, float4* sC, uint32_t* sL) {
+                                         float4* sB, float4* sC, float* sR) {
   constexpr int NTH = TS * TS / PPT;
-  constexpr int NB = kNB;
+  constexpr int NB = kNBFwd<TS>;
+  constexpr int PER = NB > NTH ? NB / NTH : 1;  // staged entries per thread
+  constexpr int NC = kSlotCols<PPT>;
+  static_assert(kSlotRows<PPT> == 2, "a region is two 8 x 4 blocks high");
   const TileInfo ti = decode_tile<TS, PPT>(b, id);
   if (!in_omega(b, ti.v, ti.k, ti.tx, ti.ty)) {
     // outside the subset's visible region: no pairs; the composite never reads this tile.
@@ -243,9 +290,12 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
     return;
   }
   const uint2 rg = b.ranges[id];
-  const int64_t start = rg.x, end = rg.y > rg.x ? rg.y : rg.x;
-  const Rec* rec = b.rec + (int64_t)ti.v * b.N;
-  const float pcx0 = (float)ti.x + 0.5f, pcx1 = (float)(ti.x + 8) + 0.5f;
+  const uint32_t start = rg.x, len = rg.y > rg.x ? rg.y - rg.x : 0u;  // the item's list
+  // the lane's pixel columns and rows, twice each for the packed evaluation of two entries
+  const f32x2 pcx0 = pack2((float)ti.x + 0.5f, (float)ti.x + 0.5f),
+              pcx1 = pack2((float)(ti.x + 8) + 0.5f, (float)(ti.x + 8) + 0.5f),
+              pcy0 = pack2((float)ti.y + 0.5f, (float)ti.y + 0.5f),
+              pcy1 = pack2((float)(ti.y + 4) + 0.5f, (float)(ti.y + 4) + 0.5f);
   const float amin = b.alpha_min, amax = b.alpha_max, epsT = b.eps_T;
   float T[PPT], c0[PPT], c1[PPT], c2[PPT], D[PPT];
   int last[PPT];
@@ -255,8 +305,8 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
     T[i] = 1.0f; c0[i] = c1[i] = c2[i] = D[i] = 0.0f; last[i] = -1;
     if (ti.x + 8 * slot_col<PPT>(i) < ti.W && ti.y + 4 * slot_row<PPT>(i) < ti.H) live |= 1u << i;
   }
-  const ImgDev im = b.imgs[ti.v * b.K + ti.k];
-  const int64_t HW = (int64_t)ti.W * ti.H;
+  // (the planes' addresses are read again where they are used: nothing holds them in
+  // registers across the walk)
   if ((b.order && b.wave > 0) || b.sat) {
     const unsigned inb = live;  // slots inside the image
     // saturation skipping: a pixel where the subsets rendered before this one took the
@@ -284,6 +334,8 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
     }
     if (!__syncthreads_or(live != 0)) {
       if (kCount && threadIdx.x == 0 && b.counters) atomicAdd(b.counters + 6, 1ull);
+      const ImgDev im = b.imgs[ti.v * b.K + ti.k];
+      const int64_t HW = (int64_t)ti.W * ti.H;
 #pragma unroll
       for (int i = 0; i < PPT; ++i) {
         if (!((inb >> i) & 1u)) continue;
@@ -305,7 +357,7 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
   // takes the pixels' state from the planes the first one wrote and walks the whole
   // sorted list from the prefix's end: its first entries are the prefix's, in its order.
   __shared__ uint32_t s_prefix_item;
-  int64_t walk0 = start;
+  uint32_t walk0 = 0;  // list position where the walk begins
   if (b.sel) {
     const uint32_t sv = b.sel[id];
     if (sv == kSelNone) {
@@ -316,7 +368,9 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
       return;
     }
     if (sv & kSelResume) {
-      walk0 = start + (sv & ~kSelResume);
+      walk0 = sv & ~kSelResume;
+      const ImgDev im = b.imgs[ti.v * b.K + ti.k];
+      const int64_t HW = (int64_t)ti.W * ti.H;
 #pragma unroll
       for (int i = 0; i < PPT; ++i) {
         const int px = ti.x + 8 * slot_col<PPT>(i), py = ti.y + 4 * slot_row<PPT>(i);
@@ -335,77 +389,196 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
     if (threadIdx.x == 0) s_prefix_item = sv && !(sv & kSelResume) ? (uint32_t)id : kSelNone;
   }
   unsigned n_eval = 0, n_pix = 0, n_blend = 0;
-  for (int64_t base = walk0; base < end; base += NB) {
-    if (__syncthreads_count(live == 0) == NTH) break;
+  const int lane = (int)(threadIdx.x & 31);
+  const int RX = ti.x - (lane & 7), RY = ti.y - (lane >> 3);  // the warp's region
+  float* ring = sR + (threadIdx.x >> 5) * (kRingItems / 2 * kPairWords);
+  unsigned tail = 0, head = 0;  // ring positions: appended, processed
+  const float lg_amin = __log2f(amin);
+  // (alpha is compared before its clamp: with amin above amax nothing may pass)
+  const float amin_raw = amin <= amax ? amin : __int_as_float(0x7f800000);
+  // a pixel's bit pair in the items' masks; kDeadPixel (which no item has) once it is done
+  uint32_t pm[PPT];
 #pragma unroll
-    for (int r = 0; r < NB / NTH; ++r) {
-      const int slot = r * NTH + (int)threadIdx.x;
-      const int64_t j = base + slot;
-      if (j < end) {
-        uint32_t g = (uint32_t)b.keys[j];  // low half of the sorted key
-        if (g >= (uint32_t)b.N) { atomicOr(b.status, ST_BOUNDS); g = 0; }
-        const Rec* rp = rec + g;
-        sA[slot] = rp->a;
-        sB[slot] = rp->b;
-        sC[slot] = rp->c;
+  for (int i = 0; i < PPT; ++i)
+    pm[i] = (live >> i) & 1u ? (1u << (8 + (lane & 7) + 8 * slot_col<PPT>(i))) |
+                                   (1u << (24 + (lane >> 3) + 4 * slot_row<PPT>(i)))
+                             : kDeadPixel;
+  auto alive = [&]() {
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < PPT; ++i) any |= pm[i] != kDeadPixel;
+    return any;
+  };
+  // Blends ring entries head and head + 1.  Both entries' alphas are evaluated at every
+  // pixel of the lane (packed over the two entries) and are 0 where the pixel does not take
+  // the entry, which leaves T as it is bit for bit.
+  auto blend_pair = [&]() {
+    const float4* q = reinterpret_cast<const float4*>(ring + ((head & (kRingItems - 1)) >> 1) * kPairWords);
+    const float4 P0 = q[0], P1 = q[1], P2 = q[2], CA = q[3], CB = q[4], MJ = q[5];
+    const uint32_t m0 = __float_as_uint(MJ.x), m1 = __float_as_uint(MJ.y);
+    const int j0 = __float_as_int(MJ.z), j1 = __float_as_int(MJ.w);
+    const f32x2 u2 = pack2(P0.x, P0.y), v2 = pack2(P0.z, P0.w), qa2 = pack2(P1.x, P1.y),
+                qb2 = pack2(P1.z, P1.w), qc2 = pack2(P2.x, P2.y), o2 = pack2(P2.z, P2.w);
+    f32x2 hx2[NC], bx2[NC], dy2[2];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const f32x2 dx2 = sub2(c ? pcx1 : pcx0, u2);
+      hx2[c] = mul2(mul2(qa2, dx2), dx2);
+      bx2[c] = mul2(qb2, dx2);
+    }
+    dy2[0] = sub2(pcy0, v2);
+    dy2[1] = sub2(pcy1, v2);
+    float al0[PPT], al1[PPT], T0[PPT], T1[PPT];
+    bool ok0[PPT], ok1[PPT];
+    float tmin = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int i = 0; i < PPT; ++i) {
+      const f32x2 dy = dy2[slot_row<PPT>(i)];
+      const f32x2 p2 = fma2(fma2(qc2, dy, bx2[slot_col<PPT>(i)]), dy, hx2[slot_col<PPT>(i)]);
+      float p0, p1, r0, r1;
+      unpack2(p2, p0, p1);
+      unpack2(mul2(o2, pack2(ex2_approx(p0), ex2_approx(p1))), r0, r1);
+      const bool in0 = (~m0 & pm[i]) == 0u, in1 = (~m1 & pm[i]) == 0u;
+      ok0[i] = in0 && p0 <= 0.0f && r0 >= amin_raw;
+      ok1[i] = in1 && p1 <= 0.0f && r1 >= amin_raw;
+      if (kCount) n_pix += (unsigned)in0 + (unsigned)in1;
+      al0[i] = ok0[i] ? fminf(r0, amax) : 0.0f;
+      al1[i] = ok1[i] ? fminf(r1, amax) : 0.0f;
+      T0[i] = T[i] * (1.0f - al0[i]);
+      T1[i] = T0[i] * (1.0f - al1[i]);
+      tmin = fminf(tmin, T1[i]);
+    }
+    head += 2;
+    if (kCount && lane == 0) n_eval += 2u;
+    if (__any_sync(0xffffffffu, tmin < epsT)) {
+      // a pixel stops before the entry that would take it below eps_T: that entry and what
+      // follows leave it as it is
+#pragma unroll
+      for (int i = 0; i < PPT; ++i) {
+        const bool s0 = ok0[i] && T0[i] < epsT;
+        const bool s1 = s0 || (ok1[i] && T1[i] < epsT);
+        ok0[i] = ok0[i] && !s0;
+        ok1[i] = ok1[i] && !s1;
+        T0[i] = s0 ? T[i] : T0[i];
+        T1[i] = s1 ? T0[i] : T1[i];
+        al0[i] = s0 ? 0.0f : al0[i];
+        al1[i] = s1 ? 0.0f : al1[i];
+        pm[i] = s1 ? kDeadPixel : pm[i];
       }
     }
-    __syncthreads();
-    if (__any_sync(0xffffffffu, live != 0)) {
-      const int cnt = (int)((end - base) < NB ? (end - base) : NB);
-      const int lane = (int)(threadIdx.x & 31);
-      uint32_t* list = sL + (threadIdx.x >> 5) * NB;
-      const int nl = compact_entries<PPT>(sB, sC, cnt, ti.x - (lane & 7), ti.y - (lane >> 3),
-                                          lane, list);
-      auto entry = [&](const uint32_t item) {
-        const int jj = (int)(item & 0xFFu);
-        const float4 Bv = sB[jj];
-        const float4 Cv = sC[jj];
-        // slots to evaluate: in the rectangle, still blending
-        const unsigned todo = live & slot_mask<PPT>(item, lane & 7, lane >> 3);
-        const float4 Av = sA[jj];
-        const ColTerms ct0 = col_terms(Av, pcx0), ct1 = col_terms(Av, pcx1);
 #pragma unroll
-        for (int i = 0; i < PPT; ++i) {
-          if (!((todo >> i) & 1u)) continue;
-          const int ci = slot_col<PPT>(i), ri = slot_row<PPT>(i);
-          if (kCount) ++n_pix;
-          float alpha, ex, dy;
-          bool cl;
-          if (!pixel_alpha(ci ? ct1 : ct0, Av.y, Bv.x, Bv.y, (float)(ti.y + 4 * ri) + 0.5f, amin,
-                           amax, alpha, ex, dy, cl))
-            continue;
-          const float Tn = T[i] * (1.0f - alpha);
-          if (Tn < epsT) { live &= ~(1u << i); continue; }
-          const float w = alpha * T[i];
-          c0[i] = fmaf(Cv.x, w, c0[i]);
-          c1[i] = fmaf(Cv.y, w, c1[i]);
-          c2[i] = fmaf(Cv.z, w, c2[i]);
-          D[i] = fmaf(Bv.z, w, D[i]);
-          T[i] = Tn;
-          last[i] = (int)(base - start) + jj;
-          if (kCount) ++n_blend;
-        }
-      };
-      // four entries per warp-wide test of whether any pixel still blends (entries after
-      // the warp's last pixel has stopped find no slot to evaluate)
-      int q = 0;
-      for (; q < nl; q += 4) {
-        if (!__any_sync(0xffffffffu, live != 0)) break;
-        entry(list[q]);
-        if (q + 1 < nl) entry(list[q + 1]);
-        if (q + 2 < nl) entry(list[q + 2]);
-        if (q + 3 < nl) entry(list[q + 3]);
+    for (int i = 0; i < PPT; ++i) {
+      const float w0 = al0[i] * T[i], w1 = al1[i] * T0[i];
+      T[i] = T1[i];
+      if (ok0[i]) {
+        c0[i] = fmaf(CA.x, w0, c0[i]);
+        c1[i] = fmaf(CA.y, w0, c1[i]);
+        c2[i] = fmaf(CA.z, w0, c2[i]);
+        D[i] = fmaf(CA.w, w0, D[i]);
       }
-      q = q < nl ? q : nl;
-      if (kCount && lane == 0) n_eval += (unsigned)q;
+      if (ok1[i]) {
+        c0[i] = fmaf(CB.x, w1, c0[i]);
+        c1[i] = fmaf(CB.y, w1, c1[i]);
+        c2[i] = fmaf(CB.z, w1, c2[i]);
+        D[i] = fmaf(CB.w, w1, D[i]);
+      }
+      last[i] = ok0[i] ? j0 : last[i];
+      last[i] = ok1[i] ? j1 : last[i];
+      if (kCount) n_blend += (unsigned)ok0[i] + (unsigned)ok1[i];
+    }
+  };
+  bool open = alive();
+  // Batches of NB entries, double-buffered: while the warps blend one, the next one's
+  // records are copied behind it (cp.async; its keys were read one batch earlier still), so
+  // one barrier per batch both publishes the batch and frees the other buffer.
+  uint32_t nk[PER];
+  auto load_keys = [&](uint32_t base) {
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const uint32_t j = base + r * NTH + threadIdx.x;
+      nk[r] = j < len ? (uint32_t)b.keys[(uint64_t)start + j] : 0u;  // low half: the Gaussian
+    }
+  };
+  auto copy_records = [&](uint32_t base, int buf) {
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const uint32_t slot = r * NTH + threadIdx.x;
+      if (slot < NB && base + slot < len) {
+        uint32_t g = nk[r];
+        if (g >= (uint32_t)b.N) { atomicOr(b.status, ST_BOUNDS); g = 0; }
+        const Rec* rp = b.rec + ((int64_t)ti.v * b.N + g);
+        cp_async16(sA + buf * NB + slot, &rp->a);
+        cp_async16(sB + buf * NB + slot, &rp->b);
+        cp_async16(sC + buf * NB + slot, &rp->c);
+      }
+    }
+    cp_async_commit();
+  };
+  if (walk0 < len) {
+    load_keys(walk0);
+    copy_records(walk0, 0);
+    load_keys(walk0 + NB < len ? walk0 + NB : len);
+  }
+  int buf = 0;
+  for (uint32_t base = walk0; base < len; base += NB, buf ^= 1) {
+    // the thread's own records have landed: the rectangles become the tile's column and row
+    // masks
+    cp_async_wait<0>();
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const uint32_t slot = r * NTH + threadIdx.x;
+      if (slot < NB && base + slot < len) {
+        float* px = &sB[buf * NB + slot].w;
+        float* py = &sC[buf * NB + slot].w;
+        const uint32_t rx = __float_as_uint(*px), ry = __float_as_uint(*py);
+        const int x0 = max((int)(rx & 0xFFFFu) - ti.tx * TS, 0), x1 = min((int)(rx >> 16) - ti.tx * TS, TS - 1);
+        const int y0 = max((int)(ry & 0xFFFFu) - ti.ty * TS, 0), y1 = min((int)(ry >> 16) - ti.ty * TS, TS - 1);
+        *px = __uint_as_float(x0 <= x1 ? ((2u << (x1 - x0)) - 1u) << x0 : 0u);
+        *py = __uint_as_float(y0 <= y1 ? ((2u << (y1 - y0)) - 1u) << y0 : 0u);
+      }
+    }
+    if (__syncthreads_count(!open) == NTH) break;
+    const bool fin = len - base <= NB;
+    if (!fin) {
+      copy_records(base + NB, buf ^ 1);
+      load_keys(len - base > 2 * NB ? base + 2 * NB : len);
+    }
+    const int cnt = (int)(fin ? len - base : NB);
+    for (int e0 = 0; e0 < cnt; e0 += 32) {
+      if (!__any_sync(0xffffffffu, open)) break;
+      tail = append_group<PPT>(sA + buf * NB, sB + buf * NB, sC + buf * NB, e0, cnt, (int)base,
+                               RX, RY, RX - ti.tx * TS, RY - ti.ty * TS, lane, lg_amin, ring,
+                               tail);
+      const bool flush = fin && e0 + 32 >= cnt;
+      if (flush && ((tail - head) & 1u)) {
+        // an entry of zeros that no pixel takes beside the last one
+        float* q = ring + ((tail & (kRingItems - 1)) >> 1) * kPairWords;
+        if (lane < 12) q[lane >= 6 && lane < 10 ? 10 + lane : 2 * lane + 1] = 0.0f;
+        ++tail;
+      }
+      __syncwarp();
+      // (fewer than half a ring stay for the next group, which so always fits)
+      if (flush || tail - head >= kRingItems / 2) {
+        while (tail - head >= 2u) {
+          blend_pair();
+          if ((head & 7u) == 0u && !__any_sync(0xffffffffu, alive())) break;
+        }
+        __syncwarp();
+        open = alive();
+      }
     }
   }
+  cp_async_wait<0>();  // (a batch in flight when the walk ended early)
+  live = 0;
+#pragma unroll
+  for (int i = 0; i < PPT; ++i) live |= pm[i] != kDeadPixel ? 1u << i : 0u;
   if (kCount) {
     flush_counter(b.counters, 0, n_eval);
     flush_counter(b.counters, 1, n_pix);
     flush_counter(b.counters, 2, n_blend);
   }
+  const ImgDev im = b.imgs[ti.v * b.K + ti.k];
+  const int64_t HW = (int64_t)ti.W * ti.H;
 #pragma unroll
   for (int i = 0; i < PPT; ++i) {
     const int px = ti.x + 8 * slot_col<PPT>(i), py = ti.y + 4 * slot_row<PPT>(i);
@@ -638,17 +811,18 @@ __device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, fl
 
 // One CTA per work item, or (kPersist) a grid sized to the SMs whose CTAs take work items
 // in order from a device counter until none is left.
-// (16x16 tiles: 128 threads held to 48 registers, 10 resident CTAs per SM; 32x32 tiles:
-// 256 threads at 64 registers, 4 CTAs)
+// Resident forward CTAs its register limits are set for: at 16x16 tiles 8 CTAs of 128
+// threads (64 registers; the 26.6 KB of shared memory allow no more), at 32x32 3 of 256
+// (80), at 8x8 28 of one warp (72).
 template <int TS>
-constexpr int kMinBlocksFwd = TS == 16 ? 10 : (TS == 32 ? 4 : 1);
+constexpr int kMinBlocksFwd = TS == 16 ? 8 : (TS == 32 ? 3 : 28);
 
 template <int TS, int PPT, bool kCount, bool kPersist>
 __global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>) k_raster_fwd(const BatchDev b) {
-  __shared__ float4 sA[kNB], sB[kNB], sC[kNB];
-  __shared__ uint32_t sL[(TS * TS / PPT / 32) * kNB];  // per-warp compacted entry lists
+  __shared__ float4 sA[2 * kNBFwd<TS>], sB[2 * kNBFwd<TS>], sC[2 * kNBFwd<TS>];
+  __shared__ __align__(16) float sR[kRingWords<TS, PPT>];
   if constexpr (!kPersist) {
-    fwd_item<TS, PPT, kCount>(b, item_of(b, blockIdx.x), sA, sB, sC, sL);
+    fwd_item<TS, PPT, kCount>(b, item_of(b, blockIdx.x), sA, sB, sC, sR);
   } else {
     __shared__ long long s_id;
     for (;;) {
@@ -657,7 +831,7 @@ __global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>) k_raster_fwd
       __syncthreads();
       const int64_t id = s_id;
       if (id >= items_of_launch(b)) return;
-      fwd_item<TS, PPT, kCount>(b, item_of(b, id), sA, sB, sC, sL);
+      fwd_item<TS, PPT, kCount>(b, item_of(b, id), sA, sB, sC, sR);
     }
   }
 }
@@ -667,12 +841,12 @@ __global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>) k_raster_fwd
 // long walk: no register cap for occupancy).
 template <int TS, int PPT, bool kCount>
 __global__ void __launch_bounds__(TS * TS / PPT) k_raster_fwd_retry(const BatchDev b) {
-  __shared__ float4 sA[kNB], sB[kNB], sC[kNB];
-  __shared__ uint32_t sL[(TS * TS / PPT / 32) * kNB];
+  __shared__ float4 sA[2 * kNBFwd<TS>], sB[2 * kNBFwd<TS>], sC[2 * kNBFwd<TS>];
+  __shared__ __align__(16) float sR[kRingWords<TS, PPT>];
   const unsigned n = *b.retry_count;
   for (unsigned w = blockIdx.x; w < n; w += gridDim.x) {
     __syncthreads();  // the previous item is done with shared memory
-    fwd_item<TS, PPT, kCount>(b, (int64_t)b.retry[w], sA, sB, sC, sL);
+    fwd_item<TS, PPT, kCount>(b, (int64_t)b.retry[w], sA, sB, sC, sR);
   }
 }
 
@@ -699,9 +873,7 @@ __global__ void __launch_bounds__(TS * TS / PPT, (kMinBlocksBwd<TS, PPT>)) k_ras
 
 // Tile side -> pixels per thread.  Forward: 2 (8 x 8 regions per warp) for 8x8 and 16x16
 // tiles, 4 for 32x32; backward: 2 for 8x8, 8 (one warp per 16x16 tile) for 16x16, 4 (16 x 8
-// regions) for 32x32.  At 16x16 the forward's smaller per-thread state gives 40 resident
-// warps per SM instead of 30 and beats the 4-pixel mapping (15.8 vs 17.1 ms on the 10M
-// step); the backward's per-entry work (record loads, rectangle tests, the warp reduction
+// regions) for 32x32.  The backward's per-entry work (record loads, rectangle tests, the warp reduction
 // and its atomics) favours more pixels per lane: one warp per tile does it once per entry
 // instead of twice (21.0 ms at 8 pixels and 27 CTAs per SM, 22.0 at 4, 29.2 at 2).
 template <int TS>
