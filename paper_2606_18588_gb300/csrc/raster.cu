@@ -1,23 +1,20 @@
 // Local rendering of every (view, subset) tile: forward (Eq. 1-4) and backward.
 //
-// One CTA per image tile of TS x TS pixels; each thread owns PPT pixels, one in each of
-// PPT blocks of 8 x 4 pixels (TS x TS/PPT threads; layout below), so the shared-memory
-// loads, the rectangle test and the dx-dependent terms of an entry are shared by PPT
-// pixels, and in the backward the per-entry warp reduction and atomics are amortised over
-// PPT pixels.
-// The tile's sorted list is walked in batches of NB entries staged in shared memory.
+// A warp owns a region of 8 x 8 pixels (16 x 8 in the forward at 32x32 tiles), a lane two of
+// its pixels four rows apart (or four); a CTA holds the warps of one image tile.  Each warp
+// picks, from the tile's sorted list, the entries that can reach alpha_min in its region.
 // A pixel takes a Gaussian only inside its integer 3-sigma rectangle (so the result does
 // not depend on TS), with alpha = min(alpha_max, o 2^(p2)) >= alpha_min, and stops before
-// the Gaussian that would take its transmittance below eps_T.  The CTA leaves the list
-// once every pixel has stopped (__syncthreads_count).
+// the Gaussian that would take its transmittance below eps_T.  The forward's CTA leaves the
+// list once every pixel has stopped (__syncthreads_count).
 //
 // The backward walks the same list back to front from each pixel's last blended entry,
 // recovering T_i = T_{i+1} / (1 - alpha_i) from the stored final T^m, and applies the
 // adjoint of Eq. 3-4 with the composite adjoint (dL/dC^m, dL/dT^m of Eq. 6-7) as input:
 //   dC^m/dc_i = alpha_i T_i,  dC^m/dalpha_i = c_i T_i - B_i / (1 - alpha_i),
 //   dT^m/dalpha_i = -T^m / (1 - alpha_i),  B_i = sum_{j>i} c_j alpha_j T_j.
-// Per-Gaussian sums over the tile's pixels are reduced with warp shuffles and added to
-// the per-(view, Gaussian) 2-D gradient with float4 atomics.  With gp = dL/dpower at a
+// Per-Gaussian sums over a warp's pixels are formed in shared memory and added to the
+// per-(view, Gaussian) 2-D gradient with float4 atomics.  With gp = dL/dpower at a
 // pixel, power = -(A dx^2 + 2 B dx dy + C dy^2) / 2 and (dx, dy) = pixel centre - (u, v),
 // the record holds the conic-free moments of ge = gp / o = dL/dalpha e^power (0 where
 // alpha is clamped), sum ge dx, ge dy, ge dx^2, ge dx dy, ge dy^2, and dL/do = sum ge;
@@ -28,19 +25,6 @@
 namespace splx {
 
 namespace {
-
-// Per-entry terms shared by the pixels of one column: dx, qa dx^2 and qb dx.
-struct ColTerms {
-  float dx, hx, bx;
-};
-
-__device__ __forceinline__ ColTerms col_terms(const float4 a, float pcx) {
-  ColTerms c;
-  c.dx = __fsub_rn(pcx, a.x);
-  c.hx = __fmul_rn(__fmul_rn(a.z, c.dx), c.dx);
-  c.bx = __fmul_rn(a.w, c.dx);
-  return c;
-}
 
 // 2^x and 1/x as single special-function-unit instructions (relative error about 2^-22;
 // subnormal results flush to zero, which the alpha threshold rejects anyway).
@@ -55,20 +39,6 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
-// alpha of an entry at one pixel of the column; the same code runs in the forward and
-// the backward so both take bit-identical decisions.  Returns false if skipped.
-__device__ __forceinline__ bool pixel_alpha(const ColTerms& c, float ay, float qc, float o,
-                                            float pcy, float amin, float amax, float& alpha,
-                                            float& ex, float& dy, bool& clamped) {
-  dy = __fsub_rn(pcy, ay);
-  const float p2 = __fmaf_rn(__fmaf_rn(qc, dy, c.bx), dy, c.hx);
-  ex = ex2_approx(p2);  // finite for the rounding-sized p2 > 0 that the test below rejects
-  const float raw = __fmul_rn(o, ex);
-  clamped = raw > amax;
-  alpha = clamped ? amax : raw;
-  return p2 <= 0.0f && alpha >= amin;
-}
-
 // Adds per-thread counts into counters[slot] with one atomic per warp.
 __device__ __forceinline__ void flush_counter(unsigned long long* counters, int slot, unsigned v) {
   if (!counters) return;
@@ -77,42 +47,10 @@ __device__ __forceinline__ void flush_counter(unsigned long long* counters, int 
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(counters + slot, (unsigned long long)v);
 }
 
-// Sum of v[0..8] over the warp by reduce-scatter: each exchange sends half of the
-// values a lane still holds, so 8 values take 4 + 2 + 1 + 1 + 1 shuffles instead of
-// 8 x 5.  Afterwards lane l holds the full sum of value (l >> 2) & 7 in `mine`, and
-// every lane holds the sum of value 8 in `v8`.
-__device__ __forceinline__ void warp_reduce9(const float (&v)[9], int lane, float& mine,
-                                             float& v8) {
-  const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0, h2 = (lane & 4) != 0;
-  float a[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float send = h4 ? v[k] : v[k + 4];
-    const float keep = h4 ? v[k + 4] : v[k];
-    a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-  float c[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const float send = h3 ? a[k] : a[k + 2];
-    const float keep = h3 ? a[k + 2] : a[k];
-    c[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-  float d = (h2 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h2 ? c[0] : c[1], 4);
-  d += __shfl_xor_sync(0xffffffffu, d, 2);
-  d += __shfl_xor_sync(0xffffffffu, d, 1);
-  mine = d;
-  float e = v[8];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-  v8 = e;
-}
-
-// Pixels of a thread: slot i of PPT is an 8 x 4 block of the tile, lanes laid out as
-// 8 columns x 4 rows inside it; a warp's PPT blocks tile a 16 x 16 region (PPT = 8), a
-// 16 x 8 region (PPT = 4) or an 8 x 8 region (PPT = 2).  A Gaussian's footprint then meets
-// few blocks, and a block it meets keeps many lanes busy.  (x, y) is the thread's pixel in
-// slot 0; slot i adds (8 (i & 1), 4 (i >> 1)) for PPT = 4 and 8, and (0, 4 i) for PPT = 2.
+// Pixels of a forward thread: slot i of PPT is an 8 x 4 block of the tile, lanes laid out as
+// 8 columns x 4 rows inside it; a warp's PPT blocks tile a 16 x 8 region (PPT = 4) or an
+// 8 x 8 region (PPT = 2).  (x, y) is the thread's pixel in slot 0; slot i adds (8 (i & 1),
+// 4 (i >> 1)) for PPT = 4 and (0, 4 i) for PPT = 2.
 struct TileInfo {
   int v, k, x, y, W, H, tx, ty;
 };
@@ -218,10 +156,7 @@ __device__ __forceinline__ TileInfo decode_tile(const BatchDev& b, int64_t id) {
   ti.ty = ty;
   const int w = (int)(threadIdx.x >> 5), l = (int)(threadIdx.x & 31);
   int rx0 = 0, ry0 = 0;
-  if (PPT == 8) {  // 16 x 16 regions
-    rx0 = 16 * (w % (TS / 16));
-    ry0 = 16 * (w / (TS / 16));
-  } else if (PPT == 4) {  // 16 x 8 regions
+  if (PPT == 4) {  // 16 x 8 regions
     constexpr int kRegionsPerRow = TS >= 16 ? TS / 16 : 1;
     rx0 = 16 * (w % kRegionsPerRow);
     ry0 = 8 * (w / kRegionsPerRow);
@@ -245,18 +180,12 @@ template <int TS>
 constexpr int kNBFwd = TS == 8 ? 32 : 128;
 template <int TS, int PPT>
 constexpr int kRingWords = TS * TS / PPT / 32 * (kRingItems / 2) * kPairWords;  // all warps' rings
-// the backward stages fewer at a time where its threads allow (one entry per thread at
-// least); one-warp CTAs stage 64, which keeps their shared memory at 7.4 KB
-template <int TS, int PPT>
-constexpr int kNBBwd = TS * TS / PPT > 128 ? TS * TS / PPT : (TS * TS / PPT == 32 ? 64 : 128);
-// resident CTAs the backward's register limit is set for
-template <int TS, int PPT>
-constexpr int kMinBlocksBwd = TS == 16 ? (PPT == 8 ? 28 : 16) : 1;
-// backward: up to this many lanes with a contribution add their gradients with their own
-// atomics (three per lane) instead of the warp reduction (about 45 instructions and nine
-// atomics); measured on the 10M step: 3 -> 18.58 ms, 12 -> 17.95, 20 -> 17.55, 32 -> 19.19
-constexpr int kDirectLanes = 20;
-
+// resident CTAs the backward's register limit is set for: 24 warps of 80 registers, as many
+// as its 9.3 KB of shared memory per warp leave room for
+template <int TS>
+constexpr int kMinBlocksBwd = TS == 8 ? 24 : 6;
+// above this an adjoint or a colour takes the backward's careful path
+constexpr float kWild = 1e18f;
 // The forward of one work item.  It is bound by instruction issue (80 % of the issue slots,
 // 40 % of the FMA pipe, 3 % of HBM), so everything here is there to issue fewer: a warp sees
 // only the entries that can reach its region (box_reached leaves 27.7M of 36.7M
@@ -627,181 +556,354 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
   }
 }
 
-template <int TS, int PPT, bool kCount>
-__device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, float4* sA,
-                                         float4* sB, float4* sC, uint32_t* sG, int& s_maxlast,
-                                         float4* sQ) {
-  constexpr int NTH = TS * TS / PPT;
-  constexpr int NB = kNBBwd<TS, PPT>;
-  const TileInfo ti = decode_tile<TS, PPT>(b, id);
+// The backward's shared memory of one warp (an 8 x 8 block of pixels).
+//   ring  items that can reach the block, two side by side (kBwdPair words per pair):
+//         [u0 u1 v0 v1] [qa0 qa1 qb0 qb1] [qc0 qc1 o0 o1] [r0 r0 g0 g0] [b0 b0 m0 j0]
+//         [r1 r1 g1 g1] [b1 b1 m1 j1]   (m: columns in bits 0-7, rows in bits 8-15 of the
+//         block that the rectangle spans; j: position in the tile's list)
+//   part  per item of a group of eight and lane: (ge, ge', aT, aT') of the lane's two pixels
+//   qxy, qz  the composite adjoint of the block's pixels: (x, x', y, y'), (z, z') per lane
+constexpr int kBwdRing = 40, kBwdPair = 28, kBwdGroup = 8, kPartStride = 36;
+struct BwdShared {
+  float ring[kBwdRing / 2 * kBwdPair];
+  float4 raw[3][32];
+  float4 part[kBwdGroup * kPartStride];
+  float4 qxy[32];
+  float2 qz[32];
+  uint32_t gid[kBwdRing];
+};
+
+// The backward of one 8 x 8 block of a work item, one warp.  It is bound by instruction issue
+// and by shared memory (69 % of the issue slots, 76 % of the shared-memory pipe, DRAM idle).
+// The list's entries that can reach the block are taken back to front in groups of eight, in
+// two halves: first each lane runs the recurrences of its two pixels over the eight items
+// and leaves (dL/dpower / o, alpha T) per item and pixel in shared memory; then four lanes per
+// item sum the item's parts over the pixels, so the nine sums take two shuffles each for
+// eight items at once (18 for a group) and no atomics but three per item and block.  Before,
+// one warp held a whole 16x16 tile, 8 pixels a lane, branched per 8 x 4 block and reduced
+// nine sums over its 32 lanes for every entry (some 50 instructions) or let up to 20 lanes
+// add their own.  2M Gaussians, 4 views, 8 subsets: 2.75 -> 2.15 ms at 16x16 tiles, 2.90 ->
+// 2.13 at 8x8, 4.55 -> 2.45 at 32x32; the 10M step's 17.5 -> 13.45 ms, the city's 3.6 ->
+// 2.42 ms.  Measured beside it: the one-warp tile with the packed arithmetic and box tests
+// alone 2.51 ms; one-warp CTAs 2.21 ms (the city 3.66: siblings share records in L1); the
+// group's four pairs not unrolled 2.22 ms; one warp taking a tile's four blocks in turn,
+// batch by batch, 2.41 ms (0.211 ms on 560 tiles).
+// kSync: the tile's warps take the batches of 32 entries together and leave their sums per
+// batch slot here; the CTA then adds them in the order of the warps, one add per tile.
+struct BwdSums {
+  float acc[2][4][32][9];  // two batches alternate, so that one barrier per batch is enough
+  unsigned have[2][4];      // per warp, the slots it has sums for
+  int maxlast;
+};
+
+template <int TS, bool kSync, bool kCount>
+__device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, const int blk,
+                                         BwdShared& sh, BwdSums* cta) {
+  const TileInfo ti = decode_tile<TS, 2>(b, id);
   if (!in_omega(b, ti.v, ti.k, ti.tx, ti.ty)) return;  // nothing written there, nothing to do
-  const uint2 rg = b.ranges[id];
-  const int64_t start = rg.x;  // (a selected prefix's range points into keys_alt)
-  const ImgDev im = b.imgs[ti.v * b.K + ti.k];
-  // composite adjoint of the thread's pixels: (dL/dC^m rgb, -T^m dL/dT^m) per slot, in
-  // shared memory (read only where a pixel takes an entry), which keeps registers down
-  float4* gq = sQ + threadIdx.x;  // slot i at gq[i * NTH]
+  const int lane = (int)(threadIdx.x & 31);
+  // the warp's block: RX, RY its origin on the image
+  const int RX = ti.tx * TS + 8 * (blk % (TS / 8)), RY = ti.ty * TS + 8 * (blk / (TS / 8));
+  const int x = RX + (lane & 7), y = RY + (lane >> 3);  // the lane's pixels: (x, y), (x, y + 4)
+  const float amax = b.alpha_max;
+  const float amin_raw = b.alpha_min <= amax ? b.alpha_min : __int_as_float(0x7f800000);
+  const float lg_amin = __log2f(b.alpha_min);
   // W = -T^m dL/dT^m - sum_ch dL/dC^m_ch B_ch: the colour suffix sums B enter the alpha
   // adjoint only through this dot product, so one scalar per pixel carries them
-  float T[PPT], W[PPT];
-  int mylast[PPT];
-  int tlast = -1;  // largest last over this thread's pixels
+  f32x2 T2, W2, qx, qy, qz;
+  int last0, last1;
+  bool wild;  // an adjoint so large that 0 x (its products) might not be 0
+  {
+    const ImgDev im = b.imgs[ti.v * b.K + ti.k];
+    float Tm[2], Wm[2];
+    float4 g[2];
+    int last[2];
+    wild = false;
 #pragma unroll
-  for (int i = 0; i < PPT; ++i) {
-    float4 gct = make_float4(0.f, 0.f, 0.f, 0.f);
-    T[i] = 1.0f;
-    mylast[i] = -1;
-    const int px = ti.x + 8 * slot_col<PPT>(i), py = ti.y + 4 * slot_row<PPT>(i);
-    if (px < ti.W && py < ti.H) {
-      const int64_t p = (int64_t)py * ti.W + px;
-      gct = im.gCT[p];
-      T[i] = im.T[p];
-      mylast[i] = im.last[p];
-      if (gct.x == 0.0f && gct.y == 0.0f && gct.z == 0.0f && gct.w == 0.0f)
-        mylast[i] = -1;
+    for (int h = 0; h < 2; ++h) {
+      g[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+      Tm[h] = 1.0f;
+      last[h] = -1;
+      if (x < ti.W && y + 4 * h < ti.H) {
+        const int64_t p = (int64_t)(y + 4 * h) * ti.W + x;
+        g[h] = im.gCT[p];
+        Tm[h] = im.T[p];
+        if (g[h].x != 0.0f || g[h].y != 0.0f || g[h].z != 0.0f || g[h].w != 0.0f)
+          last[h] = im.last[p];
+      }
+      Wm[h] = -Tm[h] * g[h].w;
+      wild |= !(fabsf(g[h].x) <= kWild) || !(fabsf(g[h].y) <= kWild) ||
+              !(fabsf(g[h].z) <= kWild) || !(fabsf(g[h].w) <= kWild);
     }
-    W[i] = -T[i] * gct.w;
-    gq[i * NTH] = make_float4(gct.x, gct.y, gct.z, 0.0f);
-    tlast = mylast[i] > tlast ? mylast[i] : tlast;
+    last0 = last[0];
+    last1 = last[1];
+    T2 = pack2(Tm[0], Tm[1]);
+    W2 = pack2(Wm[0], Wm[1]);
+    qx = pack2(g[0].x, g[1].x);
+    qy = pack2(g[0].y, g[1].y);
+    qz = pack2(g[0].z, g[1].z);
+    sh.qxy[lane] = make_float4(g[0].x, g[1].x, g[0].y, g[1].y);
+    sh.qz[lane] = make_float2(g[0].z, g[1].z);
   }
-  if (threadIdx.x == 0) s_maxlast = -1;
-  __syncthreads();
-  if (tlast >= 0) atomicMax(&s_maxlast, tlast);
-  __syncthreads();
-  const int maxlast = s_maxlast;
+  const int mylast = __reduce_max_sync(0xffffffffu, max(last0, last1));
+  int maxlast = mylast;
+  if (kSync) {
+    if (threadIdx.x == 0) cta->maxlast = -1;
+    __syncthreads();
+    if (lane == 0 && mylast >= 0) atomicMax(&cta->maxlast, mylast);
+    __syncthreads();
+    maxlast = cta->maxlast;
+  }
   if (maxlast < 0) return;
-
-  const Rec* rec = b.rec + (int64_t)ti.v * b.N;
-  float4* g2 = b.grad2d + (int64_t)ti.v * b.N * 3;
-  const float pcx0 = (float)ti.x + 0.5f, pcx1 = (float)(ti.x + 8) + 0.5f;
-  const float amin = b.alpha_min, amax = b.alpha_max;
-  const int lane = threadIdx.x & 31;
+  bool careful = __any_sync(0xffffffffu, wild);
+  const uint64_t start = b.ranges[id].x;  // (a selected prefix's range points into keys_alt)
+  const uint32_t pm0 = (1u << (lane & 7)) | (1u << (8 + (lane >> 3))),
+                 pm1 = (1u << (lane & 7)) | (1u << (12 + (lane >> 3)));
+  const f32x2 pcx2 = pack2((float)x + 0.5f, (float)x + 0.5f),
+              pcya = pack2((float)y + 0.5f, (float)y + 0.5f),
+              pcyb = pack2((float)(y + 4) + 0.5f, (float)(y + 4) + 0.5f);
+  const f32x2 one2 = pack2(1.0f, 1.0f), neg2 = pack2(-1.0f, -1.0f);
   unsigned n_evalb = 0, n_pixb = 0, n_actb = 0;
 
-  // the thread's keys of the next batch (low halves: the Gaussian indices), loaded one
-  // batch ahead so that staging waits for the records only
-  uint32_t nk[NB / NTH];
-  auto load_keys = [&](int top) {
+  // First half of a group: the pair of ring items at index ri, as items e and e + 1 of the
+  // group, against the lane's two pixels.  The exponents are packed over the two items, the
+  // recurrences of T and W over the two pixels; a pixel that does not take an item has alpha
+  // 0, which leaves T and W as they are (1/1 is exact), and e^power 0.
+  auto take_pair = [&](int ri, int e) {
+    const float4* q = reinterpret_cast<const float4*>(sh.ring + (ri >> 1) * kBwdPair);
+    const float4 P0 = q[0], P1 = q[1], P2 = q[2];
+    const f32x2 dx = sub2(pcx2, pack2(P0.x, P0.y));
+    const f32x2 hx = mul2(mul2(pack2(P1.x, P1.y), dx), dx), bx = mul2(pack2(P1.z, P1.w), dx);
+    const f32x2 dya = sub2(pcya, pack2(P0.z, P0.w)), dyb = sub2(pcyb, pack2(P0.z, P0.w));
+    const f32x2 qc2 = pack2(P2.x, P2.y), o2 = pack2(P2.z, P2.w);
+    float pa[2], pb[2], ra[2], rb[2], ea[2], eb[2];  // per item: pixel a, pixel b
+    unpack2(fma2(fma2(qc2, dya, bx), dya, hx), pa[0], pa[1]);
+    unpack2(fma2(fma2(qc2, dyb, bx), dyb, hx), pb[0], pb[1]);
 #pragma unroll
-    for (int r = 0; r < NB / NTH; ++r) {
-      const int j = top - (r * NTH + (int)threadIdx.x);
-      nk[r] = j >= 0 ? (uint32_t)b.keys[start + j] : 0u;
+    for (int h = 0; h < 2; ++h) { ea[h] = ex2_approx(pa[h]); eb[h] = ex2_approx(pb[h]); }
+    unpack2(mul2(o2, pack2(ea[0], ea[1])), ra[0], ra[1]);
+    unpack2(mul2(o2, pack2(eb[0], eb[1])), rb[0], rb[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float4 K0 = q[3 + 2 * h], K1 = q[4 + 2 * h];
+      const uint32_t nm = ~__float_as_uint(K1.z);
+      const int j = __float_as_int(K1.w);
+      const bool ina = (nm & pm0) == 0u && j <= last0, inb = (nm & pm1) == 0u && j <= last1;
+      const bool oka = ina && pa[h] <= 0.0f && ra[h] >= amin_raw;
+      const bool okb = inb && pb[h] <= 0.0f && rb[h] >= amin_raw;
+      if (kCount) {
+        n_pixb += (unsigned)ina + (unsigned)inb;
+        n_actb += (unsigned)oka + (unsigned)okb;
+      }
+      const f32x2 al = pack2(oka ? fminf(ra[h], amax) : 0.0f, okb ? fminf(rb[h], amax) : 0.0f);
+      // (dL/dpower is 0 where alpha is clamped)
+      const f32x2 em = pack2(oka && ra[h] <= amax ? ea[h] : 0.0f, okb && rb[h] <= amax ? eb[h] : 0.0f);
+      float oa, ob;
+      unpack2(sub2(one2, al), oa, ob);
+      const f32x2 rinv = pack2(rcp_approx(oa), rcp_approx(ob));
+      const f32x2 Ti = mul2(T2, rinv);
+      const f32x2 aT = mul2(al, Ti);
+      f32x2 qc = fma2(qz, pack2(K1.x, K1.y),
+                      fma2(qy, pack2(K0.z, K0.w), mul2(qx, pack2(K0.x, K0.y))));  // dL/dC^m . c_i
+      f32x2 ga = fma2(Ti, qc, mul2(W2, rinv));                                    // dL/dalpha_i
+      if (careful) {
+        // products that may overflow: nothing of a pixel that does not take the item, no
+        // dL/dpower where alpha is clamped
+        float u, w;
+        unpack2(qc, u, w);
+        qc = pack2(oka ? u : 0.0f, okb ? w : 0.0f);
+        unpack2(ga, u, w);
+        ga = pack2(oka && ra[h] <= amax ? u : 0.0f, okb && rb[h] <= amax ? w : 0.0f);
+      }
+      W2 = fma2(mul2(qc, neg2), aT, W2);
+      T2 = Ti;
+      float g0, g1, t0, t1;
+      unpack2(mul2(ga, em), g0, g1);
+      unpack2(aT, t0, t1);
+      sh.part[(e + h) * kPartStride + lane] = make_float4(g0, g1, t0, t1);
     }
   };
-  load_keys(maxlast);
-  for (int top = maxlast; top >= 0; top -= NB) {
-    const int lo = top - NB + 1 > 0 ? top - NB + 1 : 0;
-    __syncthreads();
+
+  // Second half: four lanes per item sum its parts over the block's pixels (16 each, two
+  // columns) and add them to its 2-D gradient: the moments sum ge, ge dx, ge dy, ge dx^2,
+  // ge dx dy, ge dy^2 (ge = dL/dpower / o = dL/do e^power) and dL/dcolour; the projection
+  // adjoint applies the conic and the opacity.
+  int top = maxlast;  // list position of the batch's first entry
+  auto sum_group = [&](int ri, int cnt) {
+    const int e = lane >> 2, qd = lane & 3;
+    const float* r = sh.ring + ((ri + e) >> 1) * kBwdPair + ((ri + e) & 1);
+    const float u = r[0], v = r[2];
+    const float dxa = ((float)(RX + qd) + 0.5f) - u, dxb = ((float)(RX + qd + 4) + 0.5f) - u;
+    const float4* part = sh.part + e * kPartStride + qd;
+    f32x2 a0 = 0, a1 = 0, a2 = 0, b0 = 0, b1 = 0, b2 = 0, gr = 0, gg = 0, gb = 0;
 #pragma unroll
-    for (int r = 0; r < NB / NTH; ++r) {
-      const int slot = r * NTH + (int)threadIdx.x;  // slot s holds entry top - s
-      const int j = top - slot;
-      if (j >= lo) {
-        uint32_t g = nk[r];
-        if (g >= (uint32_t)b.N) { atomicOr(b.status, ST_BOUNDS); g = 0; }
-        const Rec* rp = rec + g;
-        sA[slot] = rp->a;
-        sB[slot] = rp->b;
-        sC[slot] = rp->c;
-        sG[slot] = g;
+    for (int i = 0; i < 4; ++i) {
+      const f32x2 dy = sub2(pack2((float)(RY + i) + 0.5f, (float)(RY + i + 4) + 0.5f), pack2(v, v));
+      const f32x2 dyy = mul2(dy, dy);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const float4 s = part[8 * i + 4 * c], q4 = sh.qxy[8 * i + 4 * c + qd];
+        const float2 q2 = sh.qz[8 * i + 4 * c + qd];
+        const f32x2 ge = pack2(s.x, s.y), aT = pack2(s.z, s.w);
+        if (c == 0) {
+          a0 = add2(a0, ge);
+          a1 = fma2(ge, dy, a1);
+          a2 = fma2(ge, dyy, a2);
+        } else {
+          b0 = add2(b0, ge);
+          b1 = fma2(ge, dy, b1);
+          b2 = fma2(ge, dyy, b2);
+        }
+        f32x2 x2 = pack2(q4.x, q4.y), y2 = pack2(q4.z, q4.w), z2 = pack2(q2.x, q2.y);
+        if (careful) {
+          const bool k0 = s.z != 0.0f, k1 = s.w != 0.0f;
+          x2 = pack2(k0 ? q4.x : 0.0f, k1 ? q4.y : 0.0f);
+          y2 = pack2(k0 ? q4.z : 0.0f, k1 ? q4.w : 0.0f);
+          z2 = pack2(k0 ? q2.x : 0.0f, k1 ? q2.y : 0.0f);
+        }
+        gr = fma2(x2, aT, gr);
+        gg = fma2(y2, aT, gg);
+        gb = fma2(z2, aT, gb);
       }
     }
-    load_keys(top - NB);
-    __syncthreads();
-    const int cnt = top - lo + 1;
-    if (kCount && tlast >= lo) n_evalb += (unsigned)((tlast < top ? tlast : top) - lo + 1);
-    for (int jj = 0; jj < cnt; ++jj) {
-      const int j = top - jj;
-      // the entry's sums over the warp's pixels: ge dx, ge dy, ge dx^2, ge dx dy, ge dy^2
-      // (ge = dL/dpower / o), dL/do and dL/dcolour; the projection adjoint applies the conic
-      // and the opacity
-      float sx = 0.f, sy = 0.f, sxx = 0.f, sxy = 0.f, syy = 0.f, go = 0.f, gr = 0.f, gg = 0.f,
-            gb = 0.f;
-      bool act = false;
-      if (j <= tlast) {
-        const float4 Bv = sB[jj];
-        const float4 Cv = sC[jj];
-        const uint32_t rx = __float_as_uint(Bv.w), ry = __float_as_uint(Cv.w);
-        const int x0 = (int)(rx & 0xFFFFu), x1 = (int)(rx >> 16);
-        const int y0 = (int)(ry & 0xFFFFu), y1 = (int)(ry >> 16);
-        // inside [x0, x1] as one unsigned compare (a pixel left of x0 wraps to a large value)
-        const unsigned rw = (unsigned)(x1 - x0), rh = (unsigned)(y1 - y0);
-        bool cin[kSlotCols<PPT>], rin[kSlotRows<PPT>], anyc = false, anyr = false;
+    auto both = [](f32x2 w) {
+      float lo, hi;
+      unpack2(w, lo, hi);
+      return lo + hi;
+    };
+    const float A0 = both(a0), A1 = both(a1), B0 = both(b0), B1 = both(b1);
+    float w[9] = {dxa * A0 + dxb * B0, A1 + B1, dxa * dxa * A0 + dxb * dxb * B0,
+                  dxa * A1 + dxb * B1, both(a2) + both(b2), A0 + B0, both(gr), both(gg), both(gb)};
+    uint32_t any = 0;
 #pragma unroll
-        for (int c = 0; c < kSlotCols<PPT>; ++c) {
-          cin[c] = (unsigned)(ti.x + 8 * c - x0) <= rw;
-          anyc |= cin[c];
-        }
+    for (int i = 0; i < 9; ++i) {
+      w[i] += __shfl_xor_sync(0xffffffffu, w[i], 1);
+      w[i] += __shfl_xor_sync(0xffffffffu, w[i], 2);
+      any |= __float_as_uint(w[i]);
+    }
+    if (kSync) {
+      if (qd == 0 && e < cnt) {
+        const float* c = sh.ring + ((ri + e) >> 1) * kBwdPair + 12 + 8 * ((ri + e) & 1);
+        float* dst = cta->acc[(top >> 5) & 1][threadIdx.x >> 5][top - __float_as_int(c[7])];
 #pragma unroll
-        for (int r = 0; r < kSlotRows<PPT>; ++r) {
-          rin[r] = (unsigned)(ti.y + 4 * r - y0) <= rh;
-          anyr |= rin[r];
-        }
-        if (anyc && anyr) {
-          const float4 Av = sA[jj];
-          const ColTerms ct0 = col_terms(Av, pcx0), ct1 = col_terms(Av, pcx1);
-#pragma unroll
-          for (int i = 0; i < PPT; ++i) {
-            const int ci = slot_col<PPT>(i), ri = slot_row<PPT>(i);
-            if (j > mylast[i] || !cin[ci] || !rin[ri]) continue;
-            if (kCount) ++n_pixb;
-            const ColTerms& ct = ci ? ct1 : ct0;
-            float alpha, ex, dy;
-            bool cl;
-            if (!pixel_alpha(ct, Av.y, Bv.x, Bv.y, (float)(ti.y + 4 * ri) + 0.5f, amin, amax, alpha,
-                             ex, dy, cl))
-              continue;
-            if (kCount) ++n_actb;
-            act = true;
-            const float rinv = rcp_approx(1.0f - alpha);
-            const float Ti = T[i] * rinv;
-            const float aT = alpha * Ti;
-            const float4 q = gq[i * NTH];
-            gr = fmaf(q.x, aT, gr);
-            gg = fmaf(q.y, aT, gg);
-            gb = fmaf(q.z, aT, gb);
-            const float qc = fmaf(q.z, Cv.z, fmaf(q.y, Cv.y, q.x * Cv.x));  // dL/dC^m . c_i
-            const float ga = fmaf(Ti, qc, W[i] * rinv);                      // dL/dalpha_i
-            // dL/do = ga e^power and dL/dpower = o ga e^power where alpha is not clamped,
-            // 0 where it is; the moments are of ga e^power (the projection adjoint applies o)
-            const float ge = cl ? 0.0f : ga * ex;
-            go += ge;
-            const float px = ge * ct.dx, py = ge * dy;
-            sx += px;
-            sy += py;
-            sxx = fmaf(px, ct.dx, sxx);
-            sxy = fmaf(px, dy, sxy);
-            syy = fmaf(py, dy, syy);
-            W[i] = fmaf(-qc, aT, W[i]);
-            T[i] = Ti;
-          }
-        }
+        for (int i = 0; i < 9; ++i) dst[i] = w[i];
       }
-      const unsigned am = __ballot_sync(0xffffffffu, act);
-      if (am) {
-        if (__popc(am) <= kDirectLanes) {
-          // up to kDirectLanes lanes hold the warp's contribution: their own atomics cost
-          // the L2 more operations than the reduction's nine but skip its shuffles, and
-          // the kernel is bound by instruction issue, not by the L2
-          if (act) {
-            float4* dst = g2 + (int64_t)sG[jj] * 3;
-            atomicAdd(dst, make_float4(sx, sy, sxx, sxy));
-            atomicAdd(dst + 1, make_float4(syy, go, gr, gg));
-            atomicAdd(&dst[2].x, gb);
+    } else if (qd == 0 && e < cnt && (any << 1) != 0u) {  // (nothing to add where no pixel took it)
+      float4* dst = b.grad2d + ((int64_t)ti.v * b.N + sh.gid[ri + e]) * 3;
+      atomicAdd(dst, make_float4(w[0], w[1], w[2], w[3]));
+      atomicAdd(dst + 1, make_float4(w[4], w[5], w[6], w[7]));
+      atomicAdd(&dst[2].x, w[8]);
+    }
+  };
+
+  // Lane l holds entry top - l of each batch of 32: its record is copied behind the batch
+  // before (cp.async), its key (low half: the Gaussian) read one batch earlier still.
+  uint32_t nk = 0;
+  auto load_key = [&](int j) { nk = j >= 0 ? (uint32_t)b.keys[start + j] : 0u; };
+  auto copy_record = [&](int j) {
+    if (j >= 0) {
+      if (nk >= (uint32_t)b.N) { atomicOr(b.status, ST_BOUNDS); nk = 0; }
+      const Rec* rp = b.rec + ((int64_t)ti.v * b.N + nk);
+      cp_async16(&sh.raw[0][lane], &rp->a);
+      cp_async16(&sh.raw[1][lane], &rp->b);
+      cp_async16(&sh.raw[2][lane], &rp->c);
+    }
+    cp_async_commit();
+  };
+  load_key(maxlast - lane);
+  copy_record(maxlast - lane);
+  uint32_t g = nk;
+  load_key(maxlast - 32 - lane);
+  int head = 0, have = 0;  // ring index of the next group, items in the ring
+  for (; top >= 0; top -= 32) {
+    cp_async_wait<0>();
+    // append the lane's entry if it can reach a pixel of the block
+    uint32_t m = 0;
+    float4 A, B, C;
+    if (top - lane >= 0 && (!kSync || top - lane <= mylast)) {
+      A = sh.raw[0][lane];
+      B = sh.raw[1][lane];
+      C = sh.raw[2][lane];
+      const uint32_t rx = __float_as_uint(B.w), ry = __float_as_uint(C.w);
+      const int c0 = max((int)(rx & 0xFFFFu) - RX, 0), c1 = min((int)(rx >> 16) - RX, 7);
+      const int r0 = max((int)(ry & 0xFFFFu) - RY, 0), r1 = min((int)(ry >> 16) - RY, 7);
+      const float X0 = ((float)RX + 0.5f) - A.x, Y0 = ((float)RY + 0.5f) - A.y;
+      if (c0 <= c1 && r0 <= r1 &&
+          box_reached(A.z, A.w, B.x, B.y, X0, X0 + 7.0f, Y0, Y0 + 7.0f, lg_amin))
+        m = (((2u << (c1 - c0)) - 1u) << c0) | ((((2u << (r1 - r0)) - 1u) << r0) << 8);
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, m != 0u);
+    bool big = false;
+    if (m) {
+      int pos = head + have + __popc(hit & ((1u << lane) - 1u));
+      pos = pos >= kBwdRing ? pos - kBwdRing : pos;
+      float* q = sh.ring + (pos >> 1) * kBwdPair;
+      const int h = pos & 1;
+      q[h] = A.x;
+      q[2 + h] = A.y;
+      q[4 + h] = A.z;
+      q[6 + h] = A.w;
+      q[8 + h] = B.x;
+      q[10 + h] = B.y;
+      float4* c4 = reinterpret_cast<float4*>(q + 12) + 2 * h;
+      c4[0] = make_float4(C.x, C.x, C.y, C.y);
+      c4[1] = make_float4(C.z, C.z, __uint_as_float(m), __int_as_float(top - lane));
+      sh.gid[pos] = g;
+      big = !(C.x <= kWild) || !(C.y <= kWild) || !(C.z <= kWild);
+    }
+    careful = __any_sync(0xffffffffu, big) || careful;
+    have += __popc(hit);
+    const uint32_t g_batch = g;
+    copy_record(top - 32 - lane);
+    g = nk;
+    load_key(top - 64 - lane);
+    if (kCount && lane == 0) n_evalb += (unsigned)__popc(hit);
+    const bool fin = kSync || top < 32;  // take what is in the ring whole
+    if (fin && (have & 1)) {
+      // an item of zeros that no pixel takes beside the last one (a group starts at an even
+      // index, so the last one is the first of its pair)
+      int pos = head + have;
+      pos = pos >= kBwdRing ? pos - kBwdRing : pos;
+      float* q = sh.ring + (pos >> 1) * kBwdPair;
+      if (lane < 6) q[2 * lane + 1] = 0.0f;
+      else if (lane < 14) q[14 + lane] = 0.0f;
+    }
+    __syncwarp();
+    while (have >= kBwdGroup || (fin && have > 0)) {
+      const int cnt = have < kBwdGroup ? have : kBwdGroup;
+#pragma unroll 4
+      for (int e = 0; e < cnt; e += 2) take_pair(head + e, e);
+      __syncwarp();
+      sum_group(head, cnt);
+      __syncwarp();
+      head = head + kBwdGroup == kBwdRing ? 0 : head + kBwdGroup;
+      have -= cnt;
+    }
+    if (kSync) {
+      const int par = (top >> 5) & 1;
+      if (lane == 0) cta->have[par][threadIdx.x >> 5] = hit;
+      __syncthreads();
+      // four threads per slot, one per part of the record
+      const int slot = (int)(threadIdx.x >> 2), part = (int)(threadIdx.x & 3);
+      const uint32_t gs = __shfl_sync(0xffffffffu, g_batch, slot);
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (part < 3) {
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+          if ((cta->have[par][w] >> slot) & 1u) {
+            const float* a = cta->acc[par][w][slot] + 4 * part;
+            t.x += a[0];
+            if (part < 2) { t.y += a[1]; t.z += a[2]; t.w += a[3]; }
           }
-        } else {
-          float v[9] = {sx, sy, sxx, sxy, syy, go, gr, gg, gb};
-          float mine, v8;
-          warp_reduce9(v, lane, mine, v8);
-          // lanes 0, 4, ..., 28 hold the sums of values 0..7, lane 0 also value 8; the
-          // 2-D gradient record is 12 floats (sx, sy, sxx, sxy, syy, go, gr, gg, gb, -, -, -)
-          float* dst = reinterpret_cast<float*>(g2 + (int64_t)sG[jj] * 3);
-          if ((lane & 3) == 0) atomicAdd(dst + (lane >> 2), mine);
-          if (lane == 0) atomicAdd(dst + 8, v8);
+        if (t.x != 0.0f || t.y != 0.0f || t.z != 0.0f || t.w != 0.0f) {
+          float4* dst = b.grad2d + ((int64_t)ti.v * b.N + gs) * 3 + part;
+          if (part < 2) atomicAdd(dst, t);
+          else atomicAdd(&dst->x, t.x);
         }
       }
     }
   }
+  cp_async_wait<0>();
   if (kCount) {
     flush_counter(b.counters, 3, n_evalb);
     flush_counter(b.counters, 4, n_pixb);
@@ -850,41 +952,51 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_raster_fwd_retry(const BatchD
   }
 }
 
-template <int TS, int PPT, bool kCount, bool kPersist>
-__global__ void __launch_bounds__(TS * TS / PPT, (kMinBlocksBwd<TS, PPT>)) k_raster_bwd(const BatchDev b) {
-  __shared__ float4 sA[kNBBwd<TS, PPT>], sB[kNBBwd<TS, PPT>], sC[kNBBwd<TS, PPT>];
-  __shared__ uint32_t sG[kNBBwd<TS, PPT>];
-  __shared__ float4 sQ[TS * TS];  // composite adjoint per pixel slot
-  __shared__ int s_maxlast;
+// Backward CTAs: one warp per 8 x 8 block, up to four blocks per CTA (a 32x32 tile takes four
+// CTAs); the warps walk the tile's list on their own.
+template <int TS>
+constexpr int kBwdWarps = TS == 8 ? 1 : 4;
+template <int TS>
+constexpr int kBwdSplit = TS * TS / 64 / kBwdWarps<TS>;  // CTAs per work item
+template <int TS, bool kSync, bool kCount, bool kPersist>
+__global__ void __launch_bounds__(32 * kBwdWarps<TS>, kSync ? 4 : kMinBlocksBwd<TS>)
+    k_raster_bwd(const BatchDev b) {
+  __shared__ BwdShared sh[kBwdWarps<TS>];
+  BwdSums* sums = nullptr;
+  if constexpr (kSync) {
+    __shared__ BwdSums s_sums;
+    sums = &s_sums;
+  }
+  const int w = (int)(threadIdx.x >> 5);
   if constexpr (!kPersist) {
-    bwd_item<TS, PPT, kCount>(b, blockIdx.x, sA, sB, sC, sG, s_maxlast, sQ);
+    const unsigned id = blockIdx.x / kBwdSplit<TS>, part = blockIdx.x % kBwdSplit<TS>;
+    bwd_item<TS, kSync, kCount>(b, id, (int)part * kBwdWarps<TS> + w, sh[w], sums);
   } else {
     __shared__ long long s_id;
     for (;;) {
       __syncthreads();
       if (threadIdx.x == 0) s_id = (long long)atomicAdd(b.work_ctr + 1, 1ull);
       __syncthreads();
-      const int64_t id = s_id;
+      const int64_t id = s_id / kBwdSplit<TS>, part = s_id % kBwdSplit<TS>;
       if (id >= b.n_tiles) return;
-      bwd_item<TS, PPT, kCount>(b, id, sA, sB, sC, sG, s_maxlast, sQ);
+      bwd_item<TS, kSync, kCount>(b, id, (int)part * kBwdWarps<TS> + w, sh[w], sums);
     }
   }
 }
 
-// Tile side -> pixels per thread.  Forward: 2 (8 x 8 regions per warp) for 8x8 and 16x16
-// tiles, 4 for 32x32; backward: 2 for 8x8, 8 (one warp per 16x16 tile) for 16x16, 4 (16 x 8
-// regions) for 32x32.  The backward's per-entry work (record loads, rectangle tests, the warp reduction
-// and its atomics) favours more pixels per lane: one warp per tile does it once per entry
-// instead of twice (21.0 ms at 8 pixels and 27 CTAs per SM, 22.0 at 4, 29.2 at 2).
+// Tile side -> pixels per thread of the forward: 2 (8 x 8 regions per warp) for 8x8 and 16x16
+// tiles, 4 (16 x 8) for 32x32.
 template <int TS>
 struct PptFwd {
   static constexpr int value = TS == 32 ? 4 : 2;
 };
-template <int TS>
-struct PptBwd {
-  static constexpr int value = TS == 8 ? 2 : (TS == 16 ? 8 : 4);
-};
-
+// Launches of at most this many 16x16 items take the backward's kSync form.  There one tile's
+// latency decides (a partial wave), and a Gaussian whose footprint lies inside one tile gets
+// its whole 2-D gradient by one add, so that small problems come out the same bit for bit
+// in every run; above it the tile's four warps add on their own, in any order.  Measured
+// (raster_bwd; before | warps on their own | kSync): 560 tiles 0.447 | 0.084 | 0.107 ms, 3800
+// tiles 0.523 | 0.133 | 0.179, 34.7k tiles 1.348 | 0.896 | 1.219.
+constexpr int64_t kSyncItems = 1024;
 // Work is counted only by eager runs with a counter buffer: a captured graph launches the
 // plain variants, so replays carry no counting instructions (and keep the eager counts).
 static bool counting(const BatchDev& b, cudaStream_t s) {
@@ -901,10 +1013,16 @@ static void launch_fwd_k(const BatchDev& b, cudaStream_t s) {
 }
 template <int TS, bool kCount, bool kPersist>
 static void launch_bwd_k(const BatchDev& b, cudaStream_t s) {
-  constexpr int P = PptBwd<TS>::value;
-  const unsigned grid = kPersist ? (unsigned)std::min<int64_t>(b.n_tiles, (int64_t)b.persist_grid)
-                                 : (unsigned)b.n_tiles;
-  k_raster_bwd<TS, P, kCount, kPersist><<<grid, TS * TS / P, 0, s>>>(b);
+  const int64_t items = b.n_tiles * kBwdSplit<TS>;
+  const unsigned grid = kPersist ? (unsigned)std::min<int64_t>(items, (int64_t)b.persist_grid)
+                                 : (unsigned)items;
+  if constexpr (TS == 16) {
+    if (b.n_tiles <= kSyncItems) {
+      k_raster_bwd<TS, true, kCount, kPersist><<<grid, 32 * kBwdWarps<TS>, 0, s>>>(b);
+      return;
+    }
+  }
+  k_raster_bwd<TS, false, kCount, kPersist><<<grid, 32 * kBwdWarps<TS>, 0, s>>>(b);
 }
 template <int TS>
 static void launch_fwd_t(const BatchDev& b, cudaStream_t s) {
@@ -923,11 +1041,11 @@ static void launch_bwd_t(const BatchDev& b, cudaStream_t s) {
 
 template <int TS>
 static int max_ctas_t(bool bwd) {
-  constexpr int PF = PptFwd<TS>::value, PB = PptBwd<TS>::value;
+  constexpr int PF = PptFwd<TS>::value;
   int n = 0;
   cudaError_t e =
-      bwd ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_raster_bwd<TS, PB, false, true>,
-                                                          TS * TS / PB, 0)
+      bwd ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_raster_bwd<TS, false, false, true>,
+                                                          32 * kBwdWarps<TS>, 0)
           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_raster_fwd<TS, PF, false, true>,
                                                           TS * TS / PF, 0);
   return e == cudaSuccess ? n : 0;

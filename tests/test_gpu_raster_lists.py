@@ -108,3 +108,33 @@ def test_infinite_colour_stays_in_its_pixels(ctx, tile):
     assert 0 < alone.sum() < n
     fin = np.isfinite(s1).all(axis=(1, 2))
     assert np.allclose(s0[fin], s1[fin], rtol=1e-4, atol=1e-6)
+
+
+@pytest.mark.parametrize("w", [512, 528])
+def test_backward_on_both_sides_of_its_launch_rule(ctx, w):
+    """1024 and 1056 tiles of 16x16 (the backward's forms for small and for larger launches)
+    against the 8x8 tiles' backward and the oracle: the same sums, added in another order."""
+    from paper_2606_18588_gb300 import splx as S
+    from gpu_util import GRAD_TOL, backward_view, band_share, rel_l2, render_view, to_device
+    n = 400
+    sc = _scene(n, False)
+    off = np.array([0, n])
+    cam = I.pinhole(w, 512, 60.0, (0.0, 0.0, -2.0), (0.0, 0.0, 0.0))
+    dev = to_device(sc)
+    ref = O.render_view(sc, off, cam, O.opts(), bounds=True)
+    rng = np.random.default_rng(9)
+    dl = rng.standard_normal((3, 512, w)) * (ref["amb"] == 0)
+    band_share(ref["amb"], budget=0.02, label=f"{w} x 512")
+    gref = O.backward_view(sc, off, cam, dl, None, O.opts())
+    got = {}
+    for tile in (16, 8):
+        o = S.opts(tile=tile)
+        _, _, parts, states = render_view(ctx, dev, off, cam, o, 0)
+        got[tile] = backward_view(ctx, dev, off, cam, o, 0, parts, states,
+                                  torch.from_numpy(dl.astype(np.float32)).cuda())
+        for st in states:
+            st.close()
+    for k, gr in zip(GROUPS, gref):
+        a, b = got[16][k].cpu().numpy(), got[8][k].cpu().numpy()
+        assert rel_l2(a, gr) <= GRAD_TOL, k
+        assert rel_l2(a, b) <= 1e-5, k
