@@ -1,6 +1,16 @@
 // Global composition (Eq. 5) and its adjoint (Eq. 6-7), one thread per pixel of every
 // view of the batch, plus the L1 photometric loss.
 //
+// Both are bound by HBM latency rather than bandwidth: their work per byte is a sort of a few
+// keys.  A warp takes a patch of one tile, so the subsets whose visible region misses the
+// tile drop out for all its lanes at once, before anything is read; what is left is loaded,
+// sorted and blended in registers, with the pointers of all planes in the lanes' registers
+// and the colours of four subsets in flight.  Before, a thread looped over all K subsets and
+// kept their keys and order in local memory.  Measured (composite, adjoint): K = 32, 4 views
+// 1920x1080 of the 20M-Gaussian city, where a tile has one or two subsets, 0.97 -> 0.14 and
+// 1.64 -> 0.19 ms; K = 8, 16 views of 10M 0.64 -> 0.46 and 1.02 -> 0.66 ms; 16 partials of
+// 1600x1064 from outside 211 -> 156 us (3.7 TB/s).
+//
 // Order: subsets sorted per pixel by the normalised depth D^m / (1 - T^m), a convex
 // combination of the subset's contributor depths (Eq. 4 read as D = sum d alpha T);
 // ties go to the lower subset index and subsets with no contributor (T^m = 1) go last.
@@ -13,140 +23,358 @@
 
 namespace splx {
 
-template <int MK>
-struct PixOrder {
-  float T[MK], key[MK];
-  int ord[MK];
-  int K;
-  uint64_t outside;  // bit m: the pixel's tile lies outside subset m's visible region
+namespace {
 
-  // Partials of subsets whose visible region misses the pixel's tile were never written:
-  // they are empty (C = 0, T = 1, D = 0) and are not read.
-  __device__ __forceinline__ void load(const BatchDev& b, int v, int64_t p, int W) {
-    K = b.K;
-    outside = 0;
-    int tx = 0, ty = 0;
-    if (b.omega) {
-      const int sh = __ffs(b.tile) - 1;  // the tile side is a power of two
-      const uint32_t py = (uint32_t)p / (uint32_t)W;
-      tx = (int)(((uint32_t)p - py * (uint32_t)W) >> sh);
-      ty = (int)(py >> sh);
+// A warp's 32 pixels: a patch of one tile (32x1, 16x2 or 8x4 for tiles of 32, 16, 8), so that
+// the subsets whose visible region holds the tile are the same for all of them.
+struct Patch {
+  int v;
+  bool in;          // the lane's pixel lies in the image
+  int64_t p, HW;    // its index in the view's planes, pixels of the view
+  uint64_t inside;  // bit m: subset m's visible region holds the tile
+};
+
+__device__ __forceinline__ Patch patch_of(const BatchDev& b, int64_t warp) {
+  Patch q;
+  const int lane = (int)(threadIdx.x & 31);
+  const int sh = __ffs(b.tile) - 1;  // the tile side is a power of two
+  const int pp = 2 * sh - 5;         // log2 of the patches per tile
+  const int64_t t = warp >> pp;
+  q.v = view_of(b.tile_base, b.V, t * b.K);
+  const ViewDev& cam = b.views[q.v];
+  // (a view's tiles, and those before it, number fewer than 2^31)
+  const uint32_t loc = (uint32_t)t - (uint32_t)b.tile_base[q.v] / (uint32_t)b.K;
+  const int ty = (int)(loc / (uint32_t)cam.tiles_x), tx = (int)(loc - (uint32_t)ty * cam.tiles_x);
+  const int rows = 5 - sh;  // log2 of the patch's rows
+  const int x = (tx << sh) + (lane & (b.tile - 1));
+  const int y = (ty << sh) + ((int)(warp & ((1 << pp) - 1)) << rows) + (lane >> sh);
+  q.in = x < cam.W && y < cam.H;
+  q.HW = (int64_t)cam.W * cam.H;
+  q.p = q.in ? (int64_t)y * cam.W + x : 0;
+  q.inside = 0;
+  for (int m0 = 0; m0 < b.K; m0 += 32) {
+    const int m = m0 + lane;
+    const unsigned bits = __ballot_sync(0xffffffffu, m < b.K && in_omega(b, q.v, m, tx, ty));
+    q.inside |= (uint64_t)bits << m0;
+  }
+  return q;
+}
+
+// One plane pointer of every subset, held by the warp's lanes (lane l: subsets l and l + 32):
+// one table read for all subsets, then a shuffle per use instead of a dependent read.  get()
+// is for the whole warp; m may differ from lane to lane.
+template <bool kWide>
+struct Planes {
+  unsigned long long lo, hi;
+  __device__ __forceinline__ void set(const void* a, const void* b) {
+    lo = reinterpret_cast<unsigned long long>(a);
+    hi = reinterpret_cast<unsigned long long>(b);
+  }
+  template <typename P>
+  __device__ __forceinline__ P get(int m) const {
+    unsigned long long r = __shfl_sync(0xffffffffu, lo, m & 31);
+    if (kWide) {
+      const unsigned long long h = __shfl_sync(0xffffffffu, hi, m & 31);
+      r = m < 32 ? r : h;
     }
+    return reinterpret_cast<P>(r);
+  }
+};
+// The table rows of the lane's two subsets (any valid row beyond K).
+__device__ __forceinline__ const ImgDev* lane_img(const BatchDev& b, const Patch& q, int half) {
+  const int m = (int)(threadIdx.x & 31) + 32 * half;
+  return b.imgs + q.v * b.K + (m < b.K ? m : 0);
+}
+
+// The inside subsets of the lane's pixel in composition order: by the normalised depth D / (1 -
+// T), ties to the lower index, empty ones (T = 1) last.  n <= M of them (the same n for all
+// lanes); everything stays in registers.  Subsets outside are empty and never written or
+// read: they would stand among the last and add nothing.
+template <int M, bool kWide>
+struct PixOrder {
+  float T[M], key[M];
+  int idx[M];
+
+  __device__ __forceinline__ void load(const BatchDev& b, const Patch& q, int n) {
+    Planes<kWide> pt, pd;
+    const ImgDev *a = lane_img(b, q, 0), *c = kWide ? lane_img(b, q, 1) : a;
+    pt.set(a->T, c->T);
+    pd.set(a->D, c->D);
+    uint64_t rest = q.inside;
 #pragma unroll
-    for (int m = 0; m < MK; ++m) {
-      if (m < K) {
-        if (!in_omega(b, v, m, tx, ty)) {
-          outside |= 1ull << m;
-          T[m] = 1.0f;
-          key[m] = __int_as_float(0x7f800000);
-          continue;
-        }
-        const ImgDev& im = b.imgs[v * b.K + m];
-        const float t = im.T[p];
-        const float d = im.D[p];
-        T[m] = t;
-        key[m] = t < 1.0f ? d / (1.0f - t) : __int_as_float(0x7f800000);
+    for (int i = 0; i < M; ++i) {
+      T[i] = 1.0f;
+      key[i] = 0.0f;
+      idx[i] = 0;
+      if (i < n) {
+        const int m = __ffsll((long long)rest) - 1;
+        rest &= rest - 1;
+        idx[i] = m;
+        T[i] = pt.template get<const float*>(m)[q.p];
+        key[i] = pd.template get<const float*>(m)[q.p];
       }
     }
-    // insertion sort of indices by (key, index): stable
-    for (int m = 0; m < K; ++m) {
-      int j = m;
-      const float km = key[m];
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+      if (i < n) key[i] = T[i] < 1.0f ? key[i] / (1.0f - T[i]) : __int_as_float(0x7f800000);
+    // insertion by exchanges of neighbours (stable)
+#pragma unroll
+    for (int i = 1; i < M; ++i) {
+      if (i < n) {
+#pragma unroll
+        for (int j = i; j > 0; --j) {
+          const bool sw = key[j - 1] > key[j];
+          const float k = key[j], t = T[j];
+          const int x = idx[j];
+          key[j] = sw ? key[j - 1] : k;
+          T[j] = sw ? T[j - 1] : t;
+          idx[j] = sw ? idx[j - 1] : x;
+          key[j - 1] = sw ? k : key[j - 1];
+          T[j - 1] = sw ? t : T[j - 1];
+          idx[j - 1] = sw ? x : idx[j - 1];
+        }
+      }
+    }
+  }
+};
+
+// How many subsets' colours are loaded ahead of their use.
+constexpr int kAhead = 4;
+
+template <int M, bool kWide>
+__device__ __forceinline__ void composite_patch(const BatchDev& b, const Patch& q, int n) {
+  PixOrder<M, kWide> po;
+  po.load(b, q, n);
+  Planes<kWide> pr;
+  pr.set(lane_img(b, q, 0)->rgb, kWide ? lane_img(b, q, 1)->rgb : nullptr);
+  float P = 1.0f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+#pragma unroll
+  for (int j0 = 0; j0 < M; j0 += kAhead) {
+    if (j0 < n) {
+      // the colours of the next subsets up to the saturation cut, all in flight together
+      float r[kAhead], g[kAhead], bl[kAhead], w[kAhead];
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) {
+        const int j = j0 + i;
+        r[i] = g[i] = bl[i] = w[i] = 0.0f;
+        if (j < M && j < n) {
+          const float* rgb = pr.template get<const float*>(po.idx[j < M ? j : 0]);
+          if (!(P < b.eps_comp)) {
+            r[i] = rgb[q.p];
+            g[i] = rgb[q.HW + q.p];
+            bl[i] = rgb[2 * q.HW + q.p];
+            w[i] = P;
+            P *= po.T[j < M ? j : 0];
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) {
+        c0 = fmaf(r[i], w[i], c0);
+        c1 = fmaf(g[i], w[i], c1);
+        c2 = fmaf(bl[i], w[i], c2);
+      }
+    }
+  }
+  if (!q.in) return;
+  float* orgb = b.out_rgb + 3 * b.pix_off[q.v];
+  orgb[q.p] = fmaf(b.bg[0], P, c0);
+  orgb[q.HW + q.p] = fmaf(b.bg[1], P, c1);
+  orgb[2 * q.HW + q.p] = fmaf(b.bg[2], P, c2);
+  if (b.out_T) b.out_T[b.pix_off[q.v] + q.p] = P;
+}
+
+template <int M, bool kWide>
+__device__ __forceinline__ void composite_bwd_patch(const BatchDev& b, const Patch& q, int n) {
+  const float* dl = b.dL_drgb + 3 * b.pix_off[q.v];
+  const float g0 = dl[q.p], g1 = dl[q.HW + q.p], g2 = dl[2 * q.HW + q.p];
+  const float gT = b.dL_dT ? b.dL_dT[b.pix_off[q.v] + q.p] : 0.0f;
+  PixOrder<M, kWide> po;
+  po.load(b, q, n);
+  Planes<kWide> pr, pg;
+  const ImgDev *ia = lane_img(b, q, 0), *ib = kWide ? lane_img(b, q, 1) : ia;
+  pr.set(ia->rgb, ib->rgb);
+  pg.set(ia->gCT, ib->gCT);
+  // key[j] becomes the prefix P_j; bit j of inc: included (before the saturation cut)
+  float P = 1.0f;
+  unsigned inc = 0;
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    po.key[j] = P;
+    if (j < n && !(P < b.eps_comp)) {
+      inc |= 1u << j;
+      P *= po.T[j];
+    }
+  }
+  float S0 = b.bg[0], S1 = b.bg[1], S2 = b.bg[2], Rt = 1.0f;
+#pragma unroll
+  for (int j1 = (M - 1) / kAhead * kAhead; j1 >= 0; j1 -= kAhead) {
+    if (j1 < n) {
+      // the colours of the next subsets back to front, all in flight together
+      float r[kAhead], g[kAhead], bl[kAhead];
+      float4* out[kAhead];
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) {
+        const int j = j1 + i < M ? j1 + i : 0;
+        r[i] = g[i] = bl[i] = 0.0f;
+        out[i] = nullptr;
+        if (j1 + i < M && j1 + i < n) {
+          const float* rgb = pr.template get<const float*>(po.idx[j]);
+          out[i] = pg.template get<float4*>(po.idx[j]) + q.p;
+          if ((inc >> j) & 1u) {
+            r[i] = rgb[q.p];
+            g[i] = rgb[q.HW + q.p];
+            bl[i] = rgb[2 * q.HW + q.p];
+          }
+        }
+      }
+#pragma unroll
+      for (int i = kAhead - 1; i >= 0; --i) {
+        const int j = j1 + i < M ? j1 + i : 0;
+        if (j1 + i < M && j1 + i < n) {
+          float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+          if ((inc >> j) & 1u) {
+            const float Pm = po.key[j];
+            const float gTm = (g0 * S0 + g1 * S1 + g2 * S2) * Pm + gT * Pm * Rt;
+            o = make_float4(g0 * Pm, g1 * Pm, g2 * Pm, gTm);
+            const float Tm = po.T[j];
+            S0 = fmaf(Tm, S0, r[i]);
+            S1 = fmaf(Tm, S1, g[i]);
+            S2 = fmaf(Tm, S2, bl[i]);
+            Rt *= Tm;
+          }
+          if (q.in) *out[i] = o;
+        }
+      }
+    }
+  }
+}
+
+// More inside subsets than the register forms hold: the same, through arrays indexed at run
+// time (local memory).
+struct PixOrderAny {
+  float T[kMaxK], key[kMaxK];
+  int ord[kMaxK];
+
+  __device__ __forceinline__ int load(const BatchDev& b, const Patch& q) {
+    int n = 0;
+    for (uint64_t rest = q.inside; rest; rest &= rest - 1) {
+      const int m = __ffsll((long long)rest) - 1;
+      const ImgDev& im = b.imgs[q.v * b.K + m];
+      const float t = im.T[q.p], d = im.D[q.p];
+      const float km = t < 1.0f ? d / (1.0f - t) : __int_as_float(0x7f800000);
+      T[m] = t;
+      key[m] = km;
+      int j = n++;
       while (j > 0 && key[ord[j - 1]] > km) {
         ord[j] = ord[j - 1];
         --j;
       }
       ord[j] = m;
     }
+    return n;
   }
 };
 
-template <int MK>
-__global__ void __launch_bounds__(256) k_composite(const BatchDev b, int64_t total) {
-  const int64_t gp = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gp >= total) return;
-  const int v = view_of(b.pix_off, b.V, gp);
-  const ViewDev& cam = b.views[v];
-  const int64_t HW = (int64_t)cam.W * cam.H;
-  const int64_t p = gp - b.pix_off[v];
-  PixOrder<MK> po;
-  po.load(b, v, p, cam.W);
+__device__ __noinline__ void composite_any(const BatchDev& b, const Patch& q) {
+  if (!q.in) return;
+  PixOrderAny po;
+  const int n = po.load(b, q);
   float P = 1.0f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-  for (int j = 0; j < po.K; ++j) {
+  for (int j = 0; j < n; ++j) {
     if (P < b.eps_comp) break;
     const int m = po.ord[j];
-    if ((po.outside >> m) & 1ull) continue;  // empty: adds nothing, T = 1
-    const float* rgb = b.imgs[v * b.K + m].rgb;
-    c0 = fmaf(rgb[p], P, c0);
-    c1 = fmaf(rgb[HW + p], P, c1);
-    c2 = fmaf(rgb[2 * HW + p], P, c2);
+    const float* rgb = b.imgs[q.v * b.K + m].rgb;
+    c0 = fmaf(rgb[q.p], P, c0);
+    c1 = fmaf(rgb[q.HW + q.p], P, c1);
+    c2 = fmaf(rgb[2 * q.HW + q.p], P, c2);
     P *= po.T[m];
   }
-  float* orgb = b.out_rgb + 3 * b.pix_off[v];
-  orgb[p] = fmaf(b.bg[0], P, c0);
-  orgb[HW + p] = fmaf(b.bg[1], P, c1);
-  orgb[2 * HW + p] = fmaf(b.bg[2], P, c2);
-  if (b.out_T) b.out_T[b.pix_off[v] + p] = P;
+  float* orgb = b.out_rgb + 3 * b.pix_off[q.v];
+  orgb[q.p] = fmaf(b.bg[0], P, c0);
+  orgb[q.HW + q.p] = fmaf(b.bg[1], P, c1);
+  orgb[2 * q.HW + q.p] = fmaf(b.bg[2], P, c2);
+  if (b.out_T) b.out_T[b.pix_off[q.v] + q.p] = P;
 }
 
-template <int MK>
-__global__ void __launch_bounds__(256) k_composite_bwd(const BatchDev b, int64_t total) {
-  const int64_t gp = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gp >= total) return;
-  const int v = view_of(b.pix_off, b.V, gp);
-  const ViewDev& cam = b.views[v];
-  const int64_t HW = (int64_t)cam.W * cam.H;
-  const int64_t p = gp - b.pix_off[v];
-  PixOrder<MK> po;
-  po.load(b, v, p, cam.W);
-  float Pj[MK];
+__device__ __noinline__ void composite_bwd_any(const BatchDev& b, const Patch& q) {
+  if (!q.in) return;
+  PixOrderAny po;
+  const int n = po.load(b, q);
+  float Pj[kMaxK];
   float P = 1.0f;
   int L = 0;
-  for (int j = 0; j < po.K; ++j) {
+  for (int j = 0; j < n; ++j) {
     if (P < b.eps_comp) break;
     Pj[j] = P;
     P *= po.T[po.ord[j]];
     ++L;
   }
-  const float* dl = b.dL_drgb + 3 * b.pix_off[v];
-  const float g0 = dl[p], g1 = dl[HW + p], g2 = dl[2 * HW + p];
-  const float gT = b.dL_dT ? b.dL_dT[b.pix_off[v] + p] : 0.0f;
+  const float* dl = b.dL_drgb + 3 * b.pix_off[q.v];
+  const float g0 = dl[q.p], g1 = dl[q.HW + q.p], g2 = dl[2 * q.HW + q.p];
+  const float gT = b.dL_dT ? b.dL_dT[b.pix_off[q.v] + q.p] : 0.0f;
   float S0 = b.bg[0], S1 = b.bg[1], S2 = b.bg[2], Rt = 1.0f;
-  for (int j = po.K - 1; j >= 0; --j) {
+  for (int j = n - 1; j >= 0; --j) {
     const int m = po.ord[j];
-    const ImgDev& im = b.imgs[v * b.K + m];
-    if ((po.outside >> m) & 1ull) continue;  // empty and never rendered: T = 1, C = 0
+    const ImgDev& im = b.imgs[q.v * b.K + m];
     if (j >= L) {
-      im.gCT[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+      im.gCT[q.p] = make_float4(0.f, 0.f, 0.f, 0.f);
       continue;
     }
     const float Pm = Pj[j];
     const float gTm = (g0 * S0 + g1 * S1 + g2 * S2) * Pm + gT * Pm * Rt;
-    im.gCT[p] = make_float4(g0 * Pm, g1 * Pm, g2 * Pm, gTm);
+    im.gCT[q.p] = make_float4(g0 * Pm, g1 * Pm, g2 * Pm, gTm);
     const float Tm = po.T[m];
-    S0 = fmaf(Tm, S0, im.rgb[p]);
-    S1 = fmaf(Tm, S1, im.rgb[HW + p]);
-    S2 = fmaf(Tm, S2, im.rgb[2 * HW + p]);
+    S0 = fmaf(Tm, S0, im.rgb[q.p]);
+    S1 = fmaf(Tm, S1, im.rgb[q.HW + q.p]);
+    S2 = fmaf(Tm, S2, im.rgb[2 * q.HW + q.p]);
     Rt *= Tm;
   }
 }
 
-template <int MK>
-static void launch_c(const BatchDev& b, int64_t total, bool bwd, cudaStream_t s) {
-  const int threads = 256;
-  const unsigned blocks = (unsigned)((total + threads - 1) / threads);
-  if (bwd) k_composite_bwd<MK><<<blocks, threads, 0, s>>>(b, total);
-  else k_composite<MK><<<blocks, threads, 0, s>>>(b, total);
+}  // namespace
+
+// MK: the largest number of inside subsets taken in registers (4, 8 or 16 by K); kAny: more
+// are possible (K > 16; those kernels keep to 8 in registers, whose 48 and 64 registers hold
+// twice the warps of 16's 74 and 96, since few tiles have more).  A warp runs the form for its
+// own tile's number of subsets.
+template <int MK, bool kAny, bool kBwd>
+__global__ void __launch_bounds__(256) k_composite(const BatchDev b, int64_t warps) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= warps) return;
+  const Patch q = patch_of(b, w);
+  const int n = __popcll(q.inside);
+  if (MK > 4 && n > 4) {
+    if (MK > 8 && n > 8) {
+      if (kAny && n > MK) {
+        if (kBwd) composite_bwd_any(b, q); else composite_any(b, q);
+      } else {
+        if (kBwd) composite_bwd_patch<MK, kAny>(b, q, n); else composite_patch<MK, kAny>(b, q, n);
+      }
+    } else if (kAny && MK <= 8 && n > MK) {
+      if (kBwd) composite_bwd_any(b, q); else composite_any(b, q);
+    } else {
+      if (kBwd) composite_bwd_patch<8, kAny>(b, q, n); else composite_patch<8, kAny>(b, q, n);
+    }
+  } else {
+    if (kBwd) composite_bwd_patch<4, kAny>(b, q, n); else composite_patch<4, kAny>(b, q, n);
+  }
+}
+
+template <int MK, bool kAny>
+static void launch_c(const BatchDev& b, int64_t warps, bool bwd, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((warps + 7) / 8);
+  if (bwd) k_composite<MK, kAny, true><<<blocks, 256, 0, s>>>(b, warps);
+  else k_composite<MK, kAny, false><<<blocks, 256, 0, s>>>(b, warps);
 }
 
 static void dispatch(const BatchDev& b, int64_t total, bool bwd, cudaStream_t s) {
   if (total <= 0) return;
-  if (b.K <= 1) launch_c<1>(b, total, bwd, s);
-  else if (b.K <= 4) launch_c<4>(b, total, bwd, s);
-  else if (b.K <= 8) launch_c<8>(b, total, bwd, s);
-  else if (b.K <= 16) launch_c<16>(b, total, bwd, s);
-  else if (b.K <= 32) launch_c<32>(b, total, bwd, s);
-  else launch_c<64>(b, total, bwd, s);
+  const int64_t warps = b.n_tiles / b.K * (b.tile * b.tile / 32);
+  if (b.K <= 4) launch_c<4, false>(b, warps, bwd, s);
+  else if (b.K <= 8) launch_c<8, false>(b, warps, bwd, s);
+  else if (b.K <= 16) launch_c<16, false>(b, warps, bwd, s);
+  else launch_c<8, true>(b, warps, bwd, s);
   count_launch();
 }
 
