@@ -204,6 +204,8 @@ struct AdamTable {
   // optional, [ceil(N / 128)]: the fused projection adjoint leaves to a second, streaming
   // pass the 128-Gaussian blocks in which no Gaussian has a gradient (flag 1)
   uint8_t* defer;
+  // [8]: the step's bias-corrected rates, written by the update's first kernel
+  const float* scales;
 };
 
 __host__ __device__ inline int n_sh(int deg) { return (deg + 1) * (deg + 1); }
