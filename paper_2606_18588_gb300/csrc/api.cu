@@ -228,10 +228,11 @@ struct Plan {
   uint32_t* tile_start = nullptr;
   uint64_t* keys = nullptr;
   uint64_t* keys_alt = nullptr;
-  uint32_t* big_list = nullptr;
-  unsigned* big_count = nullptr;
+  uint32_t* seg_done = nullptr;
   uint2* chunks = nullptr;
-  unsigned* chunk_count = nullptr;
+  // [kGroups][K][kSortCounts]: the sort counters of each view group's waves (the first ones
+  // serve launches without waves)
+  unsigned* sort_counts = nullptr;
   uint2* ranges = nullptr;
   float4* grad2d = nullptr;
   uint8_t* defer = nullptr;  // [ceil(N / 128)]: blocks left to the zero-gradient Adam pass
@@ -245,19 +246,14 @@ struct Plan {
   bool split_views = false;
   cudaStream_t side[kGroups - 1] = {};
   cudaEvent_t fork_ev = nullptr, join_ev[kGroups - 1] = {};
-  uint32_t* big_list_g[kGroups - 1] = {};
-  unsigned* big_count_g[kGroups - 1] = {};
   uint2* chunks_g[kGroups - 1] = {};
-  unsigned* chunk_count_g[kGroups - 1] = {};
   // selected-prefix sort of long segments (batches; see BatchDev::sel): per image tile the
   // prefix length, and per view group the forward's retry list and its count
   bool select_prefix = false;
   bool alt_in_keys = false;  // keys_alt = keys + capacity (one allocation, owned by keys)
   uint32_t* sel = nullptr;
   uint32_t* retry = nullptr;
-  unsigned* retry_count = nullptr;
   uint32_t* retry_g[kGroups - 1] = {};
-  unsigned* retry_count_g[kGroups - 1] = {};
   int32_t* order_d = nullptr;              // [V][K] front-to-back subset order (skipping on)
   int32_t* rank_d = nullptr;               // [V][K] rank of subset k in view v's order
   // stale saturation state (with order_d): device table of the V views' state planes;
@@ -331,8 +327,8 @@ struct Plan {
     for (int c = 0; c < 3; ++c) b.bg[c] = opts.bg[c];
     b.subsets = subsets_d; b.views = views_d; b.imgs = imgs_d;
     b.rec = rec; b.counts = counts; b.tile_cnt = tile_cnt; b.tile_start = tile_start;
-    b.keys = keys; b.keys_alt = keys_alt; b.big_list = big_list; b.big_count = big_count;
-    b.chunks = chunks; b.chunk_count = chunk_count;
+    b.keys = keys; b.keys_alt = keys_alt; b.chunks = chunks;
+    b.seg_done = seg_done; set_sort_counts(b, sort_counts);
     b.ranges = ranges; b.grad2d = grad2d;
     b.status = ctx->d_status;
     b.counters = counters;
@@ -361,7 +357,6 @@ struct Plan {
     // (the cross-boundary filter's removed pairs keep the whole-segment sort)
     b.sel = select_prefix && alt_in_keys && sel && !b.removed ? sel : nullptr;
     b.retry = retry;
-    b.retry_count = retry_count;
     // composite-only plans carry no subsets; their offsets are unused
     for (int k = 0; k <= K; ++k) b.goff[k] = k < (int)subsets_h.size() ? subsets_h[k].goff : N;
     for (int v = 0; v <= V; ++v) { b.tile_base[v] = tile_base[v]; b.pix_off[v] = pix_off[v]; }
@@ -380,21 +375,17 @@ struct Plan {
     }
     void** ps[] = {(void**)&subsets_d, (void**)&views_d, (void**)&imgs_d, (void**)&rec,
                    (void**)&counts, (void**)&tile_cnt, (void**)&tile_start, (void**)&keys,
-                   (void**)&keys_alt, (void**)&big_list, (void**)&big_count, (void**)&chunks,
-                   (void**)&chunk_count, (void**)&ranges,
+                   (void**)&keys_alt, (void**)&seg_done, (void**)&sort_counts, (void**)&chunks,
+                   (void**)&ranges,
                    (void**)&grad2d, (void**)&defer, (void**)&scales, (void**)&scan_temp, (void**)&counters, (void**)&work_ctr,
                    (void**)&order_d, (void**)&rank_d, (void**)&sat_d, (void**)&tpre,
                    (void**)&omega, (void**)&cells_d,
                    (void**)&cross, (void**)&zr, (void**)&removed, (void**)&omega_x,
-                   (void**)&zr_x, (void**)&sel, (void**)&retry, (void**)&retry_count};
+                   (void**)&zr_x, (void**)&sel, (void**)&retry};
     for (void** p : ps) free_ptr(*p, s);
     for (int g = 0; g < kGroups - 1; ++g) {
       free_ptr((void*&)retry_g[g], s);
-      free_ptr((void*&)retry_count_g[g], s);
-      free_ptr((void*&)big_list_g[g], s);
-      free_ptr((void*&)big_count_g[g], s);
       free_ptr((void*&)chunks_g[g], s);
-      free_ptr((void*&)chunk_count_g[g], s);
       if (side[g]) { cudaStreamSynchronize(side[g]); cudaStreamDestroy(side[g]); side[g] = nullptr; }
       if (join_ev[g]) { cudaEventDestroy(join_ev[g]); join_ev[g] = nullptr; }
     }
@@ -404,6 +395,10 @@ struct Plan {
     for (auto& e : wev)
       if (e) cudaEventDestroy(e);
     wev.clear();
+  }
+
+  size_t sort_counts_bytes() const {
+    return sizeof(unsigned) * kSortCounts * kGroups * (size_t)std::max(K, 1);
   }
 
   // Project (counting pairs per tile) and scan the counts into segment starts.
@@ -417,8 +412,7 @@ struct Plan {
     if (b.zr) CK(cudaMemsetAsync(zr, 0xFF, sizeof(uint32_t) * 2 * (size_t)V * K, s));
     if (b.removed)
       CK(cudaMemsetAsync(removed, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(n_tiles, 1), s));
-    CK(cudaMemsetAsync(big_count, 0, 2 * sizeof(unsigned), s));
-    CK(cudaMemsetAsync(chunk_count, 0, sizeof(unsigned), s));
+    CK(cudaMemsetAsync(sort_counts, 0, sort_counts_bytes(), s));
     mark(0, s);
     launch_project(b, s);
     CK_LAUNCH();
@@ -438,8 +432,7 @@ struct Plan {
     // with saturation-skipping waves each wave sorts its own segments; with a stale state
     // one sort covers the tiles it leaves open
     if (!order_d || stale()) {
-      if (b.sel) CK(cudaMemsetAsync(retry_count, 0, sizeof(unsigned), s));
-      launch_seg_sort(b, merge_rounds_bound(max_subset()), s);
+      launch_seg_sort(b, s);
       CK_LAUNCH();
     }
     mark(4, s);
@@ -482,19 +475,15 @@ struct Plan {
         bw.item_lo = tile_base[first[g]] / K;
         bw.item_n = tile_base[first[g + 1]] / K - bw.item_lo;
         if (g > 0) {
-          bw.big_list = big_list_g[g - 1]; bw.big_count = big_count_g[g - 1];
-          bw.chunks = chunks_g[g - 1]; bw.chunk_count = chunk_count_g[g - 1];
-          bw.retry = retry_g[g - 1]; bw.retry_count = retry_count_g[g - 1];
+          bw.chunks = chunks_g[g - 1];
+          bw.retry = retry_g[g - 1];
         }
+        set_sort_counts(bw, sort_counts + kSortCounts * (g * K + r));
       }
       if (r > 0) mark_wave(2 * r, s);
-      const int rounds = merge_rounds_bound(max_subset());
       for (int g = 0; g < G; ++g) {
         cudaStream_t sg = g ? side[g - 1] : s;
-        CK(cudaMemsetAsync(bg[g].big_count, 0, 2 * sizeof(unsigned), sg));
-        CK(cudaMemsetAsync(bg[g].chunk_count, 0, sizeof(unsigned), sg));
-        if (bg[g].sel) CK(cudaMemsetAsync(bg[g].retry_count, 0, sizeof(unsigned), sg));
-        launch_seg_sort(bg[g], rounds, sg);
+        launch_seg_sort(bg[g], sg);
       }
       mark_wave(2 * r + 1, s);
       for (int g = 0; g < G; ++g) {
@@ -502,7 +491,7 @@ struct Plan {
         launch_raster_fwd(bg[g], sg);
         // items whose pixels were still open at the end of their selected prefix: full
         // sort, second forward
-        launch_sort_retries(bg[g], rounds, sg);
+        launch_sort_retries(bg[g], sg);
         launch_raster_fwd_retry(bg[g], sg);
       }
       CK_LAUNCH();
@@ -543,14 +532,9 @@ struct Plan {
     return SPLX_OK;
   }
 
-  // The other view groups' streams, events and long-segment lists (split_views).
-  int alloc_split(cudaStream_t s) {
-    int r;
-    const size_t nt = (size_t)std::max<int64_t>(n_tiles, 1);
+  // The other view groups' streams and events (split_views).
+  int alloc_split() {
     for (int g = 0; g < kGroups - 1; ++g) {
-      if ((r = ctx_alloc_t(ctx, &big_list_g[g], nt, s))) return r;
-      if ((r = ctx_alloc_t(ctx, &big_count_g[g], 2, s))) return r;
-      if ((r = ctx_alloc_t(ctx, &chunk_count_g[g], 1, s))) return r;
       CK(cudaStreamCreateWithFlags(&side[g], cudaStreamNonBlocking));
       CK(cudaEventCreateWithFlags(&join_ev[g], cudaEventDisableTiming));
     }
@@ -565,16 +549,10 @@ struct Plan {
     const size_t nt = (size_t)std::max<int64_t>(n_tiles, 1);
     if ((r = ctx_alloc_t(ctx, &sel, nt, s))) return r;
     if ((r = ctx_alloc_t(ctx, &retry, nt, s))) return r;
-    if ((r = ctx_alloc_t(ctx, &retry_count, 1, s))) return r;
     if (split_views)
-      for (int g = 0; g < kGroups - 1; ++g) {
+      for (int g = 0; g < kGroups - 1; ++g)
         if ((r = ctx_alloc_t(ctx, &retry_g[g], nt, s))) return r;
-        if ((r = ctx_alloc_t(ctx, &retry_count_g[g], 1, s))) return r;
-      }
     CK(cudaMemsetAsync(sel, 0, sizeof(uint32_t) * nt, s));
-    CK(cudaMemsetAsync(retry_count, 0, sizeof(unsigned), s));
-    for (int g = 0; g < kGroups - 1; ++g)
-      if (retry_count_g[g]) CK(cudaMemsetAsync(retry_count_g[g], 0, sizeof(unsigned), s));
     select_prefix = true;
     return SPLX_OK;
   }
@@ -589,9 +567,8 @@ struct Plan {
     if ((r = ctx_alloc_t(ctx, &counts, (size_t)std::max<int64_t>((int64_t)V * N, 1), s))) return r;
     if ((r = ctx_alloc_t(ctx, &tile_cnt, nt, s))) return r;
     if ((r = ctx_alloc_t(ctx, &tile_start, nt + 1, s))) return r;
-    if ((r = ctx_alloc_t(ctx, &big_list, nt, s))) return r;
-    if ((r = ctx_alloc_t(ctx, &big_count, 2, s))) return r;  // count, most chunks of one
-    if ((r = ctx_alloc_t(ctx, &chunk_count, 1, s))) return r;
+    if ((r = ctx_alloc_t(ctx, &seg_done, nt, s))) return r;
+    if ((r = ctx_alloc(ctx, (void**)&sort_counts, sort_counts_bytes(), s))) return r;
     if ((r = ctx_alloc(ctx, &scan_temp, scan_u32_temp_bytes(n_tiles), s))) return r;
     if ((r = ctx_alloc_t(ctx, &ranges, nt, s))) return r;
     if (!subsets_h.empty())
@@ -603,12 +580,6 @@ struct Plan {
       CK(cudaMemcpyAsync(imgs_d, imgs_h.data(), sizeof(ImgDev) * imgs_h.size(),
                          cudaMemcpyHostToDevice, s));
     return SPLX_OK;
-  }
-
-  int64_t max_subset() const {
-    int64_t m = 0;
-    for (const SubsetDev& d : subsets_h) m = std::max<int64_t>(m, d.n);
-    return m;
   }
 
   // Pair count of the last projection (synchronises).
@@ -798,10 +769,9 @@ static int render_partial_impl(splx_ctx_t ctx, const splx_gaussians* subset,
   P.free_ptr((void*&)P.scan_temp, s);
   P.free_ptr((void*&)P.keys_alt, s);
   P.free_ptr((void*&)P.tile_cnt, s);
-  P.free_ptr((void*&)P.big_list, s);
-  P.free_ptr((void*&)P.big_count, s);
+  P.free_ptr((void*&)P.seg_done, s);
+  P.free_ptr((void*&)P.sort_counts, s);
   P.free_ptr((void*&)P.chunks, s);
-  P.free_ptr((void*&)P.chunk_count, s);
   if (!state_out) return fail(SPLX_OK);
   *state_out = st;
   return SPLX_OK;
@@ -1179,7 +1149,7 @@ int splx_batch_create(splx_ctx_t ctx, const splx_gaussians* subsets, int32_t K,
     }
   }
   if ((r = P.alloc_common(s))) return fail(r);
-  if (V >= 2 && (r = P.alloc_split(s))) return fail(r);
+  if (V >= 2 && (r = P.alloc_split())) return fail(r);
   if ((r = P.alloc_select(s))) return fail(r);
   if ((r = ctx_alloc_t(ctx, &P.grad2d, (size_t)V * N * 3, s))) return fail(r);
   if ((r = ctx_alloc_t(ctx, &P.counters, kCounters, s))) return fail(r);
@@ -1249,7 +1219,7 @@ int splx_batch_forward(splx_batch_t bt, float* out_rgb, float* out_T, splx_strea
   } else {
     // (with a stale saturation state the rasteriser leaves the pruned pixels empty)
     launch_raster_fwd(b, s);
-    launch_sort_retries(b, merge_rounds_bound(P.max_subset()), s);
+    launch_sort_retries(b, s);
     launch_raster_fwd_retry(b, s);
   }
   P.mark(5, s);

@@ -15,8 +15,9 @@
 // Longer segments are cut into 4096-key chunks, each sorted the same way by a CTA of 512
 // threads, and then merged pairwise in rounds (run width 4096, 8192, ...) with merge-path
 // partitioning, one CTA per 4096 outputs, ping-ponging between the key buffer and its
-// twin; segments that end in the twin are copied back.  Every pair is read and written a
-// few times instead of once per 8-bit pass over 50+ key bits.
+// twin so that the last round ends in the key buffer.  Chunk sorts and all rounds are one
+// launch (k_long_sort).  Every pair is read and written a few times instead of once per
+// 8-bit pass over 50+ key bits.
 #include "common.cuh"
 #include "spec.cuh"
 #include "walk.cuh"
@@ -27,7 +28,7 @@ namespace {
 
 constexpr int kChunk = 2048;     // a segment up to this long is sorted by one CTA
 constexpr int kSortThreads = 256;
-constexpr int kBig = 4096;       // chunk of a longer segment (sorted, then merged)
+constexpr int kBig = (int)kSortChunk;  // chunk of a longer segment (sorted, then merged)
 constexpr int kBigThreads = 512;
 
 __device__ __forceinline__ int next_pow2(int n) {
@@ -125,22 +126,14 @@ __device__ __forceinline__ void sort_chunk(const uint64_t* in, uint64_t* out, in
   for (int i = threadIdx.x; i < n; i += TH) out[i] = src[pad(i)];
 }
 
-__device__ __forceinline__ void segment_of(const BatchDev& b, int64_t t, uint32_t& s, uint32_t& e) {
-  const uint64_t cap = (uint64_t)b.capacity;
-  uint64_t s64 = b.tile_start[t], e64 = b.tile_start[t + 1];
-  if (s64 > cap) s64 = cap;
-  if (e64 > cap) e64 = cap;
-  if (e64 < s64) e64 = s64;
-  s = (uint32_t)s64;
-  e = (uint32_t)e64;
-}
-
-// Merge rounds a segment of n keys needs: ceil(log2(number of chunks)).
-__device__ __forceinline__ int rounds_for(uint32_t n) {
-  const uint32_t nch = (n + kBig - 1) / kBig;
+// Merge rounds of a segment of nch chunks, and of one of n keys: ceil(log2(chunks)).
+__device__ __forceinline__ int rounds_of(uint32_t nch) {
   int r = 0;
   while ((1u << r) < nch) ++r;
   return r;
+}
+__device__ __forceinline__ int rounds_for(uint32_t n) {
+  return rounds_of(long_chunks(n));
 }
 
 // Number of elements taken from A among the first d of merge(A, B) (unique keys), found
@@ -152,7 +145,8 @@ __device__ __forceinline__ uint32_t merge_path_warp(const uint64_t* A, uint32_t 
   while (lo < hi) {
     const uint32_t span = hi - lo;
     const uint32_t m = lo + (uint32_t)(((uint64_t)span * (lane + 1)) / 33u);
-    const bool pred = A[m] < B[d - 1 - m];  // true exactly for m below the answer
+    // true exactly for m below the answer (past L1: other CTAs wrote the runs)
+    const bool pred = __ldcg(A + m) < __ldcg(B + (d - 1 - m));
     const unsigned bal = __ballot_sync(0xffffffffu, pred);
     const int nt = __popc(bal);
     const uint32_t m_last_true = __shfl_sync(0xffffffffu, m, nt > 0 ? nt - 1 : 0);
@@ -419,7 +413,7 @@ void launch_fill(const BatchDev& b, cudaStream_t s) {
 // longer one, its registration as chunk work items (segment list index, chunk index).
 __global__ void __launch_bounds__(kSortThreads) k_seg_sort_small(const BatchDev b) {
   __shared__ uint64_t sk[2][kPadded];
-  __shared__ unsigned s_base[2];
+  __shared__ unsigned s_base;
   __shared__ unsigned s_tmp[11];
   const int64_t t = item_of(b, blockIdx.x);
   uint32_t s, e;
@@ -441,178 +435,166 @@ __global__ void __launch_bounds__(kSortThreads) k_seg_sort_small(const BatchDev 
     return;
   }
   if (n > kChunk) {
-    const unsigned nch = (unsigned)((n + kBig - 1) / kBig);
-    if (threadIdx.x == 0) {
-      s_base[0] = atomicAdd(b.big_count, 1u);
-      s_base[1] = atomicAdd(b.chunk_count, nch);
-      atomicMax(b.big_count + 1, nch);
-    }
+    if (threadIdx.x == 0) s_base = register_long(b, t, (uint32_t)n);
     __syncthreads();
-    const unsigned i = s_base[0];
-    if (threadIdx.x == 0) b.big_list[i] = (uint32_t)t;
-    for (unsigned c = threadIdx.x; c < nch; c += kSortThreads) b.chunks[s_base[1] + c] = make_uint2(i, c);
+    const unsigned nch = long_chunks((uint32_t)n), first = s_base;
+    for (unsigned c = threadIdx.x; c < nch; c += kSortThreads)
+      b.chunks[first + c] = make_uint2((uint32_t)t, first);
     return;
   }
   sort_chunk<kSortThreads>(b.keys + s, b.keys + s, n, sk[0], sk[1]);
 }
 
-// Sorts every 4096-key chunk of the long segments (grid-stride over the chunk list); two
-// shared buffers of kBigPadded keys in dynamic shared memory.
-__global__ void __launch_bounds__(kBigThreads) k_chunk_sort(const BatchDev b) {
+// One merge item: outputs [o0, o0 + 4096) of the round that merges runs of w keys of a
+// segment of n keys from src to dst (both at the segment's start).  src holds what other
+// CTAs wrote earlier in the launch, so it is read past L1.
+__device__ __forceinline__ void merge_item(const uint64_t* src, uint64_t* dst, uint32_t n,
+                                           uint32_t w, uint32_t o0, uint64_t* sm,
+                                           uint32_t* s_split) {
+  constexpr int PER = kBig / kBigThreads;  // outputs per thread
+  const uint32_t o1 = o0 + kBig < n ? o0 + kBig : n;
+  const uint32_t p0 = (o0 / (2 * w)) * (2 * w);
+  const uint32_t na = (p0 + w < n ? p0 + w : n) - p0;
+  const uint32_t nb = (p0 + 2 * w < n ? p0 + 2 * w : n) - (p0 + na);
+  const uint64_t* A = src + p0;
+  const uint64_t* B = A + na;
+  // warp 0 finds the split at the block's first output, warp 1 at its end
+  if (threadIdx.x < 64) {
+    const uint32_t dd = (threadIdx.x < 32 ? o0 : o1) - p0;
+    const uint32_t a = merge_path_warp(A, na, B, nb, dd);
+    if ((threadIdx.x & 31) == 0) {
+      s_split[threadIdx.x >> 5] = a;
+      s_split[2 + (threadIdx.x >> 5)] = dd - a;
+    }
+  }
+  __syncthreads();
+  const uint32_t a0 = s_split[0], a1 = s_split[1], b0 = s_split[2], b1 = s_split[3];
+  const int la = (int)(a1 - a0), lb = (int)(b1 - b0);
+  for (int i = threadIdx.x; i < la; i += kBigThreads) sm[pad(i)] = __ldcg(A + a0 + i);
+  for (int i = threadIdx.x; i < lb; i += kBigThreads) sm[pad(la + i)] = __ldcg(B + b0 + i);
+  __syncthreads();
+  // each thread merges PER consecutive outputs of sm[0,la) and sm[la,la+lb)
+  const int d = threadIdx.x * PER;
+  if (d < la + lb) {
+    int ia = merge_path_smem(sm, 0, la, la, lb, d);
+    int ib = d - ia;
+    const int dend = d + PER < la + lb ? d + PER : la + lb;
+    uint64_t va = ia < la ? sm[pad(ia)] : ~0ull;  // run heads (~0 past the end)
+    uint64_t vb = ib < lb ? sm[pad(la + ib)] : ~0ull;
+    for (int o = d; o < dend; ++o) {
+      const bool takeA = va < vb;
+      dst[o0 + o] = takeA ? va : vb;
+      ia += takeA ? 1 : 0;
+      ib += takeA ? 0 : 1;
+      const bool more = takeA ? ia < la : ib < lb;
+      const uint64_t nv = more ? sm[takeA ? pad(ia) : pad(la + ib)] : ~0ull;
+      va = takeA ? nv : va;
+      vb = takeA ? vb : nv;
+    }
+  }
+}
+
+// Longest wait of a long-sort item for the earlier items of its segment: polls of about
+// half a microsecond, half a second in all (an item takes tens of microseconds).
+constexpr int kSortPolls = 1 << 20;
+
+// The long segments' whole sort in one launch: item (0, c) sorts chunk c of the chunk list,
+// item (1 + r, c) produces chunk c's 4096 outputs of merge round r (run width 4096 << r).
+// CTAs take the items in that order from a counter, and an item of a round starts when its
+// segment's chunk items of the round before are counted done (seg_done).  The order makes
+// the wait end: every earlier item was taken before and is held by a CTA that is running,
+// whether or not the whole grid is resident, and the earliest unfinished one never waits.
+// A segment merged in R rounds starts them in keys_alt when R is odd, so that its last round
+// writes keys; waiting for the whole segment keeps a round from overwriting what the round
+// before still reads.
+//
+// One launch instead of one per round: the rounds that the largest subset could need were
+// launched unseen, and most of them found nothing to do (city-scale waves: 8 of 11 launches
+// of each wave and view group; a 20M-Gaussian, 32-subset step 15.5 -> 14.1 ms, a 10k-Gaussian
+// 256x256 render 123 -> 111 us).  Two 36 KB buffers, dynamic shared memory, 3 CTAs per SM.
+__global__ void __launch_bounds__(kBigThreads) k_long_sort(const BatchDev b) {
   extern __shared__ uint64_t sk_dyn[];
   uint64_t* sa = sk_dyn;
   uint64_t* sb = sk_dyn + kBigPadded;
-  const unsigned count = *b.chunk_count;
-  for (unsigned w = blockIdx.x; w < count; w += gridDim.x) {
-    const uint2 ch = b.chunks[w];
-    const int64_t t = b.big_list[ch.x];
-    uint32_t s, e;
-    segment_of(b, t, s, e);
-    const uint32_t c0 = s + ch.y * kBig;
-    if (c0 >= e) continue;
-    const uint32_t c1 = c0 + kBig < e ? c0 + kBig : e;
-    // a segment merged in R rounds starts them in keys_alt when R is odd, so that its
-    // last round writes keys
-    uint64_t* out = ((rounds_for(e - s) & 1) ? b.keys_alt : b.keys) + c0;
-    sort_chunk<kBigThreads>(b.keys + c0, out, (int)(c1 - c0), sa, sb);
-    __syncthreads();
-  }
-}
-
-// Merge round r (run width 4096 << r): each chunk work item produces 4096 outputs of the
-// merge of the two runs its output range falls in.  A segment merged in R rounds holds the
-// input of round r in keys_alt when R - r is odd and in keys otherwise, so its last round
-// writes keys.
-__global__ void __launch_bounds__(kBigThreads) k_merge_round(const BatchDev b, int r) {
-  __shared__ uint64_t sm[kBigPadded];
   __shared__ uint32_t s_split[4];
-  constexpr int PER = kBig / kBigThreads;  // outputs per thread
-  // a round is needed only while some segment holds more than 2^r chunks (the launches
-  // cover the bound for the largest subset; most rounds of a wave find nothing to do)
-  if ((1u << r) >= b.big_count[1]) return;
+  __shared__ unsigned s_item;
+  __shared__ int s_ok;
   const unsigned count = *b.chunk_count;
-  const uint32_t w = (uint32_t)kBig << r;
-  for (unsigned wi = blockIdx.x; wi < count; wi += gridDim.x) {
-    const uint2 ch = b.chunks[wi];
-    const int64_t t = b.big_list[ch.x];
+  if (count == 0) return;
+  const unsigned items = count * (1u + (unsigned)rounds_of(b.big_count[1]));
+  for (;;) {
+    __syncthreads();  // the previous item is done with shared memory
+    if (threadIdx.x == 0) s_item = atomicAdd(b.big_count, 1u);
+    __syncthreads();
+    const unsigned item = s_item;
+    if (item >= items) return;
+    const unsigned q = item / count, ci = item - q * count;
+    const uint2 ch = b.chunks[ci];
+    const int64_t t = ch.x;
     uint32_t s, e;
     segment_of(b, t, s, e);
-    const uint32_t n = e - s;
-    if (n <= w) continue;  // this segment needs no merge at this width
-    // round r of a segment merged in R rounds reads keys_alt when R - r is odd (see the
-    // chunk sort), so its last round writes keys
-    const bool from_alt = ((rounds_for(n) - r) & 1) != 0;
-    const uint64_t* src = (from_alt ? b.keys_alt : b.keys) + s;
-    uint64_t* dst = (from_alt ? b.keys : b.keys_alt) + s;
-    const uint32_t o0 = ch.y * kBig;
-    if (o0 >= n) continue;
-    const uint32_t o1 = o0 + kBig < n ? o0 + kBig : n;
-    const uint32_t p0 = (o0 / (2 * w)) * (2 * w);
-    const uint32_t na = (p0 + w < n ? p0 + w : n) - p0;
-    const uint32_t nb = (p0 + 2 * w < n ? p0 + 2 * w : n) - (p0 + na);
-    const uint64_t* A = src + p0;
-    const uint64_t* B = A + na;
-    // warp 0 finds the split at the block's first output, warp 1 at its end
-    if (threadIdx.x < 64) {
-      const uint32_t dd = (threadIdx.x < 32 ? o0 : o1) - p0;
-      const uint32_t a = merge_path_warp(A, na, B, nb, dd);
-      if ((threadIdx.x & 31) == 0) {
-        s_split[threadIdx.x >> 5] = a;
-        s_split[2 + (threadIdx.x >> 5)] = dd - a;
+    const uint32_t n = e - s, o0 = (ci - ch.y) * kBig;
+    const unsigned R = (unsigned)rounds_for(n);
+    if (q > R) continue;  // this segment needs no merge at this width
+    if (q == 0) {
+      const uint32_t c0 = s + o0, c1 = c0 + kBig < e ? c0 + kBig : e;
+      uint64_t* out = ((R & 1u) ? b.keys_alt : b.keys) + c0;
+      sort_chunk<kBigThreads>(b.keys + c0, out, (int)(c1 - c0), sa, sb);
+    } else {
+      if (threadIdx.x == 0) {
+        const volatile uint32_t* done = b.seg_done + t;
+        const uint32_t need = q * long_chunks(n);
+        int polls = 0;
+        while (*done < need && polls < kSortPolls) {
+          __nanosleep(256);
+          ++polls;
+        }
+        s_ok = *done >= need;
+        if (!s_ok) atomicOr(b.status, ST_TIMEOUT);
+        __threadfence();
+      }
+      __syncthreads();
+      if (!s_ok) return;
+      // the input of round r = q - 1 lies in keys_alt when R - r is odd
+      const bool from_alt = ((R - (q - 1u)) & 1u) != 0u;
+      merge_item((from_alt ? b.keys_alt : b.keys) + s, (from_alt ? b.keys : b.keys_alt) + s, n,
+                 (uint32_t)kBig << (q - 1u), o0, sa, s_split);
+    }
+    if (q < R) {
+      __syncthreads();  // the item's keys are written
+      if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(b.seg_done + t, 1u);
       }
     }
-    __syncthreads();
-    const uint32_t a0 = s_split[0], a1 = s_split[1], b0 = s_split[2], b1 = s_split[3];
-    const int la = (int)(a1 - a0), lb = (int)(b1 - b0);
-    for (int i = threadIdx.x; i < la; i += kBigThreads) sm[pad(i)] = A[a0 + i];
-    for (int i = threadIdx.x; i < lb; i += kBigThreads) sm[pad(la + i)] = B[b0 + i];
-    __syncthreads();
-    // each thread merges PER consecutive outputs of sm[0,la) and sm[la,la+lb)
-    const int d = threadIdx.x * PER;
-    if (d < la + lb) {
-      int ia = merge_path_smem(sm, 0, la, la, lb, d);
-      int ib = d - ia;
-      const int dend = d + PER < la + lb ? d + PER : la + lb;
-      uint64_t va = ia < la ? sm[pad(ia)] : ~0ull;  // run heads (~0 past the end)
-      uint64_t vb = ib < lb ? sm[pad(la + ib)] : ~0ull;
-      for (int o = d; o < dend; ++o) {
-        const bool takeA = va < vb;
-        dst[o0 + o] = takeA ? va : vb;
-        ia += takeA ? 1 : 0;
-        ib += takeA ? 0 : 1;
-        const bool more = takeA ? ia < la : ib < lb;
-        const uint64_t nv = more ? sm[takeA ? pad(ia) : pad(la + ib)] : ~0ull;
-        va = takeA ? nv : va;
-        vb = takeA ? vb : nv;
-      }
-    }
-    __syncthreads();
   }
 }
 
-// The items the forward handed back (b.retry): full segment ranges, sel = 0, and their
-// segments registered as chunk work items for the long-segment sort.
-__global__ void __launch_bounds__(128) k_retry_prep(const BatchDev b) {
-  const unsigned n = *b.retry_count;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t t = b.retry[i];
-    uint32_t s, e;
-    segment_of(b, t, s, e);
-    b.ranges[t] = make_uint2(s, e);
-    // after a prefix the second forward resumes at the prefix's end (the whole sort puts
-    // the prefix's keys first, in its order); without one it starts at the beginning
-    const uint32_t sv = b.sel[t];
-    b.sel[t] = sv != kSelNone && sv != 0u ? (kSelResume | sv) : 0u;
-    const unsigned nch = (e - s + kBig - 1) / kBig;
-    const unsigned bi = atomicAdd(b.big_count, 1u);
-    const unsigned c0 = atomicAdd(b.chunk_count, nch);
-    atomicMax(b.big_count + 1, nch);
-    b.big_list[bi] = t;
-    for (unsigned c = 0; c < nch; ++c) b.chunks[c0 + c] = make_uint2(bi, c);
-  }
-}
-
-// Chunk sort and merge rounds of the segments registered in big_list / chunks.
-static void launch_long_sort(const BatchDev& b, int max_rounds, cudaStream_t s) {
-  const unsigned grid = (unsigned)device_sm_count() * 4;
+// Sort and merges of the segments registered in chunks (register_long).
+void launch_long_sort(const BatchDev& b, cudaStream_t s) {
   // 72 KB of dynamic shared memory: opted in once per device (a refused opt-in shows as
-  // the launch's error, which the callers check).  Its grid-stride loop runs one wave of
-  // resident CTAs (3 per SM at 72 KB), so that no CTA starts after the others have ended
+  // the launch's error, which the callers check).  One wave of resident CTAs (3 per SM at
+  // 72 KB), so that no CTA starts after the others have ended
   constexpr int kChunkSmem = 2 * kBigPadded * (int)sizeof(uint64_t);
-  (void)opt_in_smem((const void*)k_chunk_sort, kChunkSmem, 0);
-  const unsigned cgrid = (unsigned)device_sm_count() *
-                         (unsigned)resident_ctas((const void*)k_chunk_sort, kBigThreads,
-                                                 kChunkSmem, 0);
-  k_chunk_sort<<<cgrid, kBigThreads, kChunkSmem, s>>>(b);
-  for (int r = 0; r < max_rounds; ++r) k_merge_round<<<grid, kBigThreads, 0, s>>>(b, r);
-  count_launch(1 + max_rounds);
+  (void)opt_in_smem((const void*)k_long_sort, kChunkSmem, 0);
+  const unsigned grid = (unsigned)device_sm_count() *
+                        (unsigned)resident_ctas((const void*)k_long_sort, kBigThreads,
+                                                kChunkSmem, 0);
+  k_long_sort<<<grid, kBigThreads, kChunkSmem, s>>>(b);
+  count_launch();
 }
 
-void launch_seg_sort(const BatchDev& b, int max_rounds, cudaStream_t s) {
+void launch_seg_sort(const BatchDev& b, cudaStream_t s) {
   if (b.n_tiles == 0) return;
   const int64_t items = b.order ? b.item_n : b.n_tiles;
   k_seg_sort_small<<<(unsigned)items, kSortThreads, 0, s>>>(b);
   count_launch();
   // with selected prefixes no segment is left to the long-segment sort before the forward
-  if (!b.sel) launch_long_sort(b, max_rounds, s);
+  if (!b.sel) launch_long_sort(b, s);
 }
 
-void launch_sort_retries(const BatchDev& b, int max_rounds, cudaStream_t s) {
-  if (!b.sel || b.n_tiles == 0) return;
-  cudaMemsetAsync(b.big_count, 0, 2 * sizeof(unsigned), s);
-  cudaMemsetAsync(b.chunk_count, 0, sizeof(unsigned), s);
-  k_retry_prep<<<(unsigned)device_sm_count(), 128, 0, s>>>(b);
-  count_launch();
-  launch_long_sort(b, max_rounds, s);
-}
-
-// Merge rounds that cover any segment of a batch whose largest subset has max_n Gaussians
-// (a tile's segment holds at most one key per Gaussian of its subset).
-int merge_rounds_bound(int64_t max_n) {
-  const int64_t nch = (max_n + kBig - 1) / kBig;
-  int r = 0;
-  while ((int64_t(1) << r) < nch) ++r;
-  return r;
+void launch_sort_retries(const BatchDev& b, cudaStream_t s) {
+  if (b.sel && b.n_tiles != 0) launch_long_sort(b, s);
 }
 
 }  // namespace splx

@@ -102,9 +102,10 @@ struct BatchDev {
   uint32_t* tile_start;         // [n_tiles+1] exclusive scan of tile_cnt (last = total)
   uint64_t* keys;               // [capacity] depth bits << 32 | Gaussian index, by tile
   uint64_t* keys_alt;           // [capacity] scratch for the long-segment sort
-  uint32_t* big_list;           // [n_tiles] tiles whose segment exceeds one sort chunk
-  unsigned* big_count;          // [2]: tiles in big_list, most chunks of one of them
-  uint2* chunks;                // [n_tiles + capacity/2048 + 1] (big_list index, chunk)
+  uint32_t* seg_done;           // [n_tiles] items of a long segment's sort that are done
+  unsigned* big_count;          // [2]: items taken by the long-segment sort, most chunks of
+                                // one segment
+  uint2* chunks;                // [n_tiles + capacity/2048 + 1] (tile, its first entry here)
   unsigned* chunk_count;        // [1]
   uint2* ranges;                // [n_tiles] sorted [start, end)
   int64_t goff[kMaxK + 1];      // subset k = global indices [goff[k], goff[k+1])
@@ -218,20 +219,30 @@ constexpr uint32_t kSelNone = 0xFFFFFFFFu;
 constexpr uint32_t kSelResume = 0x80000000u;
 // largest selected prefix: keys sorted in shared memory by one sort CTA
 constexpr int kSelCap = 2048;
+// keys of one chunk of the long-segment sort
+constexpr uint32_t kSortChunk = 4096;
 
 // ---- launch wrappers (defined in the .cu files) ------------------------------------
 void launch_project(const BatchDev& b, cudaStream_t s);
 void launch_fill(const BatchDev& b, cudaStream_t s);
-// Sorts every tile segment; max_rounds = merge_rounds_bound(largest subset size).
-void launch_seg_sort(const BatchDev& b, int max_rounds, cudaStream_t s);
-int merge_rounds_bound(int64_t max_n);
+// Sorts every tile segment.
+void launch_seg_sort(const BatchDev& b, cudaStream_t s);
+// One launch's sort counters (zero before its sort): big_count[2], chunk_count, retry_count.
+constexpr int kSortCounts = 4;
+inline void set_sort_counts(BatchDev& b, unsigned* p) {
+  b.big_count = p;
+  b.chunk_count = p + 2;
+  b.retry_count = p + 3;
+}
 inline int64_t chunk_list_capacity(int64_t n_tiles, int64_t capacity) {
   return n_tiles + capacity / 2048 + 1;
 }
 void launch_raster_fwd(const BatchDev& b, cudaStream_t s);
-// The full sort of the segments the forward handed back (b.retry) and their second
+// Whole sort of the segments registered in b.chunks (register_long).
+void launch_long_sort(const BatchDev& b, cudaStream_t s);
+// The full sort of the segments the forward handed back (hand_back) and their second
 // forward: no-ops when the retry list is empty (selected-prefix sort, b.sel != nullptr).
-void launch_sort_retries(const BatchDev& b, int max_rounds, cudaStream_t s);
+void launch_sort_retries(const BatchDev& b, cudaStream_t s);
 void launch_raster_fwd_retry(const BatchDev& b, cudaStream_t s);
 void launch_composite(const BatchDev& b, int64_t total_pixels, cudaStream_t s);
 void launch_composite_bwd(const BatchDev& b, int64_t total_pixels, cudaStream_t s);
@@ -299,6 +310,44 @@ __device__ __forceinline__ int view_of(const int64_t* base, int V, int64_t x) {
     if (base[mid] <= x) lo = mid; else hi = mid - 1;
   }
   return lo;
+}
+
+__device__ __forceinline__ void segment_of(const BatchDev& b, int64_t t, uint32_t& s, uint32_t& e) {
+  const uint64_t cap = (uint64_t)b.capacity;
+  uint64_t s64 = b.tile_start[t], e64 = b.tile_start[t + 1];
+  if (s64 > cap) s64 = cap;
+  if (e64 > cap) e64 = cap;
+  if (e64 < s64) e64 = s64;
+  s = (uint32_t)s64;
+  e = (uint32_t)e64;
+}
+
+__device__ __forceinline__ uint32_t long_chunks(uint32_t n) {
+  return (n + kSortChunk - 1) / kSortChunk;
+}
+
+// Registers tile t's segment of n keys with the long-segment sort and returns its first
+// entry of b.chunks; the caller writes its long_chunks(n) entries (t, first).
+__device__ __forceinline__ uint32_t register_long(const BatchDev& b, int64_t t, uint32_t n) {
+  const uint32_t nch = long_chunks(n);
+  b.seg_done[t] = 0u;
+  atomicMax(b.big_count + 1, nch);
+  return atomicAdd(b.chunk_count, nch);
+}
+
+// Hands work item t, whose forward found its selected prefix of sv keys (kSelNone: none)
+// too short, to the second forward (b.retry): full segment range, and its segment
+// registered with the long-segment sort.  After a prefix the second forward resumes at the
+// prefix's end (the whole sort puts the prefix's keys first, in its order); without one it
+// starts at the beginning.  One thread.
+__device__ __forceinline__ void hand_back(const BatchDev& b, uint32_t t, uint32_t sv) {
+  b.retry[atomicAdd(b.retry_count, 1u)] = t;
+  uint32_t s, e;
+  segment_of(b, t, s, e);
+  b.ranges[t] = make_uint2(s, e);
+  b.sel[t] = sv != kSelNone && sv != 0u ? (kSelResume | sv) : 0u;
+  const uint32_t nch = long_chunks(e - s), first = register_long(b, t, e - s);
+  for (uint32_t c = 0; c < nch; ++c) b.chunks[first + c] = make_uint2(t, first);
 }
 
 // Work item of a launch: every (view, subset, tile), or in a saturation-skipping wave the

@@ -119,10 +119,9 @@ extern "C" int splx_render_partial_noalloc(const splx_gaussians* g, const splx_c
   uint32_t* counts = cv.take<uint32_t>((size_t)(N > 0 ? N : 1));
   uint32_t* tile_cnt = cv.take<uint32_t>((size_t)n_tiles);
   uint32_t* tile_start = cv.take<uint32_t>((size_t)n_tiles + 1);
-  uint32_t* big_list = cv.take<uint32_t>((size_t)n_tiles);
-  unsigned* big_count = cv.take<unsigned>(2);  // count, most chunks of one segment
+  uint32_t* seg_done = cv.take<uint32_t>((size_t)n_tiles);
+  unsigned* sort_counts = cv.take<unsigned>(kSortCounts);
   uint2* chunks = cv.take<uint2>((size_t)chunk_list_capacity(n_tiles, kNoAllocMaxPairs));
-  unsigned* chunk_count = cv.take<unsigned>(1);
   void* scan_temp = cv.take<unsigned char>(scan_u32_temp_bytes(n_tiles));
   uint64_t* keys = cv.take<uint64_t>(kNoAllocMaxPairs);
   uint64_t* keys_alt = cv.take<uint64_t>(kNoAllocMaxPairs);
@@ -159,8 +158,8 @@ extern "C" int splx_render_partial_noalloc(const splx_gaussians* g, const splx_c
   for (int k = 0; k < 3; ++k) b.bg[k] = o->bg[k];
   b.subsets = sub_d; b.views = view_d; b.imgs = img_d;
   b.rec = rec; b.counts = counts; b.tile_cnt = tile_cnt; b.tile_start = tile_start;
-  b.keys = keys; b.keys_alt = keys_alt; b.big_list = big_list; b.big_count = big_count;
-  b.chunks = chunks; b.chunk_count = chunk_count;
+  b.keys = keys; b.keys_alt = keys_alt; b.chunks = chunks;
+  b.seg_done = seg_done; set_sort_counts(b, sort_counts);
   b.ranges = ranges; b.grad2d = nullptr; b.status = status; b.counters = nullptr;
   b.goff[0] = 0; b.goff[1] = N;
   b.tile_base[0] = 0; b.tile_base[1] = n_tiles;
@@ -171,14 +170,14 @@ extern "C" int splx_render_partial_noalloc(const splx_gaussians* g, const splx_c
   if (e == cudaSuccess) e = cudaMemcpyAsync(view_d, &vd, sizeof(vd), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(img_d, &im, sizeof(im), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(tile_cnt, 0, sizeof(uint32_t) * (size_t)n_tiles, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(big_count, 0, 2 * sizeof(unsigned), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(chunk_count, 0, sizeof(unsigned), s);
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(sort_counts, 0, kSortCounts * sizeof(unsigned), s);
   if (e != cudaSuccess) return SPLX_ERR_CUDA;
 
   launch_project(b, s);
   scan_u32(tile_cnt, tile_start, n_tiles, scan_temp, s);
   launch_fill(b, s);
-  launch_seg_sort(b, merge_rounds_bound(N), s);
+  launch_seg_sort(b, s);
   launch_raster_fwd(b, s);
   if (cudaGetLastError() != cudaSuccess) return SPLX_ERR_CUDA;
 
@@ -190,6 +189,7 @@ extern "C" int splx_render_partial_noalloc(const splx_gaussians* g, const splx_c
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return SPLX_ERR_CUDA;
   if ((st & ST_CAPACITY) || total > (uint64_t)kNoAllocMaxPairs) return SPLX_ERR_CAPACITY;
+  if (st & ST_TIMEOUT) return SPLX_ERR_TIMEOUT;
   if (st & ST_BOUNDS) return SPLX_ERR_STATE;
   return SPLX_OK;
 }

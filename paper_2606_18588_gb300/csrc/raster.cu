@@ -291,7 +291,7 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
     const uint32_t sv = b.sel[id];
     if (sv == kSelNone) {
       if (threadIdx.x == 0) {
-        b.retry[atomicAdd(b.retry_count, 1u)] = (uint32_t)id;
+        hand_back(b, (uint32_t)id, kSelNone);
         if (kCount && b.counters) atomicAdd(b.counters + 9, 1ull);
       }
       return;
@@ -530,7 +530,7 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
       if (threadIdx.x == 0 && kCount && b.counters) atomicAdd(b.counters + 8, 1ull);
       if (more) {
         if (threadIdx.x == 0) {
-          b.retry[atomicAdd(b.retry_count, 1u)] = pid;
+          hand_back(b, pid, b.sel[pid]);
           if (kCount && b.counters) atomicAdd(b.counters + 9, 1ull);
         }
         // the planes hold the state at the prefix's end for the second forward: a pixel
