@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "spec.cuh"
 
 namespace splx {
 thread_local int64_t* g_launch_counter = nullptr;
@@ -199,6 +200,8 @@ ViewDev make_view(const splx_camera& c, int tile) {
     v.eye[k] = (float)(-((double)c.R[k] * c.t[0] + (double)c.R[3 + k] * c.t[1] +
                          (double)c.R[6 + k] * c.t[2]));
   v.W = c.width; v.H = c.height;
+  v.limx = spec_limit(c.width, c.fx);
+  v.limy = spec_limit(c.height, c.fy);
   v.tiles_x = (c.width + tile - 1) / tile;
   v.tiles_y = (c.height + tile - 1) / tile;
   return v;

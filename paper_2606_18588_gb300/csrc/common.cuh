@@ -59,6 +59,7 @@ struct ViewDev {
   float R[9], t[3];
   float fx, fy, cx, cy, near_plane;
   float eye[3];  // camera centre in world space
+  float limx, limy;  // the specification's clamps of x/z and y/z (spec_limit)
   int32_t W, H, tiles_x, tiles_y;
 };
 

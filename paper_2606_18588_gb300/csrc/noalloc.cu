@@ -28,6 +28,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "spec.cuh"
 
 namespace splx {
 
@@ -141,6 +142,8 @@ extern "C" int splx_render_partial_noalloc(const splx_gaussians* g, const splx_c
     vd.eye[k] = (float)(-((double)c->R[k] * c->t[0] + (double)c->R[3 + k] * c->t[1] +
                           (double)c->R[6 + k] * c->t[2]));
   vd.W = c->width; vd.H = c->height; vd.tiles_x = tiles_x; vd.tiles_y = tiles_y;
+  vd.limx = spec_limit(c->width, c->fx);
+  vd.limy = spec_limit(c->height, c->fy);
   ImgDev im;
   im.rgb = out->rgb; im.T = out->T; im.D = out->depth; im.last = out->last; im.gCT = nullptr;
 

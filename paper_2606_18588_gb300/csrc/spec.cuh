@@ -39,6 +39,14 @@ __device__ __forceinline__ float exp_spec(float x) {
   return fm(p, scale);
 }
 
+// The clamp of |x/z| (or |y/z|): 1.3 (extent / 2) / focal, each operation rounded to FP32 (on
+// the host; products and a quotient leave nothing to contract).
+inline float spec_limit(int extent, float focal) {
+  const float half = 0.5f * (float)extent;
+  const float wide = 1.3f * half;
+  return wide / focal;
+}
+
 struct SpecOut {
   bool visible;
   int x0, x1, y0, y1;
@@ -87,7 +95,6 @@ __device__ __forceinline__ SpecG spec_gaussian(const float ls[3], const float q[
   return G;
 }
 
-// Per-view part; cam: R[9], t[3], fx, fy, cx, cy, W, H, near.
 // Knuth's TwoSum: s = fl(a + b) and its exact rounding error e (s + e = a + b).
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = fa(a, b);
@@ -123,9 +130,12 @@ __device__ __forceinline__ void spec_center(float tx, float ty, float tz, float 
   v = fa(fd(fm(fy, ty), tz), cy);
 }
 
+// Per-view part; cam: R[9], t[3], fx, fy, cx, cy, W, H, near, and the view's clamps of x/z and
+// y/z (spec_limit: the same for every Gaussian).
 __device__ __forceinline__ SpecOut bin_spec(const float m[3], const SpecG& G, const float* R,
                                             const float* tc, float fx, float fy, float cx,
-                                            float cy, int W, int H, float near_plane) {
+                                            float cy, int W, int H, float near_plane, float limx,
+                                            float limy) {
   SpecOut o;
   o.visible = false;
   o.x0 = 0; o.x1 = -1; o.y0 = 0; o.y1 = -1;
@@ -162,8 +172,6 @@ __device__ __forceinline__ SpecOut bin_spec(const float m[3], const SpecG& G, co
     for (int j = 0; j < 3; ++j)
       V[3 * i + j] = fa(fa(fm(R[3 * i + 0], M[j]), fm(R[3 * i + 1], M[3 + j])),
                         fm(R[3 * i + 2], M[6 + j]));
-  const float limx = fd(fm(1.3f, fm(0.5f, (float)W)), fx);
-  const float limy = fd(fm(1.3f, fm(0.5f, (float)H)), fy);
   const float rx = fminf(limx, fmaxf(-limx, fd(tx, tz)));
   const float ry = fminf(limy, fmaxf(-limy, fd(ty, tz)));
   const float j00 = fd(fx, tz);
