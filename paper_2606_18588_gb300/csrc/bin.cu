@@ -269,13 +269,17 @@ constexpr int kFillThreads = 256;
 constexpr int kFillFields = 18;  // per lane: tile test (8), rect x, rect y, tile base, width,
                                  // 1/width, tiles per row, pass bits, key (2), tiles
 
-__global__ void __launch_bounds__(kFillThreads, 8) k_fill(const BatchDev b) {
+__global__ void __launch_bounds__(kFillThreads, 8) k_fill(const BatchDev b, int per_warp) {
   __shared__ float s_walk[kFillThreads / 32][kFillFields][32];
   __shared__ int s_own[kFillThreads / 32][32];
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned lanes = __ballot_sync(0xffffffffu, idx < (int64_t)b.V * b.N);
-  if (idx >= (int64_t)b.V * b.N) return;
-  const uint32_t tiles = b.counts[idx];
+  const int warp = (int)(threadIdx.x >> 5);
+  const unsigned lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+  const int64_t first = ((int64_t)blockIdx.x * (kFillThreads / 32) + warp) * per_warp;
+  const int64_t idx = first + lane;
+  if (first >= (int64_t)b.V * b.N) return;
+  // lanes without a Gaussian of their own help to walk the others' tiles
+  const bool own = (int)lane < per_warp && idx < (int64_t)b.V * b.N;
+  const uint32_t tiles = own ? b.counts[idx] : 0u;
   const int v = (int)(idx / b.N);
   const int64_t g = idx - (int64_t)v * b.N;
   int tw = 1, tiles_x = 0, rx0 = 0, rx1 = 0, ry0 = 0, ry1 = 0;
@@ -312,8 +316,6 @@ __global__ void __launch_bounds__(kFillThreads, 8) k_fill(const BatchDev b) {
     tbase = b.tile_base[v] + (int64_t)k * cam.tiles_x * cam.tiles_y + (int64_t)ty0 * cam.tiles_x + tx0;
     key = ((uint64_t)__float_as_uint(rb.z) << 32) | (uint64_t)(uint32_t)g;
   }
-  const int warp = (int)(threadIdx.x >> 5);
-  const unsigned lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
   bool overflow = false;
   // one (tile, key) candidate per lane: aggregate per tile, take slots, write the keys
   auto place = [&](unsigned t, uint64_t k) {
@@ -334,11 +336,11 @@ __global__ void __launch_bounds__(kFillThreads, 8) k_fill(const BatchDev b) {
         }
       }
     }
-    const unsigned peers = __match_any_sync(lanes, t);
+    const unsigned peers = __match_any_sync(kFullWarp, t);
     const int leader = __ffs(peers) - 1;
     unsigned old = 0;
     if (t != 0xFFFFFFFFu && (int)lane == leader) old = atomicSub(&b.tile_cnt[t], (unsigned)__popc(peers));
-    old = __shfl_sync(lanes, old, leader);
+    old = __shfl_sync(kFullWarp, old, leader);
     if (t != 0xFFFFFFFFu) {
       const uint64_t pos = (uint64_t)b.tile_start[t] + (old - 1u - (unsigned)__popc(peers & lt));
       if (pos < (uint64_t)b.capacity) b.keys[pos] = k;
@@ -364,8 +366,8 @@ __global__ void __launch_bounds__(kFillThreads, 8) k_fill(const BatchDev b) {
     // a rectangle of at most 32 tiles walks only the tiles its pass bits name (the test is
     // already taken); a larger one walks them all and takes the test
     const int cand = tiles <= 32u ? __popc(hits) : (int)tiles;
-    const WarpWalk walk = warp_walk_begin(lanes, cand);
-    for (int base = 0; base < walk.total; base += walk.nact) {
+    const WarpWalk walk = warp_walk_begin(cand);
+    for (int base = 0; base < walk.total; base += 32) {
       int j;
       const int o = warp_walk_owner(walk, base, s_own[warp], j);
       unsigned t = 0xFFFFFFFFu;
@@ -402,9 +404,10 @@ __global__ void __launch_bounds__(kFillThreads, 8) k_fill(const BatchDev b) {
 
 void launch_fill(const BatchDev& b, cudaStream_t s) {
   const int64_t n = (int64_t)b.V * b.N;
-  const int64_t blocks = (n + kFillThreads - 1) / kFillThreads;
-  if (blocks == 0) return;
-  k_fill<<<(unsigned)blocks, kFillThreads, 0, s>>>(b);
+  if (n == 0) return;
+  const int per_warp = walk_per_warp(n, device_sm_count() * 64);
+  const int64_t per_block = (int64_t)(kFillThreads / 32) * per_warp;
+  k_fill<<<(unsigned)((n + per_block - 1) / per_block), kFillThreads, 0, s>>>(b, per_warp);
   count_launch();
 }
 

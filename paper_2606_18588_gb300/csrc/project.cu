@@ -65,13 +65,13 @@ __device__ __forceinline__ int sh_slot(int l, int c) { return l * kShChunks + (c
 
 // Degree-3 batches of at least this many views stage the coefficients (see the kernel).
 // Projection of 2M Gaussians in 4 views: 0.64 ms staged, 0.63 direct; in 8 views 1.18 both;
-// 10M in 16 views 8.6 against 9.9 ms; 20M in 4 views that see a seventh of them each, 1.51
+// 10M in 16 views 8.6 against 9.9 ms; 20M in 4 views that see a part of them each, 1.51
 // against 1.32 ms.
 constexpr int kStageViews = 8;
 
 constexpr int kProjThreads = 128;
 
-// What bounds it (10M Gaussians, 16 views, 8.6 ms): issue.  The specification up to the
+// What bounds it (10M Gaussians, 16 views, 8.0 ms; 10.4 before): issue.  The specification up to the
 // culling takes 1.5 ms of it, a visible Gaussian's centre, conic and record 2, its colour
 // 2.5 and the tile walk 2.2.  The colour's 12 float4 loads lie 192 bytes apart from lane to
 // lane, 32 cache lines each, which kept the load unit at 60 %: with many views (kStage) a
@@ -79,17 +79,22 @@ constexpr int kProjThreads = 128;
 // shared memory and reads them there without bank conflicts; with few views
 // the copy costs as much as it saves, and the shared memory is left to L1.  The tile walk
 // passes a task's inputs by shuffles (not shared memory), the tile sides are shifts, and the
-// clamps of x/z come with the view.  6 CTAs of 128 threads at 80 registers (staged), 8 at 64.
+// clamps of x/z come with the view.  Small launches give a warp fewer Gaussians of its own
+// (walk_per_warp).  6 CTAs of 128 threads at 80 registers (staged), 8 at 64.
 template <int DEG, bool kStage>
-__global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const BatchDev b) {
+__global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const BatchDev b, int per_warp) {
   static_assert(!kStage || DEG == 3, "the staging layout is that of degree 3");
   __shared__ float4 s_sh[kStage ? kProjThreads * kShChunks : 1];
   // the warp's tile walk: task owners, and each lane's outcome
   __shared__ int s_own[kProjThreads / 32][32];
   __shared__ uint32_t s_hits[kProjThreads / 32][32], s_any[kProjThreads / 32][32];
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned lanes = __ballot_sync(0xffffffffu, g < b.N);  // lanes in the warp collectives
-  if (g >= b.N) return;
+  const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+  const int64_t g0 = ((int64_t)blockIdx.x * (kProjThreads / 32) + warp) * per_warp;
+  if (g0 >= b.N) return;
+  // lanes without a Gaussian of their own help to walk the others' tiles (they repeat the
+  // last one's arithmetic, invisible, and write nothing)
+  const bool own = lane < per_warp && g0 + lane < b.N;
+  const int64_t g = own ? g0 + lane : min(g0 + per_warp, b.N) - 1;
   const int k = subset_of(b, g);
   const SubsetDev S = b.subsets[k];
   const int64_t i = g - S.goff;
@@ -112,7 +117,6 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
   const bool sh_vec = (NC * 3) % 4 == 0 && (reinterpret_cast<uintptr_t>(shp) & 15) == 0;
 
   const int tsh = __ffs(b.tile) - 1;  // the tile side is a power of two
-  const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
   // Staging needs one contiguous, 16-byte aligned run of coefficients: a warp whose lanes
   // belong to one subset
   bool stage = false;
@@ -120,8 +124,8 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
   float4* sh_mine = s_sh + (kStage ? warp * 32 * kShChunks : 0);
   unsigned staged = 0u;  // lanes whose coefficients are in shared memory
   if (kStage) {
-    stage = __all_sync(lanes, sh_vec && k == __shfl_sync(lanes, k, 0));
-    sh_warp = reinterpret_cast<const float4*>(S.sh + (i - lane) * (NC * 3));
+    stage = __all_sync(kFullWarp, sh_vec && k == __shfl_sync(kFullWarp, k, 0));
+    sh_warp = reinterpret_cast<const float4*>(S.sh + (g0 - S.goff) * (NC * 3));
   }
 
   const SpecG G = spec_gaussian(ls, q);  // view-independent part of the specification
@@ -135,30 +139,30 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
     const float lo[3] = {fs(m[0], r3), fs(m[1], r3), fs(m[2], r3)};
     const float hi[3] = {fa(m[0], r3), fa(m[1], r3), fa(m[2], r3)};
     unsigned long long mask = 0ull;
-    const int own = b.cell_self >= 0 ? b.cell_self : k;
+    const int own_cell = b.cell_self >= 0 ? b.cell_self : k;
     for (int c = 0; c < b.ncells; ++c) {
-      if (c == own) continue;
+      if (c == own_cell) continue;
       const float* cb = b.cells + 6 * c;
       if (lo[0] <= cb[3] && hi[0] >= cb[0] && lo[1] <= cb[4] && hi[1] >= cb[1] &&
           lo[2] <= cb[5] && hi[2] >= cb[2])
         mask |= 1ull << c;
     }
-    b.cross[g] = mask;
+    if (own) b.cross[g] = mask;
   }
   for (int v = 0; v < b.V; ++v) {
     const ViewDev& cam = b.views[v];
     bool fresh = false;
-    const SpecOut so = bin_spec(m, G, cam.R, cam.t, cam.fx, cam.fy, cam.cx, cam.cy, cam.W,
+    SpecOut so = bin_spec(m, G, cam.R, cam.t, cam.fx, cam.fy, cam.cx, cam.cy, cam.W,
                                 cam.H, cam.near_plane, cam.limx, cam.limy);
+    so.visible = so.visible && own;
     if (kStage && stage) {
       // the coefficients of the lanes that are visible for the first time, 16 bytes a lane
       // and step in memory order; they arrive while the conic is computed
-      const unsigned need = __ballot_sync(lanes, so.visible) & ~staged;
+      const unsigned need = __ballot_sync(kFullWarp, so.visible) & ~staged;
       if (need) {
-        const int nact = __popc(lanes);
 #pragma unroll 1
         for (int it = 0; it < kShChunks; ++it) {
-          const int j = it * nact + lane, o = j / kShChunks;
+          const int j = it * 32 + lane, o = j / kShChunks;
           if ((need >> o) & 1u) cp_async16(sh_mine + sh_slot(o, j - o * kShChunks), sh_warp + j);
         }
         cp_async_commit();
@@ -184,7 +188,7 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
     }
     if (kStage && fresh) {
       cp_async_wait<0>();
-      __syncwarp(lanes);
+      __syncwarp();
     }
     if (so.visible) {
       float dx = m[0] - cam.eye[0], dy = m[1] - cam.eye[1], dz = m[2] - cam.eye[2];
@@ -227,7 +231,7 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
       const int tx0 = so.x0 >> tsh, tx1 = so.x1 >> tsh, ty0 = so.y0 >> tsh, ty1 = so.y1 >> tsh;
       tiles = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
     }
-    b.counts[(int64_t)v * b.N + g] = tiles;
+    if (own) b.counts[(int64_t)v * b.N + g] = tiles;
     // count this Gaussian in every tile of its rectangle that passes the tile test (the
     // segment sizes of the binning); lanes that hit the same tile add together
     // (neighbouring Gaussians are neighbours in memory), so most tiles see one atomic
@@ -240,8 +244,7 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
     uint32_t hits = 0;  // bit j: the j-th tile of the rectangle passes the tile test
     bool any_pair = false;
     // head: every lane tests its own first H tiles, H = the warp's mean count rounded up
-    const int nact = __popc(lanes);
-    const int H = ((int)__reduce_add_sync(lanes, tiles) + nact - 1) / nact;
+    const int H = ((int)__reduce_add_sync(kFullWarp, tiles) + 31) / 32;
     int jx = 0, jy = 0;  // column / row of the j-th tile inside the rectangle
     for (int j = 0; j < H; ++j) {
       unsigned t = 0xFFFFFFFFu;
@@ -252,30 +255,30 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
         if (j < 32) hits |= 1u << j;
       }
       if (++jx == tw) { jx = 0; ++jy; }
-      const unsigned peers = __match_any_sync(lanes, t);
+      const unsigned peers = __match_any_sync(kFullWarp, t);
       if (t != 0xFFFFFFFFu && lane == __ffs(peers) - 1)
         atomicAdd(&b.tile_cnt[t], (unsigned)__popc(peers));
     }
     // tail: the tiles beyond H of the lanes that have more, spread evenly over the warp
     const int rest = (int)tiles > H ? (int)tiles - H : 0;
-    if (__any_sync(lanes, rest > 0)) {
+    if (__any_sync(kFullWarp, rest > 0)) {
       const uint32_t rx = (uint32_t)so.x0 | ((uint32_t)so.x1 << 16);
       const uint32_t ry = (uint32_t)so.y0 | ((uint32_t)so.y1 << 16);
       s_hits[warp][lane] = 0u;
       s_any[warp][lane] = 0u;
-      const WarpWalk walk = warp_walk_begin(lanes, rest);
-      for (int base = 0; base < walk.total; base += walk.nact) {
+      const WarpWalk walk = warp_walk_begin(rest);
+      for (int base = 0; base < walk.total; base += 32) {
         int jr;
         const int o = warp_walk_owner(walk, base, s_own[warp], jr);
         // the owner's tile test, from its registers
         const int src = o >= 0 ? o : lane;
         TileCull oc;
-        oc.u = __shfl_sync(lanes, tc.u, src); oc.v = __shfl_sync(lanes, tc.v, src);
-        oc.A = __shfl_sync(lanes, tc.A, src); oc.B = __shfl_sync(lanes, tc.B, src);
-        oc.C = __shfl_sync(lanes, tc.C, src); oc.qmax = __shfl_sync(lanes, tc.qmax, src);
-        oc.rBC = __shfl_sync(lanes, tc.rBC, src); oc.rBA = __shfl_sync(lanes, tc.rBA, src);
-        const uint32_t orx = __shfl_sync(lanes, rx, src), ory = __shfl_sync(lanes, ry, src);
-        const uint32_t ob = __shfl_sync(lanes, (uint32_t)tbase, src);
+        oc.u = __shfl_sync(kFullWarp, tc.u, src); oc.v = __shfl_sync(kFullWarp, tc.v, src);
+        oc.A = __shfl_sync(kFullWarp, tc.A, src); oc.B = __shfl_sync(kFullWarp, tc.B, src);
+        oc.C = __shfl_sync(kFullWarp, tc.C, src); oc.qmax = __shfl_sync(kFullWarp, tc.qmax, src);
+        oc.rBC = __shfl_sync(kFullWarp, tc.rBC, src); oc.rBA = __shfl_sync(kFullWarp, tc.rBA, src);
+        const uint32_t orx = __shfl_sync(kFullWarp, rx, src), ory = __shfl_sync(kFullWarp, ry, src);
+        const uint32_t ob = __shfl_sync(kFullWarp, (uint32_t)tbase, src);
         unsigned t = 0xFFFFFFFFu;
         if (o >= 0) {
           const int j = H + jr;
@@ -290,17 +293,17 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
             s_any[warp][o] = 1u;
           }
         }
-        const unsigned peers = __match_any_sync(lanes, t);
+        const unsigned peers = __match_any_sync(kFullWarp, t);
         if (t != 0xFFFFFFFFu && lane == __ffs(peers) - 1)
           atomicAdd(&b.tile_cnt[t], (unsigned)__popc(peers));
       }
-      __syncwarp(lanes);
+      __syncwarp();
       hits |= s_hits[warp][lane];
       any_pair = any_pair || s_any[warp][lane] != 0u;
     }
     // cross-boundary filtering: the depth range of the subset's kept Gaussians in this view
     if (b.zr) {
-      const unsigned peers = __match_any_sync(lanes, so.visible ? k : -1);
+      const unsigned peers = __match_any_sync(kFullWarp, so.visible ? k : -1);
       if (so.visible) {
         const uint32_t d = __float_as_uint(so.tz);
         const uint32_t dmin = __reduce_min_sync(peers, d), ndmax = __reduce_min_sync(peers, ~d);
@@ -314,7 +317,7 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
     // spatial visibility: grow the subset's bounding tile rectangle in this view by this
     // Gaussian's tile rectangle (lanes of one subset reduce first, one atomic each)
     if (b.omega) {
-      const unsigned peers = __match_any_sync(lanes, any_pair ? k : -1);
+      const unsigned peers = __match_any_sync(kFullWarp, any_pair ? k : -1);
       if (any_pair) {
         uint32_t e[4] = {(uint32_t)tx0, (uint32_t)ty0, ~(uint32_t)(so.x1 >> tsh),
                          ~(uint32_t)(so.y1 >> tsh)};
@@ -337,15 +340,17 @@ __global__ void __launch_bounds__(kProjThreads, kStage ? 6 : 8) k_project(const 
 void launch_project(const BatchDev& b, cudaStream_t s) {
   const BatchDev& P = b;
   const int threads = kProjThreads;
-  const int64_t blocks = (b.N + threads - 1) / threads;
-  if (blocks == 0) return;
+  if (b.N == 0) return;
+  const int per_warp = walk_per_warp(b.N, device_sm_count() * 32);
+  const int64_t per_block = (int64_t)(threads / 32) * per_warp;
+  const int64_t blocks = (b.N + per_block - 1) / per_block;
   switch (b.sh_degree) {
-    case 0: k_project<0, false><<<(unsigned)blocks, threads, 0, s>>>(P); break;
-    case 1: k_project<1, false><<<(unsigned)blocks, threads, 0, s>>>(P); break;
-    case 2: k_project<2, false><<<(unsigned)blocks, threads, 0, s>>>(P); break;
+    case 0: k_project<0, false><<<(unsigned)blocks, threads, 0, s>>>(P, per_warp); break;
+    case 1: k_project<1, false><<<(unsigned)blocks, threads, 0, s>>>(P, per_warp); break;
+    case 2: k_project<2, false><<<(unsigned)blocks, threads, 0, s>>>(P, per_warp); break;
     default:
-      if (b.V >= kStageViews) k_project<3, true><<<(unsigned)blocks, threads, 0, s>>>(P);
-      else k_project<3, false><<<(unsigned)blocks, threads, 0, s>>>(P);
+      if (b.V >= kStageViews) k_project<3, true><<<(unsigned)blocks, threads, 0, s>>>(P, per_warp);
+      else k_project<3, false><<<(unsigned)blocks, threads, 0, s>>>(P, per_warp);
       break;
   }
   count_launch();
