@@ -10,8 +10,8 @@
 // the filter removes keeps its slot with depth bits 0xFFFFFFFF, so it sorts last, and the
 // tile's range ends before it.
 //
-// Sorting: a segment of up to 2048 keys is sorted in shared memory by one CTA of 256
-// threads (8 keys per thread by a transposition network, then merge-path merges of runs).
+// Sorting: a segment of up to 256 keys is sorted in shared memory by one warp, one of up to
+// 2048 keys by one CTA of 256 threads (8 keys per thread by a transposition network, then merge-path merges of runs).
 // Longer segments are cut into 4096-key chunks, each sorted the same way by a CTA of 512
 // threads, and then merged pairwise in rounds (run width 4096, 8192, ...) with merge-path
 // partitioning, one CTA per 4096 outputs, ping-ponging between the key buffer and its
@@ -51,6 +51,10 @@ __device__ __forceinline__ void cas(uint64_t& a, uint64_t& b) {
 __device__ __forceinline__ int pad(int i) { return i + (i >> 3); }
 constexpr int kPadded = kChunk + kChunk / 8;
 constexpr int kBigPadded = kBig + kBig / 8;
+// a segment up to this long is sorted by one warp, in its share of a CTA's buffers
+constexpr int kWarpKeys = 32 * kItems;
+constexpr int kWarpPadded = kWarpKeys + kWarpKeys / 8;
+static_assert(kSortThreads / 32 * kWarpPadded <= kPadded, "the warps' shares fit");
 
 // Number of elements taken from A = s[pad(a0 + i)] among the first d of merge(A, B) with
 // B = s[pad(b0 + j)], in shared memory.
@@ -65,19 +69,23 @@ __device__ __forceinline__ int merge_path_smem(const uint64_t* s, int a0, int na
   return lo;
 }
 
-// Sorts in[0, n) into out[0, n) (n <= CH; out may be in) with TH threads: each thread sorts kItems keys in
-// registers (odd-even transposition network), then runs of 8, 16, ... are merged pairwise
-// through two shared buffers, every thread producing kItems outputs located by merge path.
-// The array is padded to a power of two P >= 8 with ~0 keys.  sa, sb: CH + CH/8 keys each.
+// Sorts in[0, n) into out[0, n) (n <= TH * kItems; out may be in) with TH threads, t = 0 ..
+// TH - 1: a CTA's, or with TH = 32 one warp.  Each thread sorts kItems keys in registers
+// (odd-even transposition network), then runs of 8, 16, ... are merged pairwise through two
+// shared buffers, every thread producing kItems outputs located by merge path.  The array
+// is padded to a power of two P >= 8 with ~0 keys.  sa, sb: 9/8 TH kItems keys each.
 template <int TH>
 __device__ __forceinline__ void sort_chunk(const uint64_t* in, uint64_t* out, int n, uint64_t* sa,
-                                           uint64_t* sb) {
+                                           uint64_t* sb, const int t) {
+  auto sync = [] {
+    if (TH == 32) __syncwarp();
+    else __syncthreads();
+  };
   int P = next_pow2(n);
   if (P < kItems) P = kItems;
-  for (int i = threadIdx.x; i < P; i += TH) sa[pad(i)] = i < n ? in[i] : ~0ull;
-  __syncthreads();
+  for (int i = t; i < P; i += TH) sa[pad(i)] = i < n ? in[i] : ~0ull;
+  sync();
   const int active = P / kItems;  // threads holding keys
-  const int t = threadIdx.x;
   if (t < active) {
     uint64_t v[kItems];
 #pragma unroll
@@ -89,7 +97,7 @@ __device__ __forceinline__ void sort_chunk(const uint64_t* in, uint64_t* out, in
 #pragma unroll
     for (int r = 0; r < kItems; ++r) sa[pad(t * kItems + r)] = v[r];
   }
-  __syncthreads();
+  sync();
   uint64_t* src = sa;
   uint64_t* dst = sb;
   for (int w = kItems; w < P; w <<= 1) {
@@ -118,12 +126,12 @@ __device__ __forceinline__ void sort_chunk(const uint64_t* in, uint64_t* out, in
         }
       }
     }
-    __syncthreads();
+    sync();
     uint64_t* tmp = src;
     src = dst;
     dst = tmp;
   }
-  for (int i = threadIdx.x; i < n; i += TH) out[i] = src[pad(i)];
+  for (int i = t; i < n; i += TH) out[i] = src[pad(i)];
 }
 
 // Merge rounds of a segment of nch chunks, and of one of n keys: ceil(log2(chunks)).
@@ -254,7 +262,7 @@ __device__ __forceinline__ void select_prefix(const BatchDev& b, int64_t t, uint
     if (threadIdx.x == 0) { atomicOr(b.status, ST_BOUNDS); b.sel[t] = kSelNone; }
     return;
   }
-  sort_chunk<kSortThreads>(sb, b.keys_alt + s, (int)S, sa, sb);
+  sort_chunk<kSortThreads>(sb, b.keys_alt + s, (int)S, sa, sb, (int)threadIdx.x);
   if (threadIdx.x == 0) {
     b.sel[t] = S;
     const uint32_t off = (uint32_t)b.capacity + s;
@@ -412,40 +420,74 @@ void launch_fill(const BatchDev& b, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- segment sorts
-// One CTA per tile: ranges, then either the whole segment (<= kChunk keys) or, for a
-// longer one, its registration as chunk work items (segment list index, chunk index).
-__global__ void __launch_bounds__(kSortThreads) k_seg_sort_small(const BatchDev b) {
+// Ranges and sorts of the tile segments, `group` (1 to 8) tiles per CTA.  Each of its first
+// `group` warps takes a tile: a segment of up to 256 keys is sorted by its warp alone, in an
+// eighth of the shared memory; a longer one by the whole CTA afterwards, if it has at most
+// kChunk keys, or else as a selected prefix or registered with the long-segment sort.
+//
+// With one CTA per tile most tiles used one warp of eight (a 2M-Gaussian batch of 4 views
+// has 180 keys a segment on average) and the others waited at its barriers: the segment
+// sorts of 4 views and 32 subsets over 20M Gaussians, 20 keys a segment, 1.22 -> 0.41 ms.
+// kSolo (small launches): one tile per CTA, looked up by all its warps and sorted by the
+// whole CTA without the exchange (a 10k-Gaussian 256x256 render 105.6 us, 108 with it).
+template <bool kSolo>
+__global__ void __launch_bounds__(kSortThreads, 6) k_seg_sort(const BatchDev b, int group) {
   __shared__ uint64_t sk[2][kPadded];
   __shared__ unsigned s_base;
   __shared__ unsigned s_tmp[11];
-  const int64_t t = item_of(b, blockIdx.x);
-  uint32_t s, e;
-  segment_of(b, t, s, e);
-  // the pairs the cross-boundary filter removed sort last and stay out of the range
-  if (threadIdx.x == 0) {
-    const uint32_t cut = b.removed ? min(b.removed[t], e - s) : 0u;
-    b.ranges[t] = make_uint2(s, e - cut);
-    if (b.sel) b.sel[t] = 0u;
+  __shared__ uint2 s_seg[kSortThreads / 32];  // start and length of the longer segments
+  const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+  const int64_t first = (int64_t)blockIdx.x * group;
+  uint2 longer = make_uint2(0u, 0u);
+  const int mine = kSolo ? 0 : warp;
+  if (mine < group && first + mine < items_of_launch(b)) {
+    const int64_t t = item_of(b, first + mine);
+    uint32_t s, e;
+    segment_of(b, t, s, e);
+    // the pairs the cross-boundary filter removed sort last and stay out of the range
+    if (lane == 0 && warp == mine) {
+      const uint32_t cut = b.removed ? min(b.removed[t], e - s) : 0u;
+      b.ranges[t] = make_uint2(s, e - cut);
+      if (b.sel) b.sel[t] = 0u;
+    }
+    const int n = (int)(e - s);
+    // saturation-skipping waves sort only what the wave's rasteriser will walk; likewise
+    // with a stale saturation state a tile pruned at every pixel stays unsorted
+    if (n > 1 && !(b.order && b.wave > 0 && item_saturated(b, t)) &&
+        !(b.sat && item_pruned(b, t))) {
+      if (kSolo || n > kWarpKeys)
+        longer = make_uint2(s, (uint32_t)n);
+      else
+        sort_chunk<32>(b.keys + s, b.keys + s, n, sk[0] + warp * kWarpPadded,
+                       sk[1] + warp * kWarpPadded, lane);
+    }
   }
-  const int n = (int)(e - s);
-  if (n <= 1) return;
-  // saturation-skipping waves sort only what the wave's rasteriser will walk
-  if (b.order && b.wave > 0 && item_saturated(b, t)) return;
-  // likewise with a stale saturation state: a tile pruned at every pixel stays unsorted
-  if (b.sat && item_pruned(b, t)) return;
-  if (n > kChunk && b.sel) {
-    select_prefix(b, t, s, e, sk[0], sk[1], s_tmp);
-    return;
-  }
-  if (n > kChunk) {
-    if (threadIdx.x == 0) s_base = register_long(b, t, (uint32_t)n);
+  if (!kSolo) {
+    if (lane == 0) s_seg[warp] = longer;
     __syncthreads();
-    const unsigned nch = long_chunks((uint32_t)n), first = s_base;
-    for (unsigned c = threadIdx.x; c < nch; c += kSortThreads)
-      b.chunks[first + c] = make_uint2((uint32_t)t, first);
-    return;
   }
-  sort_chunk<kSortThreads>(b.keys + s, b.keys + s, n, sk[0], sk[1]);
+  for (int q = 0; q < (kSolo ? 1 : group); ++q) {
+    const uint2 seg = kSolo ? longer : s_seg[q];
+    const uint32_t s = seg.x;
+    const int n = (int)seg.y;
+    if (n == 0) continue;
+    if (n <= kChunk) {
+      sort_chunk<kSortThreads>(b.keys + s, b.keys + s, n, sk[0], sk[1], (int)threadIdx.x);
+      __syncthreads();  // shared memory is free for the next segment
+      continue;
+    }
+    const int64_t t = item_of(b, first + q);
+    if (b.sel) {
+      select_prefix(b, t, s, s + (uint32_t)n, sk[0], sk[1], s_tmp);
+    } else {
+      if (threadIdx.x == 0) s_base = register_long(b, t, (uint32_t)n);
+      __syncthreads();
+      const unsigned nch = long_chunks((uint32_t)n), at = s_base;
+      for (unsigned c = threadIdx.x; c < nch; c += kSortThreads)
+        b.chunks[at + c] = make_uint2((uint32_t)t, at);
+    }
+    __syncthreads();  // likewise
+  }
 }
 
 // One merge item: outputs [o0, o0 + 4096) of the round that merges runs of w keys of a
@@ -542,7 +584,7 @@ __global__ void __launch_bounds__(kBigThreads) k_long_sort(const BatchDev b) {
     if (q == 0) {
       const uint32_t c0 = s + o0, c1 = c0 + kBig < e ? c0 + kBig : e;
       uint64_t* out = ((R & 1u) ? b.keys_alt : b.keys) + c0;
-      sort_chunk<kBigThreads>(b.keys + c0, out, (int)(c1 - c0), sa, sb);
+      sort_chunk<kBigThreads>(b.keys + c0, out, (int)(c1 - c0), sa, sb, (int)threadIdx.x);
     } else {
       if (threadIdx.x == 0) {
         const volatile uint32_t* done = b.seg_done + t;
@@ -589,8 +631,17 @@ void launch_long_sort(const BatchDev& b, cudaStream_t s) {
 
 void launch_seg_sort(const BatchDev& b, cudaStream_t s) {
   if (b.n_tiles == 0) return;
-  const int64_t items = b.order ? b.item_n : b.n_tiles;
-  k_seg_sort_small<<<(unsigned)items, kSortThreads, 0, s>>>(b);
+  const int64_t items = items_of_launch(b);
+  // Tiles per CTA.  Short lists (by the room for pairs per tile: the true mean is not known
+  // here) go eight to a CTA, longer ones, which its tiles take in turn as whole CTAs, two: 1M
+  // lists of 20 keys on average 0.42 ms at 8, 0.51 at 4, 0.74 at 2, 1.22 at 1; 170k lists of
+  // 180 keys 0.73, 0.69, 0.70, 0.77; 35k lists of 300 keys 0.28, 0.24, 0.23, 0.23.  Fewer
+  // where that would leave less than two CTAs of work for every resident one
+  int group = b.capacity < 128 * b.n_tiles ? kSortThreads / 32 : 2;
+  while (group > 1 && items < (int64_t)device_sm_count() * 12 * group) group /= 2;
+  const unsigned grid = (unsigned)((items + group - 1) / group);
+  if (group == 1) k_seg_sort<true><<<grid, kSortThreads, 0, s>>>(b, 1);
+  else k_seg_sort<false><<<grid, kSortThreads, 0, s>>>(b, group);
   count_launch();
   // with selected prefixes no segment is left to the long-segment sort before the forward
   if (!b.sel) launch_long_sort(b, s);

@@ -362,13 +362,13 @@ __device__ __forceinline__ int64_t item_of(const BatchDev& b, int64_t w) {
   return b.tile_base[v] + (int64_t)k * nt + (w - b.tile_base[v] / b.K);
 }
 
-__device__ __forceinline__ int64_t items_of_launch(const BatchDev& b) {
+__host__ __device__ __forceinline__ int64_t items_of_launch(const BatchDev& b) {
   return b.order ? b.item_n : b.n_tiles;
 }
 
 // Saturation skipping test of work item `id` in a wave after the first: true if every pixel
-// of its tile has prefix transmittance below eps_comp.  Whole-CTA call (uses
-// __syncthreads_or); the rasteriser and the segment sort take the same decision.
+// of its tile has prefix transmittance below eps_comp.  Whole-warp call; the rasteriser and
+// the segment sort take the same decision.
 __device__ __forceinline__ bool item_saturated(const BatchDev& b, int64_t id) {
   const int v = view_of(b.tile_base, b.V, id);
   const ViewDev& cam = b.views[v];
@@ -376,12 +376,13 @@ __device__ __forceinline__ bool item_saturated(const BatchDev& b, int64_t id) {
   const int64_t t = (id - b.tile_base[v]) % nt;
   const int x0 = (int)(t % cam.tiles_x) * b.tile, y0 = (int)(t / cam.tiles_x) * b.tile;
   const float* tp = b.tpre + b.pix_off[v];
+  const int tsh = __ffs(b.tile) - 1;  // the tile side is a power of two
   bool open = false;
-  for (int i = threadIdx.x; i < b.tile * b.tile; i += blockDim.x) {
-    const int x = x0 + i % b.tile, y = y0 + i / b.tile;
+  for (int i = threadIdx.x & 31; i < b.tile * b.tile; i += 32) {
+    const int x = x0 + (i & (b.tile - 1)), y = y0 + (i >> tsh);
     if (x < cam.W && y < cam.H) open |= tp[(int64_t)y * cam.W + x] >= b.eps_comp;
   }
-  return !__syncthreads_or(open);
+  return !__any_sync(0xffffffffu, open);
 }
 
 // Cross-boundary per-ray filtering (Sec. 8.1): whether a Gaussian of subset k whose support
@@ -409,7 +410,7 @@ __device__ __forceinline__ bool cross_removed(const BatchDev& b, int v, int k,
 }
 
 // Stale-state test of work item `id` (a whole tile of subset k in view v): true if every
-// pixel of the tile has subset k pruned (its rank >= the pixel's state).  Whole-CTA call;
+// pixel of the tile has subset k pruned (its rank >= the pixel's state).  Whole-warp call;
 // the rasteriser and the segment sort take the same decision.
 __device__ __forceinline__ bool item_pruned(const BatchDev& b, int64_t id) {
   const int v = view_of(b.tile_base, b.V, id);
@@ -420,12 +421,13 @@ __device__ __forceinline__ bool item_pruned(const BatchDev& b, int64_t id) {
   const int x0 = (int)(t % cam.tiles_x) * b.tile, y0 = (int)(t / cam.tiles_x) * b.tile;
   const uint8_t* sp = b.sat[v];
   const int rk = b.rank[v * b.K + k];
+  const int tsh = __ffs(b.tile) - 1;  // the tile side is a power of two
   bool open = false;
-  for (int i = threadIdx.x; i < b.tile * b.tile; i += blockDim.x) {
-    const int x = x0 + i % b.tile, y = y0 + i / b.tile;
+  for (int i = threadIdx.x & 31; i < b.tile * b.tile; i += 32) {
+    const int x = x0 + (i & (b.tile - 1)), y = y0 + (i >> tsh);
     if (x < cam.W && y < cam.H) open |= (int)sp[(int64_t)y * cam.W + x] > rk;
   }
-  return !__syncthreads_or(open);
+  return !__any_sync(0xffffffffu, open);
 }
 
 // Two FP32 values in one 64-bit register pair, and the packed operations on them (sm_100 and
