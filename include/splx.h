@@ -321,7 +321,11 @@ int splx_batch_set_prefix_sort(splx_batch_t b, int32_t enable);
 /* Keeps the selected-prefix sort on only if the last eager forward handed at most a
  * quarter of its prefix items back to the whole sort (their pixels still blending at the
  * prefix's end: tiles with long lists of small or faint Gaussians), and turns it off
- * otherwise, for launches issued afterwards; call it between an eager forward and a graph
+ * otherwise; with subset orders set, also where that forward's waves skipped under a
+ * sixteenth of the work items inside the visible regions and under a 64th of them had such
+ * a list.  With it off by this call, saturation skipping sorts every segment first and
+ * renders all subsets in one launch, a tile's front to back, instead of waves (the same
+ * results).  For launches issued afterwards; call it between an eager forward and a graph
  * capture.  Synchronises `stream`; not capturable; SPLX_ERR_INVALID without a batch state. */
 int splx_batch_tune_prefix_sort(splx_batch_t b, splx_stream_t stream);
 /* Cross-boundary per-ray filtering (Sec. 8.1, appendix "Cross-boundary Gaussians
@@ -378,9 +382,9 @@ int splx_batch_kernel_times(splx_batch_t b, float* ms_out);
 int splx_batch_kernel_times_slot(splx_batch_t b, splx_graph_t g, int32_t slot, float* ms_out);
 /* Work counters (synchronises; host array of 11): out[0] = (Gaussian, tile) pairs of the
  * last run; then, from the last EAGER run (replays of a captured graph do not count):
- * forward rasteriser out[1] = (thread, list entry) pairs examined, out[2] = (pixel,
- * entry) alpha evaluations, out[3] = (pixel, entry) blends; backward rasteriser out[4] =
- * (thread, entry) pairs, out[5] = alpha evaluations, out[6] = contributions (alpha >=
+ * forward rasteriser out[1] = (warp, list entry) pairs whose entry reaches the warp's
+ * pixels, out[2] = (pixel, entry) alpha evaluations, out[3] = (pixel, entry) blends;
+ * backward rasteriser out[4] = the same (warp, entry) pairs, out[5] = alpha evaluations, out[6] = contributions (alpha >=
  * alpha_min); out[7] = (view, subset, tile) work items left empty by saturation skipping
  * (no open pixel); out[8] = work items outside their subset's visible region; out[9] =
  * work items whose segment, longer than 2048 keys, the forward walked on its sorted
@@ -388,8 +392,8 @@ int splx_batch_kernel_times_slot(splx_batch_t b, splx_graph_t g, int32_t slot, f
  * prefix) whose pixels were still open at the prefix's end, so that the segment was
  * sorted whole and the item rendered again (the batch's results are those of whole
  * sorts either way).
- * A forward thread owns 2 pixels (8x8, 16x16 tiles) or 4 (32x32); a backward thread 2
- * (8x8), 8 (16x16: one warp per tile) or 4 (32x32). */
+ * A forward warp owns an 8x8 region (8x8, 16x16 tiles) or a 16x8 one (32x32), a backward
+ * warp an 8x8 block. */
 int splx_batch_counters(splx_batch_t b, int64_t* out, splx_stream_t stream);
 /* Number of (view, Gaussian) pairs that the last forward's projection kept (a tile count
  * above zero: the Gaussians that write a record and may receive a 2-D gradient), for the

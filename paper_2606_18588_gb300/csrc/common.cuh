@@ -116,8 +116,8 @@ struct BatchDev {
   // ge dx, ge dy, ge dx^2, ge dx dy, ge dy^2 (ge = dL/dpower / o), dL/do, dL/dcolour
   float4* grad2d;
   int* status;                  // device status word
-  // work counters (nullable; kept by eager runs): forward [0] thread-entries examined,
-  // [1] (pixel, entry) alpha evaluations, [2] blends; backward [3] thread-entries,
+  // work counters (nullable; kept by eager runs): forward [0] (warp, entry) pairs that meet,
+  // [1] (pixel, entry) alpha evaluations, [2] blends; backward [3] (warp, entry) pairs,
   // [4] alpha evaluations, [5] contributions (alpha >= alpha_min); [6] work items left
   // empty by saturation skipping; [7] work items outside their subset's visible region;
   // [8] work items the forward walked on a selected prefix, [9] of those, the ones it
@@ -239,6 +239,8 @@ inline int64_t chunk_list_capacity(int64_t n_tiles, int64_t capacity) {
   return n_tiles + capacity / 2048 + 1;
 }
 void launch_raster_fwd(const BatchDev& b, cudaStream_t s);
+// The saturation-skipping waves of all views in one launch, after one sort of every segment.
+void launch_raster_fwd_ordered(const BatchDev& b, cudaStream_t s);
 // Whole sort of the segments registered in b.chunks (register_long).
 void launch_long_sort(const BatchDev& b, cudaStream_t s);
 // The full sort of the segments the forward handed back (hand_back) and their second

@@ -197,8 +197,8 @@ constexpr float kWild = 1e18f;
 // 2.37 ms, a branch per stopping pair 2.46 ms, 10 CTAs per SM at 48 registers (spilling)
 // and 7 at 72 1-2 % more than 8 at 64.
 template <int TS, int PPT, bool kCount>
-__device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, float4* sA,
-                                         float4* sB, float4* sC, float* sR) {
+__device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, const int wave,
+                                         float4* sA, float4* sB, float4* sC, float* sR) {
   constexpr int NTH = TS * TS / PPT;
   constexpr int NB = kNBFwd<TS>;
   constexpr int PER = NB > NTH ? NB / NTH : 1;  // staged entries per thread
@@ -209,7 +209,7 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
     // outside the subset's visible region: no pairs; the composite never reads this tile.
     // Its transmittance is 1, which the first saturation-skipping wave must still record.
     if (kCount && threadIdx.x == 0 && b.counters) atomicAdd(b.counters + 7, 1ull);
-    if (b.order && b.wave == 0) {
+    if (b.order && wave == 0) {
 #pragma unroll
       for (int i = 0; i < PPT; ++i) {
         const int px = ti.x + 8 * slot_col<PPT>(i), py = ti.y + 4 * slot_row<PPT>(i);
@@ -236,7 +236,7 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
   }
   // (the planes' addresses are read again where they are used: nothing holds them in
   // registers across the walk)
-  if ((b.order && b.wave > 0) || b.sat) {
+  if ((b.order && wave > 0) || b.sat) {
     const unsigned inb = live;  // slots inside the image
     // saturation skipping: a pixel where the subsets rendered before this one took the
     // transmittance below eps_comp leaves this subset's pixel set (the composite would
@@ -551,7 +551,7 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, fl
       const int px = ti.x + 8 * slot_col<PPT>(i), py = ti.y + 4 * slot_row<PPT>(i);
       if (px >= ti.W || py >= ti.H) continue;
       float* tp = b.tpre + b.pix_off[ti.v] + (int64_t)py * ti.W + px;
-      *tp = b.wave == 0 ? T[i] : *tp * T[i];
+      *tp = wave == 0 ? T[i] : *tp * T[i];
     }
   }
 }
@@ -924,7 +924,7 @@ __global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>) k_raster_fwd
   __shared__ float4 sA[2 * kNBFwd<TS>], sB[2 * kNBFwd<TS>], sC[2 * kNBFwd<TS>];
   __shared__ __align__(16) float sR[kRingWords<TS, PPT>];
   if constexpr (!kPersist) {
-    fwd_item<TS, PPT, kCount>(b, item_of(b, blockIdx.x), sA, sB, sC, sR);
+    fwd_item<TS, PPT, kCount>(b, item_of(b, blockIdx.x), b.wave, sA, sB, sC, sR);
   } else {
     __shared__ long long s_id;
     for (;;) {
@@ -933,8 +933,33 @@ __global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>) k_raster_fwd
       __syncthreads();
       const int64_t id = s_id;
       if (id >= items_of_launch(b)) return;
-      fwd_item<TS, PPT, kCount>(b, item_of(b, id), sA, sB, sC, sR);
+      fwd_item<TS, PPT, kCount>(b, item_of(b, id), b.wave, sA, sB, sC, sR);
     }
+  }
+}
+
+// Saturation skipping without waves: a CTA per image tile of a view renders the tile's K
+// subsets in the view's order, one after another; the prefix transmittance it reads is the
+// one its own threads wrote.  The same items in the same order as the waves, so the same
+// results; it needs every segment sorted beforehand, also those that the waves would have
+// left unsorted behind saturated tiles, and no selected prefixes (a handed-back item would
+// have to be finished before the next).  For scenes whose lists are walked to their ends
+// (launch_raster_fwd_ordered's caller): 20M Gaussians, 32 subsets, 4 views at 1080p, sorts
+// and forward 3.5 ms in 128 launches of each kind.
+template <int TS, int PPT, bool kCount>
+__global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>)
+    k_raster_fwd_ordered(const BatchDev b) {
+  __shared__ float4 sA[2 * kNBFwd<TS>], sB[2 * kNBFwd<TS>], sC[2 * kNBFwd<TS>];
+  __shared__ __align__(16) float sR[kRingWords<TS, PPT>];
+  const int64_t w = blockIdx.x;
+  const int v = view_of(b.tile_base, b.V, w * b.K);
+  const int64_t nt = (b.tile_base[v + 1] - b.tile_base[v]) / b.K;
+  const int64_t t0 = b.tile_base[v] + (w - b.tile_base[v] / b.K);
+  const int32_t* order = b.order + (int64_t)v * b.K;
+#pragma unroll 1
+  for (int r = 0; r < b.K; ++r) {
+    fwd_item<TS, PPT, kCount>(b, t0 + order[r] * nt, r, sA, sB, sC, sR);
+    __syncthreads();  // shared memory is free for the next subset
   }
 }
 
@@ -948,7 +973,7 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_raster_fwd_retry(const BatchD
   const unsigned n = *b.retry_count;
   for (unsigned w = blockIdx.x; w < n; w += gridDim.x) {
     __syncthreads();  // the previous item is done with shared memory
-    fwd_item<TS, PPT, kCount>(b, (int64_t)b.retry[w], sA, sB, sC, sR);
+    fwd_item<TS, PPT, kCount>(b, (int64_t)b.retry[w], b.wave, sA, sB, sC, sR);
   }
 }
 
@@ -1065,6 +1090,24 @@ void launch_raster_fwd(const BatchDev& b, cudaStream_t s) {
     case 8: launch_fwd_t<8>(b, s); break;
     case 32: launch_fwd_t<32>(b, s); break;
     default: launch_fwd_t<16>(b, s); break;
+  }
+  count_launch();
+}
+
+template <int TS>
+static void launch_fwd_ordered_t(const BatchDev& b, cudaStream_t s) {
+  constexpr int P = PptFwd<TS>::value;
+  const unsigned grid = (unsigned)(b.n_tiles / b.K);
+  if (counting(b, s)) k_raster_fwd_ordered<TS, P, true><<<grid, TS * TS / P, 0, s>>>(b);
+  else k_raster_fwd_ordered<TS, P, false><<<grid, TS * TS / P, 0, s>>>(b);
+}
+
+void launch_raster_fwd_ordered(const BatchDev& b, cudaStream_t s) {
+  if (b.n_tiles == 0) return;
+  switch (b.tile) {
+    case 8: launch_fwd_ordered_t<8>(b, s); break;
+    case 32: launch_fwd_ordered_t<32>(b, s); break;
+    default: launch_fwd_ordered_t<16>(b, s); break;
   }
   count_launch();
 }

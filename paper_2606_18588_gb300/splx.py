@@ -544,7 +544,9 @@ class Batch:
 
     def tune_prefix_sort(self, stream=None):
         """Keeps the selected-prefix sort only if the last eager forward handed at most a
-        quarter of its prefix items back to the whole sort (synchronises)."""
+        quarter of its prefix items back to the whole sort and, with subset orders set, skipped
+        or long lists are not rare; otherwise saturation skipping takes one sort and one
+        forward launch instead of waves (synchronises)."""
         _check(_lib.splx_batch_tune_prefix_sort(self.h, _stream(stream)),
                "splx_batch_tune_prefix_sort")
 
