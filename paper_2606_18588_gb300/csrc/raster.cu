@@ -290,6 +290,10 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, co
   if (b.sel) {
     const uint32_t sv = b.sel[id];
     if (sv == kSelNone) {
+      // (hand_back rewrites sel[id] and ranges[id]: not before every warp has read them, or a
+      // late one would take the unsorted segment for a sorted list.  sv is the same for the
+      // whole CTA, so all its threads meet here)
+      __syncthreads();
       if (threadIdx.x == 0) {
         hand_back(b, (uint32_t)id, kSelNone);
         if (kCount && b.counters) atomicAdd(b.counters + 9, 1ull);
