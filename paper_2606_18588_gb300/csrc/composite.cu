@@ -2,14 +2,21 @@
 // view of the batch, plus the L1 photometric loss.
 //
 // Both are bound by HBM latency rather than bandwidth: their work per byte is a sort of a few
-// keys.  A warp takes a patch of one tile, so the subsets whose visible region misses the
-// tile drop out for all its lanes at once, before anything is read; what is left is loaded,
-// sorted and blended in registers, with the pointers of all planes in the lanes' registers
-// and the colours of four subsets in flight.  Before, a thread looped over all K subsets and
-// kept their keys and order in local memory.  Measured (composite, adjoint): K = 32, 4 views
-// 1920x1080 of the 20M-Gaussian city, where a tile has one or two subsets, 0.97 -> 0.14 and
-// 1.64 -> 0.19 ms; K = 8, 16 views of 10M 0.64 -> 0.46 and 1.02 -> 0.66 ms; 16 partials of
-// 1600x1064 from outside 211 -> 156 us (3.7 TB/s).
+// keys.  With visible regions a warp takes a patch of one tile, so the subsets whose region
+// misses the tile drop out for all its lanes at once, before anything is read; without them
+// it takes 32 consecutive pixels, whole lines of every plane.  What is left is loaded, sorted
+// and blended in registers, with the pointers of all planes in the lanes' registers and the
+// colours of four subsets in flight.  Measured (composite, adjoint; before: a thread per
+// pixel, keys and order in local memory): K = 32, 4 views 1920x1080 of the 20M-Gaussian city,
+// where a tile has one or two subsets, 0.97 -> 0.14 and 1.64 -> 0.19 ms; K = 8, 16 views of
+// 10M 0.64 -> 0.46 and 1.02 -> 0.66 ms; 16 partials of 1600x1064 from outside 212 -> 153 us
+// (157 in patches of a tile).
+//
+// The thread per pixel stays where it is the better form.  One subset has no order (1M
+// Gaussians, 2 views 1600x1064: composite 24 us, adjoint 23; a patch 24 and 42).  More than
+// 16 subsets without regions go through local memory: 24 partials of 1600x1064, every pixel
+// covered, 0.90 ms, against 1.05 ms by the patches' array form, which stays for tiles with
+// more than 8 subsets of a launch with regions (K = 24, every tile with all: 1.08 ms).
 //
 // Order: subsets sorted per pixel by the normalised depth D^m / (1 - T^m), a convex
 // combination of the subset's contributor depths (Eq. 4 read as D = sum d alpha T);
@@ -25,8 +32,10 @@ namespace splx {
 
 namespace {
 
-// A warp's 32 pixels: a patch of one tile (32x1, 16x2 or 8x4 for tiles of 32, 16, 8), so that
-// the subsets whose visible region holds the tile are the same for all of them.
+// A warp's 32 pixels: with visible regions a patch of one tile (32x1, 16x2 or 8x4 for tiles of
+// 32, 16, 8), so that the subsets whose visible region holds the tile are the same for all of
+// them; without (every subset everywhere) 32 consecutive pixels of a view, so that a plane is
+// read and written by whole lines.
 struct Patch {
   int v;
   bool in;          // the lane's pixel lies in the image
@@ -37,6 +46,22 @@ struct Patch {
 __device__ __forceinline__ Patch patch_of(const BatchDev& b, int64_t warp) {
   Patch q;
   const int lane = (int)(threadIdx.x & 31);
+  if (!b.omega) {
+    // view v's warps start at first_warp(v): room for a last warp of fewer pixels
+    auto first_warp = [&](int v) { return (b.pix_off[v] >> 5) + v; };
+    int lo = 0, hi = b.V - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (first_warp(mid) <= warp) lo = mid; else hi = mid - 1;
+    }
+    q.v = lo;
+    q.HW = b.pix_off[lo + 1] - b.pix_off[lo];
+    const int64_t p = ((warp - first_warp(lo)) << 5) + lane;
+    q.in = p < q.HW;
+    q.p = q.in ? p : 0;
+    q.inside = ~0ull >> (64 - b.K);
+    return q;
+  }
   const int sh = __ffs(b.tile) - 1;  // the tile side is a power of two
   const int pp = 2 * sh - 5;         // log2 of the patches per tile
   const int64_t t = warp >> pp;
@@ -251,45 +276,82 @@ __device__ __forceinline__ void composite_bwd_patch(const BatchDev& b, const Pat
 }
 
 // More inside subsets than the register forms hold: the same, through arrays indexed at run
-// time (local memory).
+// time (local memory).  All lanes run along (the planes' pointers come by shuffles).
 struct PixOrderAny {
   float T[kMaxK], key[kMaxK];
   int ord[kMaxK];
 
+  // kLoads: subsets whose planes are in flight together
+  template <int kLoads>
   __device__ __forceinline__ int load(const BatchDev& b, const Patch& q) {
+    Planes<true> pt, pd;
+    const ImgDev *a = lane_img(b, q, 0), *c = lane_img(b, q, 1);
+    pt.set(a->T, c->T);
+    pd.set(a->D, c->D);
     int n = 0;
-    for (uint64_t rest = q.inside; rest; rest &= rest - 1) {
-      const int m = __ffsll((long long)rest) - 1;
-      const ImgDev& im = b.imgs[q.v * b.K + m];
-      const float t = im.T[q.p], d = im.D[q.p];
-      const float km = t < 1.0f ? d / (1.0f - t) : __int_as_float(0x7f800000);
-      T[m] = t;
-      key[m] = km;
-      int j = n++;
-      while (j > 0 && key[ord[j - 1]] > km) {
-        ord[j] = ord[j - 1];
-        --j;
+    for (uint64_t rest = q.inside; rest;) {
+      float t[kLoads], d[kLoads];
+      int m[kLoads];
+#pragma unroll
+      for (int i = 0; i < kLoads; ++i) {
+        m[i] = -1;
+        if (rest) {
+          m[i] = __ffsll((long long)rest) - 1;
+          rest &= rest - 1;
+          t[i] = pt.get<const float*>(m[i])[q.p];
+          d[i] = pd.get<const float*>(m[i])[q.p];
+        }
       }
-      ord[j] = m;
+#pragma unroll
+      for (int i = 0; i < kLoads; ++i) {
+        if (m[i] < 0) continue;
+        const float km = t[i] < 1.0f ? d[i] / (1.0f - t[i]) : __int_as_float(0x7f800000);
+        T[m[i]] = t[i];
+        key[m[i]] = km;
+        int j = n++;
+        while (j > 0 && key[ord[j - 1]] > km) {
+          ord[j] = ord[j - 1];
+          --j;
+        }
+        ord[j] = m[i];
+      }
     }
     return n;
   }
 };
 
 __device__ __noinline__ void composite_any(const BatchDev& b, const Patch& q) {
-  if (!q.in) return;
   PixOrderAny po;
-  const int n = po.load(b, q);
+  const int n = po.load<4>(b, q);
+  Planes<true> pr;
+  pr.set(lane_img(b, q, 0)->rgb, lane_img(b, q, 1)->rgb);
   float P = 1.0f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-  for (int j = 0; j < n; ++j) {
-    if (P < b.eps_comp) break;
-    const int m = po.ord[j];
-    const float* rgb = b.imgs[q.v * b.K + m].rgb;
-    c0 = fmaf(rgb[q.p], P, c0);
-    c1 = fmaf(rgb[q.HW + q.p], P, c1);
-    c2 = fmaf(rgb[2 * q.HW + q.p], P, c2);
-    P *= po.T[m];
+  for (int j0 = 0; j0 < n; j0 += kAhead) {
+    if (__all_sync(0xffffffffu, P < b.eps_comp)) break;
+    float r[kAhead], g[kAhead], bl[kAhead], w[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      r[i] = g[i] = bl[i] = w[i] = 0.0f;
+      if (j0 + i < n) {
+        const int m = po.ord[j0 + i];
+        const float* rgb = pr.get<const float*>(m);
+        if (!(P < b.eps_comp)) {
+          r[i] = rgb[q.p];
+          g[i] = rgb[q.HW + q.p];
+          bl[i] = rgb[2 * q.HW + q.p];
+          w[i] = P;
+          P *= po.T[m];
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      c0 = fmaf(r[i], w[i], c0);
+      c1 = fmaf(g[i], w[i], c1);
+      c2 = fmaf(bl[i], w[i], c2);
+    }
   }
+  if (!q.in) return;
   float* orgb = b.out_rgb + 3 * b.pix_off[q.v];
   orgb[q.p] = fmaf(b.bg[0], P, c0);
   orgb[q.HW + q.p] = fmaf(b.bg[1], P, c1);
@@ -298,48 +360,79 @@ __device__ __noinline__ void composite_any(const BatchDev& b, const Patch& q) {
 }
 
 __device__ __noinline__ void composite_bwd_any(const BatchDev& b, const Patch& q) {
-  if (!q.in) return;
   PixOrderAny po;
-  const int n = po.load(b, q);
-  float Pj[kMaxK];
+  const int n = po.load<8>(b, q);
+  Planes<true> pr, pg;
+  const ImgDev *ia = lane_img(b, q, 0), *ib = lane_img(b, q, 1);
+  pr.set(ia->rgb, ib->rgb);
+  pg.set(ia->gCT, ib->gCT);
+  // key[m] becomes the prefix P of the subsets before the cut, the first L in the order
   float P = 1.0f;
   int L = 0;
   for (int j = 0; j < n; ++j) {
     if (P < b.eps_comp) break;
-    Pj[j] = P;
-    P *= po.T[po.ord[j]];
+    const int m = po.ord[j];
+    po.key[m] = P;
+    P *= po.T[m];
     ++L;
   }
   const float* dl = b.dL_drgb + 3 * b.pix_off[q.v];
   const float g0 = dl[q.p], g1 = dl[q.HW + q.p], g2 = dl[2 * q.HW + q.p];
   const float gT = b.dL_dT ? b.dL_dT[b.pix_off[q.v] + q.p] : 0.0f;
   float S0 = b.bg[0], S1 = b.bg[1], S2 = b.bg[2], Rt = 1.0f;
-  for (int j = n - 1; j >= 0; --j) {
-    const int m = po.ord[j];
-    const ImgDev& im = b.imgs[q.v * b.K + m];
-    if (j >= L) {
-      im.gCT[q.p] = make_float4(0.f, 0.f, 0.f, 0.f);
-      continue;
+  for (int j1 = n - 1; j1 >= 0; j1 -= kAhead) {
+    float r[kAhead], g[kAhead], bl[kAhead];
+    float4* out[kAhead];
+    int m[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int j = j1 - i;
+      r[i] = g[i] = bl[i] = 0.0f;
+      m[i] = 0;
+      out[i] = nullptr;
+      if (j >= 0) {
+        m[i] = po.ord[j];
+        const float* rgb = pr.get<const float*>(m[i]);
+        out[i] = pg.get<float4*>(m[i]) + q.p;
+        if (j < L) {
+          r[i] = rgb[q.p];
+          g[i] = rgb[q.HW + q.p];
+          bl[i] = rgb[2 * q.HW + q.p];
+        }
+      }
     }
-    const float Pm = Pj[j];
-    const float gTm = (g0 * S0 + g1 * S1 + g2 * S2) * Pm + gT * Pm * Rt;
-    im.gCT[q.p] = make_float4(g0 * Pm, g1 * Pm, g2 * Pm, gTm);
-    const float Tm = po.T[m];
-    S0 = fmaf(Tm, S0, im.rgb[q.p]);
-    S1 = fmaf(Tm, S1, im.rgb[q.HW + q.p]);
-    S2 = fmaf(Tm, S2, im.rgb[2 * q.HW + q.p]);
-    Rt *= Tm;
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int j = j1 - i;
+      if (j < 0) continue;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j < L) {
+        const float Pm = po.key[m[i]], Tm = po.T[m[i]];
+        const float gTm = (g0 * S0 + g1 * S1 + g2 * S2) * Pm + gT * Pm * Rt;
+        o = make_float4(g0 * Pm, g1 * Pm, g2 * Pm, gTm);
+        S0 = fmaf(Tm, S0, r[i]);
+        S1 = fmaf(Tm, S1, g[i]);
+        S2 = fmaf(Tm, S2, bl[i]);
+        Rt *= Tm;
+      }
+      if (q.in) *out[i] = o;
+    }
   }
 }
 
 }  // namespace
 
-// MK: the largest number of inside subsets taken in registers (4, 8 or 16 by K); kAny: more
-// are possible (K > 16; those kernels keep to 8 in registers, whose 48 and 64 registers hold
-// twice the warps of 16's 74 and 96, since few tiles have more).  A warp runs the form for its
-// own tile's number of subsets.
+// Resident CTAs of 256 threads that the register limits are set for.
 template <int MK, bool kAny, bool kBwd>
-__global__ void __launch_bounds__(256) k_composite(const BatchDev b, int64_t warps) {
+constexpr int kCompositeCtas = kBwd ? (MK <= 2 ? 6 : MK <= 4 ? 5 : MK <= 8 ? 4 : 2)
+                                    : (MK <= 2 ? 8 : MK <= 4 || kAny ? 6 : MK <= 8 ? 5 : 3);
+
+// MK: the largest number of inside subsets taken in registers (2, 4, 8 or 16 by K); kAny: more
+// are possible (K > 16 with visible regions; those kernels keep to 8 in registers, since few
+// tiles have more: their 40 and 64 registers hold twice the warps of 16's 76 and 93).  A warp
+// runs the form for its own tile's number of subsets.
+template <int MK, bool kAny, bool kBwd>
+__global__ void __launch_bounds__(256, kCompositeCtas<MK, kAny, kBwd>) k_composite(const BatchDev b, int64_t warps) {
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= warps) return;
   const Patch q = patch_of(b, w);
@@ -357,24 +450,168 @@ __global__ void __launch_bounds__(256) k_composite(const BatchDev b, int64_t war
       if (kBwd) composite_bwd_patch<8, kAny>(b, q, n); else composite_patch<8, kAny>(b, q, n);
     }
   } else {
-    if (kBwd) composite_bwd_patch<4, kAny>(b, q, n); else composite_patch<4, kAny>(b, q, n);
+    constexpr int M = MK < 4 ? MK : 4;
+    if (kBwd) composite_bwd_patch<M, kAny>(b, q, n); else composite_patch<M, kAny>(b, q, n);
   }
 }
 
+// More than 16 subsets without visible regions (splx_composite): a thread takes a pixel, its
+// order in local memory, MK subsets' planes unrolled.  32 registers: what bounds it is the
+// latency of the insertion's moves, which only more warps hide.
+template <int MK>
+struct PixOrderMany {
+  float T[MK], key[MK];
+  int ord[MK];
+
+  __device__ __forceinline__ void load(const BatchDev& b, int v, int64_t p) {
+#pragma unroll
+    for (int m = 0; m < MK; ++m) {
+      if (m < b.K) {
+        const ImgDev& im = b.imgs[v * b.K + m];
+        const float t = im.T[p];
+        const float d = im.D[p];
+        T[m] = t;
+        key[m] = t < 1.0f ? d / (1.0f - t) : __int_as_float(0x7f800000);
+      }
+    }
+    for (int m = 0; m < b.K; ++m) {  // insertion by (key, index): stable
+      int j = m;
+      const float km = key[m];
+      while (j > 0 && key[ord[j - 1]] > km) {
+        ord[j] = ord[j - 1];
+        --j;
+      }
+      ord[j] = m;
+    }
+  }
+};
+
+template <int MK, bool kBwd>
+__global__ void __launch_bounds__(256) k_composite_many(const BatchDev b, int64_t total) {
+  const int64_t gp = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (gp >= total) return;
+  const int v = view_of(b.pix_off, b.V, gp);
+  const ViewDev& cam = b.views[v];
+  const int64_t HW = (int64_t)cam.W * cam.H;
+  const int64_t p = gp - b.pix_off[v];
+  PixOrderMany<MK> po;
+  po.load(b, v, p);
+  float P = 1.0f;
+  if (!kBwd) {
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f;
+    for (int j = 0; j < b.K; ++j) {
+      if (P < b.eps_comp) break;
+      const int m = po.ord[j];
+      const float* rgb = b.imgs[v * b.K + m].rgb;
+      c0 = fmaf(rgb[p], P, c0);
+      c1 = fmaf(rgb[HW + p], P, c1);
+      c2 = fmaf(rgb[2 * HW + p], P, c2);
+      P *= po.T[m];
+    }
+    float* orgb = b.out_rgb + 3 * b.pix_off[v];
+    orgb[p] = fmaf(b.bg[0], P, c0);
+    orgb[HW + p] = fmaf(b.bg[1], P, c1);
+    orgb[2 * HW + p] = fmaf(b.bg[2], P, c2);
+    if (b.out_T) b.out_T[b.pix_off[v] + p] = P;
+    return;
+  }
+  float Pj[MK];
+  int L = 0;  // subsets before the cut
+  for (int j = 0; j < b.K; ++j) {
+    if (P < b.eps_comp) break;
+    Pj[j] = P;
+    P *= po.T[po.ord[j]];
+    ++L;
+  }
+  const float* dl = b.dL_drgb + 3 * b.pix_off[v];
+  const float g0 = dl[p], g1 = dl[HW + p], g2 = dl[2 * HW + p];
+  const float gT = b.dL_dT ? b.dL_dT[b.pix_off[v] + p] : 0.0f;
+  float S0 = b.bg[0], S1 = b.bg[1], S2 = b.bg[2], Rt = 1.0f;
+  for (int j = b.K - 1; j >= 0; --j) {
+    const int m = po.ord[j];
+    const ImgDev& im = b.imgs[v * b.K + m];
+    if (j >= L) {
+      im.gCT[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+      continue;
+    }
+    const float Pm = Pj[j];
+    const float gTm = (g0 * S0 + g1 * S1 + g2 * S2) * Pm + gT * Pm * Rt;
+    im.gCT[p] = make_float4(g0 * Pm, g1 * Pm, g2 * Pm, gTm);
+    const float Tm = po.T[m];
+    S0 = fmaf(Tm, S0, im.rgb[p]);
+    S1 = fmaf(Tm, S1, im.rgb[HW + p]);
+    S2 = fmaf(Tm, S2, im.rgb[2 * HW + p]);
+    Rt *= Tm;
+  }
+}
+
+// One subset: nothing to sort, so a thread takes a pixel of its own, in the planes' order.
+template <bool kBwd>
+__global__ void __launch_bounds__(256) k_composite_one(const BatchDev b, int64_t total) {
+  const int64_t gp = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (gp >= total) return;
+  const int v = view_of(b.pix_off, b.V, gp);
+  const ViewDev& cam = b.views[v];
+  const int64_t HW = (int64_t)cam.W * cam.H, p = gp - b.pix_off[v];
+  bool inside = true;
+  if (b.omega) {
+    const int sh = __ffs(b.tile) - 1;  // the tile side is a power of two
+    const uint32_t py = (uint32_t)p / (uint32_t)cam.W;
+    inside = in_omega(b, v, 0, (int)(((uint32_t)p - py * (uint32_t)cam.W) >> sh), (int)(py >> sh));
+  }
+  const ImgDev& im = b.imgs[v];
+  const bool take = inside && !(1.0f < b.eps_comp);
+  if (kBwd) {
+    if (!inside) return;  // never rendered
+    const float* dl = b.dL_drgb + 3 * b.pix_off[v];
+    const float g0 = dl[p], g1 = dl[HW + p], g2 = dl[2 * HW + p];
+    const float gT = b.dL_dT ? b.dL_dT[gp] : 0.0f;
+    im.gCT[p] = take ? make_float4(g0, g1, g2, g0 * b.bg[0] + g1 * b.bg[1] + g2 * b.bg[2] + gT)
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  float P = 1.0f, c[3] = {0.f, 0.f, 0.f};
+  if (take) {
+    P = im.T[p];
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) c[ch] = im.rgb[ch * HW + p];
+  }
+  float* orgb = b.out_rgb + 3 * b.pix_off[v];
+#pragma unroll
+  for (int ch = 0; ch < 3; ++ch) orgb[ch * HW + p] = fmaf(b.bg[ch], P, c[ch]);
+  if (b.out_T) b.out_T[gp] = P;
+}
+
 template <int MK, bool kAny>
-static void launch_c(const BatchDev& b, int64_t warps, bool bwd, cudaStream_t s) {
+static void launch_c(const BatchDev& b, int64_t total, bool bwd, cudaStream_t s) {
+  const int64_t warps =
+      b.omega ? b.n_tiles / b.K * (b.tile * b.tile / 32) : (total >> 5) + b.V;
   const unsigned blocks = (unsigned)((warps + 7) / 8);
   if (bwd) k_composite<MK, kAny, true><<<blocks, 256, 0, s>>>(b, warps);
   else k_composite<MK, kAny, false><<<blocks, 256, 0, s>>>(b, warps);
 }
+template <int MK>
+static void launch_pixels(const BatchDev& b, int64_t total, bool bwd, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((total + 255) / 256);
+  if constexpr (MK == 1) {
+    if (bwd) k_composite_one<true><<<blocks, 256, 0, s>>>(b, total);
+    else k_composite_one<false><<<blocks, 256, 0, s>>>(b, total);
+  } else {
+    if (bwd) k_composite_many<MK, true><<<blocks, 256, 0, s>>>(b, total);
+    else k_composite_many<MK, false><<<blocks, 256, 0, s>>>(b, total);
+  }
+}
 
 static void dispatch(const BatchDev& b, int64_t total, bool bwd, cudaStream_t s) {
   if (total <= 0) return;
-  const int64_t warps = b.n_tiles / b.K * (b.tile * b.tile / 32);
-  if (b.K <= 4) launch_c<4, false>(b, warps, bwd, s);
-  else if (b.K <= 8) launch_c<8, false>(b, warps, bwd, s);
-  else if (b.K <= 16) launch_c<16, false>(b, warps, bwd, s);
-  else launch_c<8, true>(b, warps, bwd, s);
+  if (b.K == 1) launch_pixels<1>(b, total, bwd, s);
+  else if (b.K <= 2) launch_c<2, false>(b, total, bwd, s);
+  else if (b.K <= 4) launch_c<4, false>(b, total, bwd, s);
+  else if (b.K <= 8) launch_c<8, false>(b, total, bwd, s);
+  else if (b.K <= 16) launch_c<16, false>(b, total, bwd, s);
+  else if (b.omega) launch_c<8, true>(b, total, bwd, s);
+  else if (b.K <= 32) launch_pixels<32>(b, total, bwd, s);
+  else launch_pixels<64>(b, total, bwd, s);
   count_launch();
 }
 
