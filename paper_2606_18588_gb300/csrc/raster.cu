@@ -606,9 +606,35 @@ __device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, co
   const TileInfo ti = decode_tile<TS, 2>(b, id);
   if (!in_omega(b, ti.v, ti.k, ti.tx, ti.ty)) return;  // nothing written there, nothing to do
   const int lane = (int)(threadIdx.x & 31);
+  const uint2 rg = b.ranges[id];  // (a selected prefix's range points into keys_alt)
+  const uint32_t start = rg.x;
+  const int len = rg.y > rg.x ? (int)(rg.y - rg.x) : 0;
+  if (len == 0) return;
   // the warp's block: RX, RY its origin on the image
   const int RX = ti.tx * TS + 8 * (blk % (TS / 8)), RY = ti.ty * TS + 8 * (blk / (TS / 8));
   const int x = RX + (lane & 7), y = RY + (lane >> 3);  // the lane's pixels: (x, y), (x, y + 4)
+  // Lane l holds entry top - l of each batch of 32: its record is copied behind the batch
+  // before (cp.async), its key (low half: the Gaussian) read one batch earlier still.  The
+  // walk of a list of at most 32 entries starts at its end, not at the pixels' last
+  // contributor (entries behind that are left out), so that its keys are on their way while
+  // the pixels' state is read: a short list's time is the latency of its reads, one behind
+  // the other.  500k Gaussians in 16 overlapping subsets, 2 views 1600x1064 (lists of tens):
+  // 1.84 -> 1.69 ms, in 40 subsets 2.82 -> 2.51; the 2M step 2.29 -> 2.22.
+  const bool whole = len <= 32;
+  int top = len - 1;  // list position of the batch's first entry
+  uint32_t nk = 0;
+  auto load_key = [&](int j) { nk = j >= 0 ? (uint32_t)b.keys[(uint64_t)start + j] : 0u; };
+  auto copy_record = [&](int j) {
+    if (j >= 0) {
+      if (nk >= (uint32_t)b.N) { atomicOr(b.status, ST_BOUNDS); nk = 0; }
+      const Rec* rp = b.rec + ((int64_t)ti.v * b.N + nk);
+      cp_async16(&sh.raw[0][lane], &rp->a);
+      cp_async16(&sh.raw[1][lane], &rp->b);
+      cp_async16(&sh.raw[2][lane], &rp->c);
+    }
+    cp_async_commit();
+  };
+  if (whole) load_key(top - lane);
   const float amax = b.alpha_max;
   const float amin_raw = b.alpha_min <= amax ? b.alpha_min : __int_as_float(0x7f800000);
   const float lg_amin = __log2f(b.alpha_min);
@@ -618,7 +644,7 @@ __device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, co
   int last0, last1;
   bool wild;  // an adjoint so large that 0 x (its products) might not be 0
   {
-    const ImgDev im = b.imgs[ti.v * b.K + ti.k];
+    const ImgDev& im = b.imgs[ti.v * b.K + ti.k];
     float Tm[2], Wm[2];
     float4 g[2];
     int last[2];
@@ -632,8 +658,8 @@ __device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, co
         const int64_t p = (int64_t)(y + 4 * h) * ti.W + x;
         g[h] = im.gCT[p];
         Tm[h] = im.T[p];
-        if (g[h].x != 0.0f || g[h].y != 0.0f || g[h].z != 0.0f || g[h].w != 0.0f)
-          last[h] = im.last[p];
+        last[h] = im.last[p];
+        if (g[h].x == 0.0f && g[h].y == 0.0f && g[h].z == 0.0f && g[h].w == 0.0f) last[h] = -1;
       }
       Wm[h] = -Tm[h] * g[h].w;
       wild |= !(fabsf(g[h].x) <= kWild) || !(fabsf(g[h].y) <= kWild) ||
@@ -659,8 +685,14 @@ __device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, co
     maxlast = cta->maxlast;
   }
   if (maxlast < 0) return;
+  if (!whole) {
+    top = maxlast;
+    load_key(top - lane);
+  }
+  copy_record(top - lane);
+  uint32_t g = nk;
+  load_key(top - 32 - lane);
   bool careful = __any_sync(0xffffffffu, wild);
-  const uint64_t start = b.ranges[id].x;  // (a selected prefix's range points into keys_alt)
   const uint32_t pm0 = (1u << (lane & 7)) | (1u << (8 + (lane >> 3))),
                  pm1 = (1u << (lane & 7)) | (1u << (12 + (lane >> 3)));
   const f32x2 pcx2 = pack2((float)x + 0.5f, (float)x + 0.5f),
@@ -732,7 +764,6 @@ __device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, co
   // columns) and add them to its 2-D gradient: the moments sum ge, ge dx, ge dy, ge dx^2,
   // ge dx dy, ge dy^2 (ge = dL/dpower / o = dL/do e^power) and dL/dcolour; the projection
   // adjoint applies the conic and the opacity.
-  int top = maxlast;  // list position of the batch's first entry
   auto sum_group = [&](int ri, int cnt) {
     const int e = lane >> 2, qd = lane & 3;
     const float* r = sh.ring + ((ri + e) >> 1) * kBwdPair + ((ri + e) & 1);
@@ -800,31 +831,13 @@ __device__ __forceinline__ void bwd_item(const BatchDev& b, const int64_t id, co
     }
   };
 
-  // Lane l holds entry top - l of each batch of 32: its record is copied behind the batch
-  // before (cp.async), its key (low half: the Gaussian) read one batch earlier still.
-  uint32_t nk = 0;
-  auto load_key = [&](int j) { nk = j >= 0 ? (uint32_t)b.keys[start + j] : 0u; };
-  auto copy_record = [&](int j) {
-    if (j >= 0) {
-      if (nk >= (uint32_t)b.N) { atomicOr(b.status, ST_BOUNDS); nk = 0; }
-      const Rec* rp = b.rec + ((int64_t)ti.v * b.N + nk);
-      cp_async16(&sh.raw[0][lane], &rp->a);
-      cp_async16(&sh.raw[1][lane], &rp->b);
-      cp_async16(&sh.raw[2][lane], &rp->c);
-    }
-    cp_async_commit();
-  };
-  load_key(maxlast - lane);
-  copy_record(maxlast - lane);
-  uint32_t g = nk;
-  load_key(maxlast - 32 - lane);
   int head = 0, have = 0;  // ring index of the next group, items in the ring
   for (; top >= 0; top -= 32) {
     cp_async_wait<0>();
     // append the lane's entry if it can reach a pixel of the block
     uint32_t m = 0;
     float4 A, B, C;
-    if (top - lane >= 0 && (!kSync || top - lane <= mylast)) {
+    if (top - lane >= 0 && top - lane <= mylast) {
       A = sh.raw[0][lane];
       B = sh.raw[1][lane];
       C = sh.raw[2][lane];
