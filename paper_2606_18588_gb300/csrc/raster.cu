@@ -192,7 +192,7 @@ constexpr float kWild = 1e18f;
 // warp-entries of the 2M-Gaussian, 4-view step), and it takes them two at a time with the
 // exponents of both in packed FP32 instructions, without a branch per pixel.  Measured on
 // that step (8 subsets, no skipping, 16x16 tiles): 2.89 -> 2.12 ms, 3.07e9 -> 2.06e9 warp
-// instructions; 8x8 tiles 3.39 -> 1.96 ms, 32x32 4.14 -> 3.91 ms; the 10M step 58.4
+// instructions; 8x8 tiles 3.39 -> 1.96 ms, 32x32 4.14 -> 3.78 ms; the 10M step 58.4
 // -> 55.5 ms.  Packing the colours too (channel pairs, with w moved into both halves) took
 // 2.37 ms, a branch per stopping pair 2.46 ms, 10 CTAs per SM at 48 registers (spilling)
 // and 7 at 72 1-2 % more than 8 at 64.
@@ -352,72 +352,76 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, co
     const int j0 = __float_as_int(MJ.z), j1 = __float_as_int(MJ.w);
     const f32x2 u2 = pack2(P0.x, P0.y), v2 = pack2(P0.z, P0.w), qa2 = pack2(P1.x, P1.y),
                 qb2 = pack2(P1.z, P1.w), qc2 = pack2(P2.x, P2.y), o2 = pack2(P2.z, P2.w);
-    f32x2 hx2[NC], bx2[NC], dy2[2];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const f32x2 dx2 = sub2(c ? pcx1 : pcx0, u2);
-      hx2[c] = mul2(mul2(qa2, dx2), dx2);
-      bx2[c] = mul2(qb2, dx2);
-    }
-    dy2[0] = sub2(pcy0, v2);
-    dy2[1] = sub2(pcy1, v2);
-    float al0[PPT], al1[PPT], T0[PPT], T1[PPT];
-    bool ok0[PPT], ok1[PPT];
-    float tmin = __int_as_float(0x7f800000);
-#pragma unroll
-    for (int i = 0; i < PPT; ++i) {
-      const f32x2 dy = dy2[slot_row<PPT>(i)];
-      const f32x2 p2 = fma2(fma2(qc2, dy, bx2[slot_col<PPT>(i)]), dy, hx2[slot_col<PPT>(i)]);
-      float p0, p1, r0, r1;
-      unpack2(p2, p0, p1);
-      unpack2(mul2(o2, pack2(ex2_approx(p0), ex2_approx(p1))), r0, r1);
-      const bool in0 = (~m0 & pm[i]) == 0u, in1 = (~m1 & pm[i]) == 0u;
-      ok0[i] = in0 && p0 <= 0.0f && r0 >= amin_raw;
-      ok1[i] = in1 && p1 <= 0.0f && r1 >= amin_raw;
-      if (kCount) n_pix += (unsigned)in0 + (unsigned)in1;
-      al0[i] = ok0[i] ? fminf(r0, amax) : 0.0f;
-      al1[i] = ok1[i] ? fminf(r1, amax) : 0.0f;
-      T0[i] = T[i] * (1.0f - al0[i]);
-      T1[i] = T0[i] * (1.0f - al1[i]);
-      tmin = fminf(tmin, T1[i]);
-    }
+    const f32x2 dy2[2] = {sub2(pcy0, v2), sub2(pcy1, v2)};
     head += 2;
     if (kCount && lane == 0) n_eval += 2u;
-    if (__any_sync(0xffffffffu, tmin < epsT)) {
-      // a pixel stops before the entry that would take it below eps_T: that entry and what
-      // follows leave it as it is
+    // a column of blocks (two slots) at a time; of a 16 x 8 region's two, those that the pair's
+    // rectangles meet (a small Gaussian meets one: 32x32 tiles, the 2M step 3.99 -> 3.78 ms,
+    // 3M Gaussians of a pixel or less 2.15 -> 1.96; a test per slot spilled and took 5.4)
 #pragma unroll
-      for (int i = 0; i < PPT; ++i) {
-        const bool s0 = ok0[i] && T0[i] < epsT;
-        const bool s1 = s0 || (ok1[i] && T1[i] < epsT);
-        ok0[i] = ok0[i] && !s0;
-        ok1[i] = ok1[i] && !s1;
-        T0[i] = s0 ? T[i] : T0[i];
-        T1[i] = s1 ? T0[i] : T1[i];
-        al0[i] = s0 ? 0.0f : al0[i];
-        al1[i] = s1 ? 0.0f : al1[i];
-        pm[i] = s1 ? kDeadPixel : pm[i];
-      }
-    }
+    for (int c = 0; c < NC; ++c) {
+      if (NC > 1 && (((m0 | m1) >> (8 + 8 * c)) & 0xFFu) == 0u) continue;
+      const f32x2 dx2 = sub2(c ? pcx1 : pcx0, u2);
+      const f32x2 hx2 = mul2(mul2(qa2, dx2), dx2), bx2 = mul2(qb2, dx2);
+      float al0[2], al1[2], T0[2], T1[2];
+      bool ok0[2], ok1[2];
+      float tmin = __int_as_float(0x7f800000);
 #pragma unroll
-    for (int i = 0; i < PPT; ++i) {
-      const float w0 = al0[i] * T[i], w1 = al1[i] * T0[i];
-      T[i] = T1[i];
-      if (ok0[i]) {
-        c0[i] = fmaf(CA.x, w0, c0[i]);
-        c1[i] = fmaf(CA.y, w0, c1[i]);
-        c2[i] = fmaf(CA.z, w0, c2[i]);
-        D[i] = fmaf(CA.w, w0, D[i]);
+      for (int r = 0; r < 2; ++r) {
+        const int i = NC * r + c;
+        const f32x2 dy = dy2[r];
+        const f32x2 p2 = fma2(fma2(qc2, dy, bx2), dy, hx2);
+        float p0, p1, r0, r1;
+        unpack2(p2, p0, p1);
+        unpack2(mul2(o2, pack2(ex2_approx(p0), ex2_approx(p1))), r0, r1);
+        const bool in0 = (~m0 & pm[i]) == 0u, in1 = (~m1 & pm[i]) == 0u;
+        ok0[r] = in0 && p0 <= 0.0f && r0 >= amin_raw;
+        ok1[r] = in1 && p1 <= 0.0f && r1 >= amin_raw;
+        if (kCount) n_pix += (unsigned)in0 + (unsigned)in1;
+        al0[r] = ok0[r] ? fminf(r0, amax) : 0.0f;
+        al1[r] = ok1[r] ? fminf(r1, amax) : 0.0f;
+        T0[r] = T[i] * (1.0f - al0[r]);
+        T1[r] = T0[r] * (1.0f - al1[r]);
+        tmin = fminf(tmin, T1[r]);
       }
-      if (ok1[i]) {
-        c0[i] = fmaf(CB.x, w1, c0[i]);
-        c1[i] = fmaf(CB.y, w1, c1[i]);
-        c2[i] = fmaf(CB.z, w1, c2[i]);
-        D[i] = fmaf(CB.w, w1, D[i]);
+      if (__any_sync(0xffffffffu, tmin < epsT)) {
+        // a pixel stops before the entry that would take it below eps_T: that entry and what
+        // follows leave it as it is
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int i = NC * r + c;
+          const bool s0 = ok0[r] && T0[r] < epsT;
+          const bool s1 = s0 || (ok1[r] && T1[r] < epsT);
+          ok0[r] = ok0[r] && !s0;
+          ok1[r] = ok1[r] && !s1;
+          T0[r] = s0 ? T[i] : T0[r];
+          T1[r] = s1 ? T0[r] : T1[r];
+          al0[r] = s0 ? 0.0f : al0[r];
+          al1[r] = s1 ? 0.0f : al1[r];
+          pm[i] = s1 ? kDeadPixel : pm[i];
+        }
       }
-      last[i] = ok0[i] ? j0 : last[i];
-      last[i] = ok1[i] ? j1 : last[i];
-      if (kCount) n_blend += (unsigned)ok0[i] + (unsigned)ok1[i];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int i = NC * r + c;
+        const float w0 = al0[r] * T[i], w1 = al1[r] * T0[r];
+        T[i] = T1[r];
+        if (ok0[r]) {
+          c0[i] = fmaf(CA.x, w0, c0[i]);
+          c1[i] = fmaf(CA.y, w0, c1[i]);
+          c2[i] = fmaf(CA.z, w0, c2[i]);
+          D[i] = fmaf(CA.w, w0, D[i]);
+        }
+        if (ok1[r]) {
+          c0[i] = fmaf(CB.x, w1, c0[i]);
+          c1[i] = fmaf(CB.y, w1, c1[i]);
+          c2[i] = fmaf(CB.z, w1, c2[i]);
+          D[i] = fmaf(CB.w, w1, D[i]);
+        }
+        last[i] = ok0[r] ? j0 : last[i];
+        last[i] = ok1[r] ? j1 : last[i];
+        if (kCount) n_blend += (unsigned)ok0[r] + (unsigned)ok1[r];
+      }
     }
   };
   bool open = alive();
