@@ -283,6 +283,7 @@ struct Plan {
   int ncells = 0, cell_self = -1;
   void* scan_temp = nullptr;
   int64_t capacity = 0, n_tiles = 0, total_pixels = 0;
+  int64_t pairs_seen = 0;  // pairs of the last forward that the host read (0: none)
   splx_opts opts{};
   std::vector<int64_t> tile_base, pix_off;
   // per-kernel timing: events at the marks below, recorded as graph event nodes when
@@ -329,6 +330,7 @@ struct Plan {
     b.n_tiles = n_tiles;
     b.tile_bits = bits_for(n_tiles + 1);
     b.capacity = capacity;
+    b.pairs = pairs_seen;
     b.eps_T = opts.eps_T; b.eps_comp = opts.eps_comp;
     b.alpha_min = opts.alpha_min; b.alpha_max = opts.alpha_max;
     for (int c = 0; c < 3; ++c) b.bg[c] = opts.bg[c];
@@ -607,6 +609,7 @@ struct Plan {
     CK(cudaMemcpyAsync(&t, tile_start + n_tiles, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     *total = t;
+    pairs_seen = t;
     return SPLX_OK;
   }
 };
@@ -1411,8 +1414,11 @@ int splx_batch_tune_prefix_sort(splx_batch_t bt, splx_stream_t stream) {
   CtxScope scope(P.ctx);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   unsigned long long c[kCounters] = {};
+  uint32_t total = 0;
   CK(cudaMemcpyAsync(c, P.counters, sizeof(c), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(&total, P.tile_start + P.n_tiles, sizeof(total), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  if (bt->forward_done) P.pairs_seen = total;
   // counters[8]: items walked on a selected prefix, [9]: items handed to the whole sort
   // counters[6]: items the waves left empty, [7]: items outside the visible regions
   const unsigned long long in = (unsigned long long)P.n_tiles - c[7];
@@ -1611,6 +1617,7 @@ int splx_batch_status(splx_batch_t bt, int64_t* pairs_out, splx_stream_t stream)
   CK(cudaMemcpyAsync(&st, P.ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (pairs_out) *pairs_out = (int64_t)total;
+  if (bt->forward_done) P.pairs_seen = total;
   if (st & ST_CAPACITY || total > (uint64_t)P.capacity) return SPLX_ERR_CAPACITY;
   if (st & ST_TIMEOUT) return SPLX_ERR_TIMEOUT;
   return SPLX_OK;
@@ -1791,6 +1798,7 @@ int srv_render(splx_server_s* S, SrvLaunch& L, uint64_t total) {
   Plan& P = L.P;
   int r;
   if (total >= (uint64_t)UINT32_MAX) return SPLX_ERR_CAPACITY;
+  P.pairs_seen = (int64_t)total;
   if ((r = P.alloc_pairs((int64_t)total, L.s))) return r;
   if ((r = P.fill_and_sort(L.s))) return r;
   BatchDev b = P.dev();

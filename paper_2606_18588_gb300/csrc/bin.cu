@@ -632,15 +632,23 @@ void launch_long_sort(const BatchDev& b, cudaStream_t s) {
 void launch_seg_sort(const BatchDev& b, cudaStream_t s) {
   if (b.n_tiles == 0) return;
   const int64_t items = items_of_launch(b);
-  // Tiles per CTA.  Short lists (by the room for pairs per tile: the true mean is not known
-  // here) go eight to a CTA, longer ones, which its tiles take in turn as whole CTAs, two: 1M
+  // Tiles per CTA, by the mean list: the pairs of an earlier forward where the host knows them,
+  // else four fifths of the room (a batch that sizes itself leaves a quarter).  Short lists go
+  // eight to a CTA, longer ones, which its tiles take in turn as whole CTAs, two or one: 1M
   // lists of 20 keys on average 0.42 ms at 8, 0.51 at 4, 0.74 at 2, 1.22 at 1; 170k lists of
-  // 180 keys 0.73, 0.69, 0.70, 0.77; 35k lists of 300 keys 0.28, 0.24, 0.23, 0.23.  Fewer
-  // where that would leave less than two CTAs of work for every resident one
-  int group = b.capacity < 128 * b.n_tiles ? kSortThreads / 32 : 2;
-  while (group > 1 && items < (int64_t)device_sm_count() * 12 * group) group /= 2;
+  // 180 keys 0.73, 0.69, 0.70, 0.77; 35k lists of 300 keys 0.28, 0.24, 0.23, 0.23; 27k lists
+  // of 440 in the middle of their views 0.234 at 2, 0.193 at 1.  Fewer where that would leave
+  // less than two CTAs of work for every resident one, and then, at one, without the exchange
+  // (kSolo), which in larger launches would have every warp look at every tile's pixels
+  const double mean = b.pairs > 0 ? (double)b.pairs / (double)b.n_tiles
+                                  : 0.8 * (double)b.capacity / (double)b.n_tiles;
+  const int want = mean < 100.0 ? kSortThreads / 32 : mean < 200.0 ? 2 : 1;
+  const int64_t fill = (int64_t)device_sm_count() * 12;
+  int group = want;
+  while (group > 1 && items < fill * group) group /= 2;
+  const bool solo = group == 1 && items < fill * 2;
   const unsigned grid = (unsigned)((items + group - 1) / group);
-  if (group == 1) k_seg_sort<true><<<grid, kSortThreads, 0, s>>>(b, 1);
+  if (solo) k_seg_sort<true><<<grid, kSortThreads, 0, s>>>(b, 1);
   else k_seg_sort<false><<<grid, kSortThreads, 0, s>>>(b, group);
   count_launch();
   // with selected prefixes no segment is left to the long-segment sort before the forward

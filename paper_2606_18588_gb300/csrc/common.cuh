@@ -92,6 +92,7 @@ struct BatchDev {
   int32_t tile_bits;            // bits of the image-tile id in a sort key
   int64_t n_tiles;              // image tiles over all (view, subset)
   int64_t capacity;             // pair capacity
+  int64_t pairs;                // pairs of an earlier forward (0: none known): launch shapes only
   float eps_T, eps_comp, alpha_min, alpha_max;
   float bg[3];
   const SubsetDev* subsets;     // [K]
@@ -368,6 +369,26 @@ __host__ __device__ __forceinline__ int64_t items_of_launch(const BatchDev& b) {
   return b.order ? b.item_n : b.n_tiles;
 }
 
+// Whether open(p) holds at a pixel of the tile with origin (x0, y0) (p: its index in the view's
+// planes).  Whole-warp call: eight pixels of a lane are read together, and the warp stops
+// there if one is open (32x32 tiles have 1024 pixels, one by one a chain of 32 reads).
+template <typename F>
+__device__ __forceinline__ bool tile_open(const BatchDev& b, const ViewDev& cam, int x0, int y0,
+                                          F&& open) {
+  const int tsh = __ffs(b.tile) - 1;  // the tile side is a power of two
+  const int n = b.tile * b.tile;
+  for (int i0 = (int)(threadIdx.x & 31); i0 < n; i0 += 256) {
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + 32 * u, x = x0 + (i & (b.tile - 1)), y = y0 + (i >> tsh);
+      if (i < n && x < cam.W && y < cam.H) any |= open((int64_t)y * cam.W + x);
+    }
+    if (__any_sync(0xffffffffu, any)) return true;
+  }
+  return false;
+}
+
 // Saturation skipping test of work item `id` in a wave after the first: true if every pixel
 // of its tile has prefix transmittance below eps_comp.  Whole-warp call; the rasteriser and
 // the segment sort take the same decision.
@@ -378,13 +399,7 @@ __device__ __forceinline__ bool item_saturated(const BatchDev& b, int64_t id) {
   const int64_t t = (id - b.tile_base[v]) % nt;
   const int x0 = (int)(t % cam.tiles_x) * b.tile, y0 = (int)(t / cam.tiles_x) * b.tile;
   const float* tp = b.tpre + b.pix_off[v];
-  const int tsh = __ffs(b.tile) - 1;  // the tile side is a power of two
-  bool open = false;
-  for (int i = threadIdx.x & 31; i < b.tile * b.tile; i += 32) {
-    const int x = x0 + (i & (b.tile - 1)), y = y0 + (i >> tsh);
-    if (x < cam.W && y < cam.H) open |= tp[(int64_t)y * cam.W + x] >= b.eps_comp;
-  }
-  return !__any_sync(0xffffffffu, open);
+  return !tile_open(b, cam, x0, y0, [&](int64_t p) { return tp[p] >= b.eps_comp; });
 }
 
 // Cross-boundary per-ray filtering (Sec. 8.1): whether a Gaussian of subset k whose support
@@ -423,13 +438,7 @@ __device__ __forceinline__ bool item_pruned(const BatchDev& b, int64_t id) {
   const int x0 = (int)(t % cam.tiles_x) * b.tile, y0 = (int)(t / cam.tiles_x) * b.tile;
   const uint8_t* sp = b.sat[v];
   const int rk = b.rank[v * b.K + k];
-  const int tsh = __ffs(b.tile) - 1;  // the tile side is a power of two
-  bool open = false;
-  for (int i = threadIdx.x & 31; i < b.tile * b.tile; i += 32) {
-    const int x = x0 + (i & (b.tile - 1)), y = y0 + (i >> tsh);
-    if (x < cam.W && y < cam.H) open |= (int)sp[(int64_t)y * cam.W + x] > rk;
-  }
-  return !__any_sync(0xffffffffu, open);
+  return !tile_open(b, cam, x0, y0, [&](int64_t p) { return (int)sp[p] > rk; });
 }
 
 // Two FP32 values in one 64-bit register pair, and the packed operations on them (sm_100 and
