@@ -257,6 +257,7 @@ struct Plan {
   // that little is skipped: saturation skipping then takes one sort and one forward instead
   // of K waves
   bool long_walks = false;
+  bool waves_ran = false;  // the last eager forward (its counters) ran saturation-skipping waves
   bool alt_in_keys = false;  // keys_alt = keys + capacity (one allocation, owned by keys)
   uint32_t* sel = nullptr;
   uint32_t* retry = nullptr;
@@ -1234,6 +1235,7 @@ int splx_batch_forward(splx_batch_t bt, float* out_rgb, float* out_T, splx_strea
   BatchDev b = P.dev();
   b.out_rgb = out_rgb;
   b.out_T = out_T;
+  if (!stream_capturing(s)) P.waves_ran = P.order_d && !P.stale();
   if (P.order_d && !P.stale()) {
     // saturation skipping: K waves, each sorting and rendering one subset of every view,
     // front to back
@@ -1428,7 +1430,10 @@ int splx_batch_tune_prefix_sort(splx_batch_t bt, splx_stream_t stream) {
   // views: 71 of 42,000 items skipped, 134 prefixes; sort and forward 2.5 ms in one launch
   // each, 3.5 ms in waves.  10M, 8 subsets, 16 views: 83,000 of 252,000 skipped; 20 ms with
   // nothing skipped, 13.7 ms in waves
-  const bool little_skipped = P.order_d && c[0] > 0 && 16 * c[6] < in && 64 * c[8] < in;
+  // (only the counters of waves say what waves skip; with a stale state, persistent CTAs or no
+  // order there are none to replace)
+  const bool little_skipped = P.order_d && P.waves_ran && !P.stale() && P.persist_grid == 0 &&
+                              c[0] > 0 && 16 * c[6] < in && 64 * c[8] < in;
   if (handed_back || little_skipped) {
     P.select_prefix = false;
     P.long_walks = true;
