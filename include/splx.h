@@ -318,15 +318,18 @@ int splx_batch_set_visibility(splx_batch_t b, int32_t enable);
  * was captured with).  Off while cross-boundary filtering is on, and for a pair capacity
  * of 2^31 or more. */
 int splx_batch_set_prefix_sort(splx_batch_t b, int32_t enable);
-/* Keeps the selected-prefix sort on only if the last eager forward handed at most a
- * quarter of its prefix items back to the whole sort (their pixels still blending at the
- * prefix's end: tiles with long lists of small or faint Gaussians), and turns it off
- * otherwise; with subset orders set, also where that forward's waves skipped under a
- * sixteenth of the work items inside the visible regions and under a 64th of them had such
- * a list.  With it off by this call, saturation skipping sorts every segment first and
- * renders all subsets in one launch, a tile's front to back, instead of waves (the same
- * results).  For launches issued afterwards; call it between an eager forward and a graph
- * capture.  Synchronises `stream`; not capturable; SPLX_ERR_INVALID without a batch state. */
+/* Decides from the counters of the last eager forward how launches issued afterwards sort.
+ * The selected-prefix sort stays on only if that forward handed at most a quarter of its
+ * prefix items back to the whole sort (their pixels still blending at the prefix's end: tiles
+ * with long lists of small or faint Gaussians).  With subset orders set, no stale state and
+ * one CTA per work item, and where prefixes went off, or that forward skipped under a
+ * sixteenth of the work items inside the visible regions and under a 64th of them had a
+ * prefix, saturation skipping sorts every segment whole and renders all subsets in one
+ * launch, a tile's front to back, instead of K waves (the same results).  That lasts until
+ * splx_batch_set_cameras, splx_batch_set_order or splx_batch_set_prefix_sort; a captured graph
+ * keeps the mode it was captured with.  May be called again after another eager forward.  Call
+ * it between an eager forward and a graph capture.  Synchronises `stream`; not capturable;
+ * SPLX_ERR_INVALID without a batch state. */
 int splx_batch_tune_prefix_sort(splx_batch_t b, splx_stream_t stream);
 /* Cross-boundary per-ray filtering (Sec. 8.1, appendix "Cross-boundary Gaussians
  * Handling").  cells (host, [K][6] floats: lo x, y, z, hi x, y, z of subset k's k-d box,

@@ -252,12 +252,12 @@ struct Plan {
   uint2* chunks_g[kGroups - 1] = {};
   // selected-prefix sort of long segments (batches; see BatchDev::sel): per image tile the
   // prefix length, and per view group the forward's retry list and its count
-  bool select_prefix = false;
+  bool select_prefix = false, prefix_wanted = false;  // ... and the caller's switch
   // the tuning found that lists are walked to their ends (selected prefixes handed back) or
-  // that little is skipped: saturation skipping then takes one sort and one forward instead
-  // of K waves
-  bool long_walks = false;
-  bool waves_ran = false;  // the last eager forward (its counters) ran saturation-skipping waves
+  // that little is skipped: saturation skipping then takes whole sorts and one forward
+  // instead of K waves, until the views or their orders change
+  bool one_launch = false;
+  bool skipping_ran = false;  // the last eager forward (its counters) skipped by exact waves
   bool alt_in_keys = false;  // keys_alt = keys + capacity (one allocation, owned by keys)
   uint32_t* sel = nullptr;
   uint32_t* retry = nullptr;
@@ -268,6 +268,8 @@ struct Plan {
   // the forward then runs one launch per stage and re-evaluates the states in place
   uint8_t** sat_d = nullptr;
   bool stale() const { return sat_d && order_d; }
+  // the forward skips in one launch (persistent CTAs, stale states and plain launches do not)
+  bool in_one_launch() const { return one_launch && order_d && !sat_d && persist_grid == 0; }
   uint32_t* omega = nullptr;               // [V][K][4] visible regions (internal partials only)
   bool visibility = false;                 // use omega (batches and server launches)
   float* tpre = nullptr;                   // [total pixels] prefix transmittance of the waves
@@ -365,7 +367,7 @@ struct Plan {
     b.sat = stale() ? sat_d : nullptr;
     b.rank = rank_d;
     // (the cross-boundary filter's removed pairs keep the whole-segment sort)
-    b.sel = select_prefix && alt_in_keys && sel && !b.removed ? sel : nullptr;
+    b.sel = select_prefix && alt_in_keys && sel && !b.removed && !in_one_launch() ? sel : nullptr;
     b.retry = retry;
     // composite-only plans carry no subsets; their offsets are unused
     for (int k = 0; k <= K; ++k) b.goff[k] = k < (int)subsets_h.size() ? subsets_h[k].goff : N;
@@ -457,7 +459,6 @@ struct Plan {
   // on their own streams, so that one group's kernels fill the others' wave tails; the
   // groups share nothing but the read-only inputs.
   int waves(const BatchDev& b, cudaStream_t s) {
-    const int64_t nw = n_tiles / K;
     // first view of each group; groups[G] = V
     int G = 1, first[kGroups + 1] = {0};
     if (split_views && persist_grid == 0 && V >= 2) {
@@ -471,7 +472,7 @@ struct Plan {
     }
     first[G] = V;
     mark_wave(0, s);
-    if (long_walks && !b.sel && persist_grid == 0) {
+    if (in_one_launch()) {
       // little is skipped where lists are walked to their ends, so sorting all segments
       // costs little, and 2 launches take the place of 3 K of every view group
       launch_seg_sort(b, s);
@@ -523,7 +524,6 @@ struct Plan {
       CK(cudaStreamWaitEvent(s, join_ev[g - 1], 0));
     }
     mark_wave(2 * K, s);
-    (void)nw;
     return SPLX_OK;
   }
 
@@ -575,7 +575,7 @@ struct Plan {
       for (int g = 0; g < kGroups - 1; ++g)
         if ((r = ctx_alloc_t(ctx, &retry_g[g], nt, s))) return r;
     CK(cudaMemsetAsync(sel, 0, sizeof(uint32_t) * nt, s));
-    select_prefix = true;
+    select_prefix = prefix_wanted = true;
     return SPLX_OK;
   }
 
@@ -1210,6 +1210,7 @@ int splx_batch_set_cameras(splx_batch_t bt, const splx_camera* cams, int32_t V, 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   CK(cudaStreamSynchronize(s));
   for (int v = 0; v < V; ++v) P.views_h[v] = make_view(cams[v], P.tile);
+  P.one_launch = false;  // (what the tuning found holds for the views it saw)
   CK(cudaMemcpyAsync(P.views_d, P.views_h.data(), sizeof(ViewDev) * V, cudaMemcpyHostToDevice, s));
   CK(cudaStreamSynchronize(s));
   return SPLX_OK;
@@ -1235,7 +1236,7 @@ int splx_batch_forward(splx_batch_t bt, float* out_rgb, float* out_T, splx_strea
   BatchDev b = P.dev();
   b.out_rgb = out_rgb;
   b.out_T = out_T;
-  if (!stream_capturing(s)) P.waves_ran = P.order_d && !P.stale();
+  if (!stream_capturing(s)) P.skipping_ran = P.order_d && !P.stale();
   if (P.order_d && !P.stale()) {
     // saturation skipping: K waves, each sorting and rendering one subset of every view,
     // front to back
@@ -1404,15 +1405,15 @@ int splx_batch_set_visibility(splx_batch_t bt, int32_t enable) {
 
 int splx_batch_set_prefix_sort(splx_batch_t bt, int32_t enable) {
   if (!bt || !bt->plan.sel) return SPLX_ERR_INVALID;
-  bt->plan.select_prefix = enable != 0;
-  bt->plan.long_walks = false;
+  bt->plan.select_prefix = bt->plan.prefix_wanted = enable != 0;
+  bt->plan.one_launch = false;
   return SPLX_OK;
 }
 
 int splx_batch_tune_prefix_sort(splx_batch_t bt, splx_stream_t stream) {
   if (!bt || !bt->plan.sel) return SPLX_ERR_INVALID;
   Plan& P = bt->plan;
-  if (!P.select_prefix || !P.counters) return SPLX_OK;
+  if (!P.prefix_wanted || !P.counters) return SPLX_OK;
   CtxScope scope(P.ctx);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   unsigned long long c[kCounters] = {};
@@ -1430,14 +1431,11 @@ int splx_batch_tune_prefix_sort(splx_batch_t bt, splx_stream_t stream) {
   // views: 71 of 42,000 items skipped, 134 prefixes; sort and forward 2.5 ms in one launch
   // each, 3.5 ms in waves.  10M, 8 subsets, 16 views: 83,000 of 252,000 skipped; 20 ms with
   // nothing skipped, 13.7 ms in waves
-  // (only the counters of waves say what waves skip; with a stale state, persistent CTAs or no
-  // order there are none to replace)
-  const bool little_skipped = P.order_d && P.waves_ran && !P.stale() && P.persist_grid == 0 &&
-                              c[0] > 0 && 16 * c[6] < in && 64 * c[8] < in;
-  if (handed_back || little_skipped) {
-    P.select_prefix = false;
-    P.long_walks = true;
-  }
+  // (only a forward that skipped counts what skipping leaves out, in waves or in one launch)
+  const bool little_skipped =
+      P.skipping_ran && c[0] > 0 && 16 * c[6] < in && 64 * c[8] < in;
+  if (handed_back) P.select_prefix = false;
+  P.one_launch = handed_back || little_skipped;
   return SPLX_OK;
 }
 
@@ -1445,6 +1443,7 @@ int splx_batch_set_order(splx_batch_t bt, const int32_t* order) {
   if (!bt) return SPLX_ERR_INVALID;
   Plan& P = bt->plan;
   CtxScope scope(P.ctx);
+  P.one_launch = false;  // (what the tuning found holds for the orders it saw)
   if (!order) {
     P.free_ptr((void*&)P.order_d, nullptr);
     P.free_ptr((void*&)P.rank_d, nullptr);
