@@ -322,10 +322,11 @@ int splx_batch_set_prefix_sort(splx_batch_t b, int32_t enable);
  * The selected-prefix sort stays on only if that forward handed at most a quarter of its
  * prefix items back to the whole sort (their pixels still blending at the prefix's end: tiles
  * with long lists of small or faint Gaussians).  With subset orders set, no stale state and
- * one CTA per work item, and where prefixes went off, or that forward skipped under a
- * sixteenth of the work items inside the visible regions and under a 64th of them had a
- * prefix, saturation skipping sorts every segment whole and renders all subsets in one
- * launch, a tile's front to back, instead of K waves (the same results).  That lasts until
+ * one CTA per work item, where the waves of that forward left few pairs unsorted (those of
+ * skipped work items and, where prefixes stay on, of the segments they served: under a
+ * sixteenth of all, or under half a million for each wave after the first), saturation
+ * skipping sorts every segment whole and renders all subsets in one launch, a tile's front
+ * to back, instead of K waves (the same results).  That lasts until
  * splx_batch_set_cameras, splx_batch_set_order or splx_batch_set_prefix_sort; a captured graph
  * keeps the mode it was captured with.  May be called again after another eager forward.  Call
  * it between an eager forward and a graph capture.  Synchronises `stream`; not capturable;

@@ -253,9 +253,8 @@ struct Plan {
   // selected-prefix sort of long segments (batches; see BatchDev::sel): per image tile the
   // prefix length, and per view group the forward's retry list and its count
   bool select_prefix = false, prefix_wanted = false;  // ... and the caller's switch
-  // the tuning found that lists are walked to their ends (selected prefixes handed back) or
-  // that little is skipped: saturation skipping then takes whole sorts and one forward
-  // instead of K waves, until the views or their orders change
+  // the tuning found that the waves leave little unsorted: saturation skipping then takes whole
+  // sorts and one forward instead of K waves, until the views or their orders change
   bool one_launch = false;
   bool skipping_ran = false;  // the last eager forward (its counters) skipped by exact waves
   bool alt_in_keys = false;  // keys_alt = keys + capacity (one allocation, owned by keys)
@@ -473,8 +472,8 @@ struct Plan {
     first[G] = V;
     mark_wave(0, s);
     if (in_one_launch()) {
-      // little is skipped where lists are walked to their ends, so sorting all segments
-      // costs little, and 2 launches take the place of 3 K of every view group
+      // the waves would leave little unsorted: 3 launches take the place of 4 K of every view
+      // group
       launch_seg_sort(b, s);
       BatchDev bo = b;
       bo.order = order_d;
@@ -1422,20 +1421,19 @@ int splx_batch_tune_prefix_sort(splx_batch_t bt, splx_stream_t stream) {
   CK(cudaMemcpyAsync(&total, P.tile_start + P.n_tiles, sizeof(total), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (bt->forward_done) P.pairs_seen = total;
-  // counters[8]: items walked on a selected prefix, [9]: items handed to the whole sort
-  // counters[6]: items the waves left empty, [7]: items outside the visible regions
-  const unsigned long long in = (unsigned long long)P.n_tiles - c[7];
-  const bool handed_back = c[8] > 0 && 4 * c[9] > c[8];
-  // skipping leaves out under a sixteenth of the items, and under a 64th have a long list: a
-  // sort of everything costs less than the waves' launches.  20M Gaussians, 32 subsets, 4
-  // views: 71 of 42,000 items skipped, 134 prefixes; sort and forward 2.5 ms in one launch
-  // each, 3.5 ms in waves.  10M, 8 subsets, 16 views: 83,000 of 252,000 skipped; 20 ms with
-  // nothing skipped, 13.7 ms in waves
-  // (only a forward that skipped counts what skipping leaves out, in waves or in one launch)
-  const bool little_skipped =
-      P.skipping_ran && c[0] > 0 && 16 * c[6] < in && 64 * c[8] < in;
-  if (handed_back) P.select_prefix = false;
-  P.one_launch = handed_back || little_skipped;
+  // selected prefixes pay unless most of them are too short ([8] walked, [9] handed back)
+  if (c[8] > 0 && 4 * c[9] > c[8]) P.select_prefix = false;
+  // One launch saves the waves' launches and tails, 10 to 50 us each, and sorts what the waves
+  // leave unsorted, 18 ps a key: the keys of the items that skipping empties ([10]) and, where
+  // prefixes stay, of the lists that they serve ([11]; only a forward that skipped counts
+  // these).  Measured (forward; waves with the sort that the tuning leaves them, one launch):
+  // 20M, 32 subsets, city, 0.3M such keys 5.41, 4.21 ms; 2M in 32, 6.8M 7.93, 5.98; 600k in 4,
+  // 0.1M 1.81, 1.64, 2.0M 1.30, 1.26; 2M in 8, 14M 3.21, 3.25; 1M in 2, 0.6M 1.94, 1.98; 10M
+  // in 8, 3.6M of 268M 50.6, 49.6, 95M of 355M (most prefixes handed back) 45.5, 47.1, 337M
+  // of 435M 29.7, 35.9
+  const unsigned long long more = c[10] + (P.select_prefix ? c[11] : 0ull);
+  P.one_launch = P.skipping_ran && total > 0 &&
+                 (16 * more < total || more < 500000ull * (unsigned)(P.K - 1));
   return SPLX_OK;
 }
 
@@ -1584,7 +1582,7 @@ int splx_batch_counters(splx_batch_t bt, int64_t* out, splx_stream_t stream) {
   CK(cudaMemcpyAsync(&total, P.tile_start + P.n_tiles, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   out[0] = (int64_t)total;
-  for (int i = 0; i < kCounters; ++i) out[1 + i] = (int64_t)c[i];
+  for (int i = 0; i < kPublicCounters; ++i) out[1 + i] = (int64_t)c[i];
   return SPLX_OK;
 }
 

@@ -9,7 +9,8 @@
 namespace splx {
 
 constexpr int kMaxK = 64;        // subsets per view
-constexpr int kCounters = 10;    // work counters of a batch (BatchDev::counters)
+constexpr int kCounters = 12;    // work counters of a batch (BatchDev::counters)
+constexpr int kPublicCounters = 10;  // ... of which splx_batch_counters reports the first
 constexpr int kMaxViews = 256;   // views per batch
 
 // Concatenated views of the D-SSIM loss: view v's [3][H][W] image at 3 * pix_off[v];
@@ -122,7 +123,8 @@ struct BatchDev {
   // [4] alpha evaluations, [5] contributions (alpha >= alpha_min); [6] work items left
   // empty by saturation skipping; [7] work items outside their subset's visible region;
   // [8] work items the forward walked on a selected prefix, [9] of those, the ones it
-  // handed to the full sort (see sel)
+  // handed to the full sort (see sel); [10] keys of the items of [6], [11] keys of the
+  // segments whose selected prefix was enough
   unsigned long long* counters;
   // selected-prefix sort (sel != nullptr; the batched path, with keys_alt = keys +
   // capacity and 2 capacity < 2^32): a tile segment longer than one sort chunk gets only

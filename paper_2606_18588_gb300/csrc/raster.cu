@@ -262,7 +262,10 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, co
           live &= ~(1u << i);
     }
     if (!__syncthreads_or(live != 0)) {
-      if (kCount && threadIdx.x == 0 && b.counters) atomicAdd(b.counters + 6, 1ull);
+      if (kCount && threadIdx.x == 0 && b.counters) {
+        atomicAdd(b.counters + 6, 1ull);
+        atomicAdd(b.counters + 10, (unsigned long long)len);
+      }
       const ImgDev im = b.imgs[ti.v * b.K + ti.k];
       const int64_t HW = (int64_t)ti.W * ti.H;
 #pragma unroll
@@ -550,6 +553,11 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, co
             im.last[(int64_t)py * ti.W + px] = -3 - last[i];
         }
         return;  // the second forward writes the prefix transmittance and the planes
+      }
+      if (threadIdx.x == 0 && kCount && b.counters) {
+        uint32_t s, e;
+        segment_of(b, pid, s, e);
+        atomicAdd(b.counters + 11, (unsigned long long)(e - s));
       }
     }
   }
@@ -964,9 +972,9 @@ __global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>) k_raster_fwd
 // one its own threads wrote.  The same items in the same order as the waves, so the same
 // results; it needs every segment sorted beforehand, also those that the waves would have
 // left unsorted behind saturated tiles, and no selected prefixes (a handed-back item would
-// have to be finished before the next).  For scenes whose lists are walked to their ends
-// (launch_raster_fwd_ordered's caller): 20M Gaussians, 32 subsets, 4 views at 1080p, sorts
-// and forward 3.5 ms in 128 launches of each kind.
+// have to be finished before the next).  For scenes whose waves leave little unsorted
+// (splx_batch_tune_prefix_sort): 20M Gaussians, 32 subsets, 4 views at 1080p, sorts and
+// forward 3.5 ms in 128 launches of each kind, 2.5 ms in three launches.
 template <int TS, int PPT, bool kCount>
 __global__ void __launch_bounds__(TS * TS / PPT, kMinBlocksFwd<TS>)
     k_raster_fwd_ordered(const BatchDev b) {

@@ -543,10 +543,10 @@ class Batch:
                "splx_batch_set_prefix_sort")
 
     def tune_prefix_sort(self, stream=None):
-        """Keeps the selected-prefix sort only if the last eager forward handed at most a
-        quarter of its prefix items back to the whole sort and, with subset orders set, skipped
-        or long lists are not rare; otherwise saturation skipping takes one sort and one
-        forward launch instead of waves (synchronises)."""
+        """Decides from the last eager forward's counters (synchronises): the selected-prefix
+        sort stays only if at most a quarter of its prefix items went back to the whole sort;
+        with subset orders set, waves that left few pairs unsorted give way to one sort and
+        one forward launch, until the cameras or orders change."""
         _check(_lib.splx_batch_tune_prefix_sort(self.h, _stream(stream)),
                "splx_batch_tune_prefix_sort")
 

@@ -45,12 +45,12 @@ def _open_scene(clump=4_000):
     return sc.take(perm), np.array([0, near.size, n + clump])
 
 
-def _batch(ctx, sc, off, cam=CAM):
+def _batch(ctx, sc, off, cam=CAM, capacity=1 << 20):
     from paper_2606_18588_gb300 import splx as S
     from gpu_util import subset_struct, to_device
     dev = to_device(sc)
     b = S.Batch(ctx, [subset_struct(dev, int(off[k]), int(off[k + 1]), 0)
-                      for k in range(len(off) - 1)], [cam], S.opts(), 1 << 20)
+                      for k in range(len(off) - 1)], [cam], S.opts(), capacity)
     b.keep = dev
     return b
 
@@ -131,32 +131,74 @@ def _walled_scene(x0, x1, n=3_000):
         parts.append(I.Scene(m, np.full((n, 3), -2.6, np.float32),
                              np.tile(np.float32([1, 0, 0, 0]), (n, 1)),
                              np.full(n, 4.0, np.float32), np.zeros((n, 1, 3), np.float32), 0))
-    faint = I.uniform_scene(2_000, 61, 0, log_scale_mu=-3.0, extent=1.0)
+    faint = I.uniform_scene(900_000, 61, 0, log_scale_mu=-2.6, extent=1.0)
     faint.means[:, 0] *= 2.4
-    faint.opacity_logits[:] = -3.0
+    faint.opacity_logits[:] = -4.5
     parts.append(faint)
     sc = I.Scene(*[np.concatenate(a) for a in zip(*[p.arrays() for p in parts])], 0)
-    return sc, np.array([0, n, 2 * n, 2 * n + 2_000])
+    return sc, np.array([0, n, 2 * n, 2 * n + 900_000])
 
 
 WALL_ORDER = np.array([[0, 1, 2]])
 
 
 def test_one_launch_is_weighed_again(ctx):
-    # found on a view that looks past the walls; then the camera moves before them: a forward
-    # in waves skips, and stays in waves
+    # found on a view that looks past the walls (and hands its prefixes back: whole sorts from
+    # then on); then the camera moves before them: a forward in waves skips, and stays in waves
     sc, off = _walled_scene(1.4, 2.6)
-    b = _batch(ctx, sc, off, I.pinhole(256, 192, 40.0, (-0.8, 0.0, -3.0), (-0.8, 0.0, 0.0)))
+    cam = I.pinhole(256, 192, 40.0, (-0.8, 0.0, -3.0), (-0.8, 0.0, 0.0))
+    b = _batch(ctx, sc, off, cam, 1 << 23)
     b.set_order(WALL_ORDER)
     waves, _, c = _launches(ctx, b)
-    assert c["skipped_items"] == 0
+    assert c["skipped_items"] == 0 and 4 * c["retried_items"] > c["prefix_items"] > 0
     b.tune_prefix_sort()
-    one = _launches(ctx, b)[0]
-    assert one < waves
+    waves -= 3  # (no second forward)
+    assert _launches(ctx, b)[0] == waves - 6  # 3 x (sort, long sort, forward) - 3
     b.set_cameras([I.pinhole(256, 192, 30.0, (2.0, 0.0, -3.0), (2.0, 0.0, 0.0))])
     n, ref, c = _launches(ctx, b)
     assert n == waves and 4 * c["skipped_items"] > 192
     b.tune_prefix_sort()
     n, rgb, _ = _launches(ctx, b)
     assert n == waves and torch.equal(rgb, ref)
+    b.close()
+
+
+def _wall(rng, n, x, y, z, ls):
+    m = np.stack([rng.uniform(*x, n), rng.uniform(*y, n), rng.uniform(z, z + 0.1, n)], 1)
+    return I.Scene(m.astype(np.float32), np.full((n, 3), ls, np.float32),
+                   np.tile(np.float32([1, 0, 0, 0]), (n, 1)), np.full(n, 4.0, np.float32),
+                   np.zeros((n, 1, 3), np.float32), 0)
+
+
+@pytest.mark.parametrize("form", ["handed back", "few items"])
+def test_waves_stay_where_skipping_saves_most_keys(ctx, form):
+    """Two walls and what they hide.  "handed back": faint Gaussians everywhere, whose lists
+    outlast their prefixes beside the walls, where most of them are, behind them.  "few
+    items": a clump behind a small part of walls that fill the view, so that few items are
+    skipped, with most of the keys."""
+    rng = np.random.default_rng(8)
+    if form == "handed back":
+        cam = I.pinhole(256, 192, 60.0, (0.0, 0.0, -3.0), (0.0, 0.0, 0.0))
+        walls = [_wall(rng, 4_000, (-0.5, 1.3), (-0.9, 0.9), z, -2.8) for z in (-1.3, -1.15)]
+        back = I.uniform_scene(400_000, 5, 0, log_scale_mu=-2.6, extent=1.0)
+        back.means[:, :2] *= 1.7
+        back.opacity_logits[:] = -4.0
+    else:
+        cam = I.pinhole(512, 384, 60.0, (0.0, 0.0, -3.0), (0.0, 0.0, 0.0))
+        walls = [_wall(rng, 9_000, (-1.3, 1.3), (-1.0, 1.0), z, -2.8) for z in (-1.3, -1.15)]
+        back = I.uniform_scene(40_000, 5, 0, log_scale_mu=-2.5, log_scale_sigma=0.1, extent=0.05)
+    parts = [*walls, back]
+    sc = I.Scene(*[np.concatenate(a) for a in zip(*[p.arrays() for p in parts])], 0)
+    b = _batch(ctx, sc, np.cumsum([0] + [p.n for p in parts]), cam, 1 << 23)
+    b.set_order(WALL_ORDER)
+    waves, ref, c = _launches(ctx, b)
+    inside = 3 * ((cam.width + 15) // 16) * ((cam.height + 15) // 16) - c["outside_items"]
+    if form == "handed back":
+        assert 4 * c["retried_items"] > c["prefix_items"] > 0
+    else:
+        assert 0 < 16 * c["skipped_items"] < inside and c["prefix_items"] == 0
+    b.tune_prefix_sort()
+    n, rgb, c = _launches(ctx, b)
+    assert n == (waves - 3 if form == "handed back" else waves) and torch.equal(rgb, ref)
+    assert c["prefix_items"] == 0  # (off where they were handed back)
     b.close()
