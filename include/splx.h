@@ -123,6 +123,12 @@ typedef struct {
 int splx_create(splx_ctx_t* out, int device, size_t hbm_budget_bytes);
 /* Synchronises the device, frees all scratch and the context. */
 int splx_destroy(splx_ctx_t ctx);
+/* Longest wait of a kernel of this context's later launches for work of the same launch (the
+ * sort of long tile lists), in polls of about half a microsecond: 0 (give up at once) to 2^20
+ * (the default, half a second; an item waits tens of microseconds).  A wait that gives up
+ * leaves its list unsorted and the status SPLX_ERR_TIMEOUT: of the requests in a server's
+ * launch, else in splx_device_status (and splx_batch_status). */
+int splx_set_wait_limit(splx_ctx_t ctx, int32_t polls);
 /* Scratch bytes currently held by the context (host value). */
 size_t splx_scratch_bytes(splx_ctx_t ctx);
 
@@ -133,7 +139,8 @@ size_t splx_scratch_bytes(splx_ctx_t ctx);
  * tile's list by depth with the Gaussian index as tie-break, front-to-back blending into
  * `out` (sized to cam->width x cam->height).  If state_out is non-NULL the projected
  * records and sorted lists are kept for splx_backward and must be released with
- * splx_state_release.  Synchronises once (to size the pair list). */
+ * splx_state_release.  Synchronises once (to size the pair list); what the device finds
+ * after that (a wait that gave up: the image is not valid) shows in splx_device_status. */
 int splx_render_partial(splx_ctx_t ctx, const splx_gaussians* subset, const splx_camera* cam,
                         const splx_opts* opts, const splx_partial* out, splx_state_t* state_out,
                         splx_stream_t stream);
@@ -436,7 +443,8 @@ int splx_server_submit(splx_server_t s, const splx_camera* cam, const int32_t* o
 /* Scheduling pass (never waits on the device): retires finished launches, renders
  * launches whose pair count has arrived, admits queued requests into idle slots; then
  * reports up to `cap` finished requests as (ids[i], status[i]) host arrays, *n_out of
- * them.  status is SPLX_OK or the error that ended the request. */
+ * them.  status is SPLX_OK or the error that ended the request (SPLX_ERR_TIMEOUT: a wait of
+ * its launch gave up; the request's image is not valid). */
 int splx_server_poll(splx_server_t s, int64_t* ids, int32_t* status, int32_t cap,
                      int32_t* n_out);
 /* Host outputs (each nullable): queued requests, requests in flight, reserved bytes. */
@@ -489,7 +497,8 @@ int splx_render_partial_noalloc(const splx_gaussians* subset, const splx_camera*
 
 /* ---- diagnostics ---------------------------------------------------------------- */
 /* Synchronises `stream`, returns and clears the context's device status word
- * (SPLX_OK, SPLX_ERR_CAPACITY or SPLX_ERR_TIMEOUT). */
+ * (SPLX_OK, SPLX_ERR_CAPACITY, SPLX_ERR_TIMEOUT or SPLX_ERR_STATE), with what finished server
+ * launches left in theirs. */
 int splx_device_status(splx_ctx_t ctx, splx_stream_t stream);
 /* Text of a status code (static storage). */
 const char* splx_strerror(int status);

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -96,6 +97,14 @@ int cuda_fail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, "kernel launch");       \
   } while (0)
 
+// The error a device status word reports.
+int status_code(int st) {
+  if (st & ST_CAPACITY) return SPLX_ERR_CAPACITY;
+  if (st & ST_TIMEOUT) return SPLX_ERR_TIMEOUT;
+  if (st & ST_BOUNDS) return SPLX_ERR_STATE;
+  return SPLX_OK;
+}
+
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 }  // namespace
@@ -107,6 +116,8 @@ struct splx_ctx_s {
   size_t in_use = 0;
   cudaMemPool_t pool = nullptr;
   int* d_status = nullptr;
+  std::atomic<int> launch_status{0};  // what launches with a status word of their own left
+  std::atomic<int> wait_polls{kWaitPolls};
   int64_t launches = 0;
   std::mutex mu;
   std::unordered_map<void*, size_t> sizes;
@@ -237,6 +248,7 @@ struct Plan {
   // serve launches without waves)
   unsigned* sort_counts = nullptr;
   uint2* ranges = nullptr;
+  int* status = nullptr;  // the plan's own status word (server launches), else the context's
   float4* grad2d = nullptr;
   uint8_t* defer = nullptr;  // [ceil(N / 128)]: blocks left to the zero-gradient Adam pass
   float* scales = nullptr;   // [8]: the update step's bias-corrected rates
@@ -341,7 +353,8 @@ struct Plan {
     b.keys = keys; b.keys_alt = keys_alt; b.chunks = chunks;
     b.seg_done = seg_done; set_sort_counts(b, sort_counts);
     b.ranges = ranges; b.grad2d = grad2d;
-    b.status = ctx->d_status;
+    b.status = status ? status : ctx->d_status;
+    b.wait_polls = ctx->wait_polls.load(std::memory_order_relaxed);
     b.counters = counters;
     b.persist_grid = persist_grid;
     b.work_ctr = work_ctr;
@@ -387,7 +400,7 @@ struct Plan {
     void** ps[] = {(void**)&subsets_d, (void**)&views_d, (void**)&imgs_d, (void**)&rec,
                    (void**)&counts, (void**)&tile_cnt, (void**)&tile_start, (void**)&keys,
                    (void**)&keys_alt, (void**)&seg_done, (void**)&sort_counts, (void**)&chunks,
-                   (void**)&ranges,
+                   (void**)&ranges, (void**)&status,
                    (void**)&grad2d, (void**)&defer, (void**)&scales, (void**)&scan_temp, (void**)&counters, (void**)&work_ctr,
                    (void**)&order_d, (void**)&rank_d, (void**)&sat_d, (void**)&tpre,
                    (void**)&omega, (void**)&cells_d,
@@ -1663,7 +1676,7 @@ struct SrvLaunch {
   // device timeline of the launch: before its first kernel, after its projection and tile
   // counts (the pair count's copy), after its last copy-out
   cudaEvent_t t_begin = nullptr, t_counted = nullptr, t_end = nullptr;
-  uint32_t* total_h = nullptr;
+  uint32_t* total_h = nullptr;  // pinned: the pair count, the status word
   Plan P;
   float* partial = nullptr;
   int32_t* last = nullptr;
@@ -1775,6 +1788,9 @@ int srv_start(splx_server_s* S, SrvLaunch& L) {
   if ((r = P.alloc_common(L.s))) return r;
   if ((r = ctx_alloc_t(S->ctx, &P.omega, (size_t)4 * V * K, L.s))) return r;
   P.visibility = true;
+  // a status word of the launch's own: a wait that gave up fails its requests, not others'
+  if ((r = ctx_alloc_t(S->ctx, &P.status, 1, L.s))) return r;
+  CK(cudaMemsetAsync(P.status, 0, sizeof(int), L.s));
   bool ordered = true;
   for (const SrvReq& q : L.reqs) ordered = ordered && q.has_order;
   if (ordered) {  // saturation skipping for the launch: per-view orders, prefix buffer
@@ -1818,6 +1834,7 @@ int srv_render(splx_server_s* S, SrvLaunch& L, uint64_t total) {
     CK(cudaMemcpyAsync(L.reqs[v].out, L.out_cat + 3 * P.pix_off[v], bytes,
                        cudaMemcpyDeviceToDevice, L.s));
   }
+  CK(cudaMemcpyAsync(L.total_h + 1, P.status, sizeof(int), cudaMemcpyDeviceToHost, L.s));
   CK(cudaEventRecord(L.t_end, L.s));
   CK(cudaEventRecord(L.ev, L.s));
   L.phase = 2;
@@ -1842,6 +1859,12 @@ int srv_advance(splx_server_s* S) {
       continue;
     }
     if (L.phase == 2) {
+      const int st = (int)L.total_h[1];
+      if (st) {
+        S->ctx->launch_status.fetch_or(st);
+        srv_fail_launch(S, L, status_code(st));
+        continue;
+      }
       std::array<float, 3> t = {0.0f, 0.0f, 0.0f};
       cudaEvent_t marks[3] = {L.t_begin, L.t_counted, L.t_end};
       for (int i = 0; i < 3; ++i)
@@ -1959,7 +1982,7 @@ int splx_server_create(splx_ctx_t ctx, const splx_gaussians* subsets, int32_t K,
     if (e == cudaSuccess) e = cudaEventCreate(&L.t_begin);
     if (e == cudaSuccess) e = cudaEventCreate(&L.t_counted);
     if (e == cudaSuccess) e = cudaEventCreate(&L.t_end);
-    if (e == cudaSuccess) e = cudaMallocHost(&L.total_h, sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMallocHost(&L.total_h, 2 * sizeof(uint32_t));
   }
   if (e == cudaSuccess) e = cudaEventCreate(&S->epoch);
   if (e == cudaSuccess) e = cudaEventRecord(S->epoch, S->slots[0].s);
@@ -2137,9 +2160,12 @@ int splx_device_status(splx_ctx_t ctx, splx_stream_t stream) {
   CK(cudaMemcpyAsync(&st, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), s));
   CK(cudaStreamSynchronize(s));
-  if (st & ST_CAPACITY) return SPLX_ERR_CAPACITY;
-  if (st & ST_TIMEOUT) return SPLX_ERR_TIMEOUT;
-  if (st & ST_BOUNDS) return SPLX_ERR_STATE;
+  return status_code(st | ctx->launch_status.exchange(0));
+}
+
+int splx_set_wait_limit(splx_ctx_t ctx, int32_t polls) {
+  if (!ctx || polls < 0 || polls > kWaitPolls) return SPLX_ERR_INVALID;
+  ctx->wait_polls = polls;
   return SPLX_OK;
 }
 

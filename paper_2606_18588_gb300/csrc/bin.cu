@@ -539,14 +539,11 @@ __device__ __forceinline__ void merge_item(const uint64_t* src, uint64_t* dst, u
   }
 }
 
-// Longest wait of a long-sort item for the earlier items of its segment: polls of about
-// half a microsecond, half a second in all (an item takes tens of microseconds).
-constexpr int kSortPolls = 1 << 20;
-
 // The long segments' whole sort in one launch: item (0, c) sorts chunk c of the chunk list,
 // item (1 + r, c) produces chunk c's 4096 outputs of merge round r (run width 4096 << r).
 // CTAs take the items in that order from a counter, and an item of a round starts when its
-// segment's chunk items of the round before are counted done (seg_done).  The order makes
+// segment's chunk items of the round before are counted done (seg_done).  A wait longer than
+// b.wait_polls polls gives up: ST_TIMEOUT, the segment stays unsorted.  The order makes
 // the wait end: every earlier item was taken before and is held by a CTA that is running,
 // whether or not the whole grid is resident, and the earliest unfinished one never waits.
 // A segment merged in R rounds starts them in keys_alt when R is odd, so that its last round
@@ -590,7 +587,7 @@ __global__ void __launch_bounds__(kBigThreads) k_long_sort(const BatchDev b) {
         const volatile uint32_t* done = b.seg_done + t;
         const uint32_t need = q * long_chunks(n);
         int polls = 0;
-        while (*done < need && polls < kSortPolls) {
+        while (*done < need && polls < b.wait_polls) {
           __nanosleep(256);
           ++polls;
         }

@@ -118,6 +118,7 @@ struct BatchDev {
   // ge dx, ge dy, ge dx^2, ge dx dy, ge dy^2 (ge = dL/dpower / o), dL/do, dL/dcolour
   float4* grad2d;
   int* status;                  // device status word
+  int wait_polls;               // longest wait of the long-segment sort (kWaitPolls)
   // work counters (nullable; kept by eager runs): forward [0] (warp, entry) pairs that meet,
   // [1] (pixel, entry) alpha evaluations, [2] blends; backward [3] (warp, entry) pairs,
   // [4] alpha evaluations, [5] contributions (alpha >= alpha_min); [6] work items left
@@ -223,6 +224,9 @@ constexpr uint32_t kSelNone = 0xFFFFFFFFu;
 constexpr uint32_t kSelResume = 0x80000000u;
 // largest selected prefix: keys sorted in shared memory by one sort CTA
 constexpr int kSelCap = 2048;
+// Longest wait of a long-sort item for the earlier items of its segment: polls of about
+// half a microsecond, half a second in all (an item takes tens of microseconds).
+constexpr int kWaitPolls = 1 << 20;
 // keys of one chunk of the long-segment sort
 constexpr uint32_t kSortChunk = 4096;
 

@@ -163,6 +163,7 @@ extern "C" int splx_render_partial_noalloc(const splx_gaussians* g, const splx_c
   b.rec = rec; b.counts = counts; b.tile_cnt = tile_cnt; b.tile_start = tile_start;
   b.keys = keys; b.keys_alt = keys_alt; b.chunks = chunks;
   b.seg_done = seg_done; set_sort_counts(b, sort_counts);
+  b.wait_polls = kWaitPolls;
   b.ranges = ranges; b.grad2d = nullptr; b.status = status; b.counters = nullptr;
   b.goff[0] = 0; b.goff[1] = N;
   b.tile_base[0] = 0; b.tile_base[1] = n_tiles;

@@ -121,6 +121,7 @@ _sigs = {
     "splx_graph_destroy": (C.c_int, [_P]),
     "splx_render_partial_noalloc": (C.c_int, [_P, _P, _P, _P, _P]),
     "splx_device_status": (C.c_int, [_P, _P]),
+    "splx_set_wait_limit": (C.c_int, [_P, C.c_int32]),
     "splx_strerror": (C.c_char_p, [C.c_int]),
     "splx_last_cuda_error": (C.c_char_p, []),
     "splx_launch_count": (C.c_int64, [_P]),
@@ -211,6 +212,11 @@ class Context:
     @property
     def launch_count(self) -> int:
         return int(_lib.splx_launch_count(self.h))
+
+    def set_wait_limit(self, polls: int):
+        """Longest wait of a later launch's kernels for each other's work, in polls of about half
+        a microsecond (0 to 2^20, the default)."""
+        _check(_lib.splx_set_wait_limit(self.h, int(polls)), "splx_set_wait_limit")
 
     def device_status(self, stream=None) -> int:
         return int(_lib.splx_device_status(self.h, _stream(stream)))
