@@ -19,7 +19,7 @@
 // image), a thread makes four outputs of a row and then four of a column, so that each staged
 // value is loaded once for four, tap sums run in registers with two statistics to a packed
 // instruction ((x, y) and (E[x^2], E[y^2]) sit side by side in shared memory for that), and
-// the loss is summed in float-float up to one FP64 add per CTA.  1920x1080x3: forward 128 ->
+// the loss is summed in FP32 parts (Sum3) up to one FP64 add per CTA.  1920x1080x3: forward 128 ->
 // 67 us, backward 102 -> 49 us (cold), the call 241 -> 126 us; the forward now issues on 79 %
 // of the slots.
 #include <cmath>
@@ -126,45 +126,70 @@ __device__ __forceinline__ void column_sums(const float2 (*ha)[kH], const float2
   }
 }
 
-// A sum of FP32 values in float-float (Knuth's TwoSum carries each addition's rounding
-// error): as good as FP64 for a few terms, at the FP32 rate.
-struct FloatSum {
-  float hi = 0.0f, lo = 0.0f;
+// A sum of FP32 values in three FP32 parts: Knuth's TwoSum carries every addition's rounding
+// error into the second part and the errors of those into the third, some 70 bits, so that a
+// CTA's thousand terms add up no worse than in FP64 (53 bits; a 64th of the FP32 rate, and two
+// parts would keep 48).
+struct Sum3 {
+  float hi, mid, lo;
+  __device__ __forceinline__ static float two_sum(float a, float b, float& err) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+  }
   __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(hi, v), bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb)));
-    hi = s;
+    float e1, e2;
+    hi = two_sum(hi, v, e1);
+    mid = two_sum(mid, e1, e2);
+    lo = __fadd_rn(lo, e2);
   }
-  __device__ __forceinline__ void add(const FloatSum& o) {
-    add(o.hi);
-    lo = __fadd_rn(lo, o.lo);
+  __device__ __forceinline__ void add(const Sum3& o) {
+    float e1, e2, e3;
+    hi = two_sum(hi, o.hi, e1);
+    mid = two_sum(mid, o.mid, e2);
+    mid = two_sum(mid, e1, e3);
+    lo = __fadd_rn(__fadd_rn(lo, o.lo), __fadd_rn(e2, e3));
   }
-  // the sum over groups of 2^steps lanes
-  __device__ __forceinline__ void reduce(int steps) {
-    for (int o = 1; o < 1 << steps; o <<= 1) {
-      FloatSum t;
-      t.hi = __shfl_xor_sync(0xffffffffu, hi, o);
-      t.lo = __shfl_xor_sync(0xffffffffu, lo, o);
-      add(t);
-    }
+  // with the lanes `o` away, over 2 o lanes
+  __device__ __forceinline__ void add_lane(int o) {
+    Sum3 t;
+    t.hi = __shfl_xor_sync(0xffffffffu, hi, o);
+    t.mid = __shfl_xor_sync(0xffffffffu, mid, o);
+    t.lo = __shfl_xor_sync(0xffffffffu, lo, o);
+    add(t);
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ double value() const {
+    // (an infinite sum has no error terms)
+    return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
+  }
 };
 
-// The CTA's sums of a and b, in thread 0 (red: one entry per warp).
-__device__ __forceinline__ void block_sums(FloatSum& a, FloatSum& b, float4* red) {
+// The CTA's sums of the threads' a and b, a's in thread 0 and b's in thread 16 (red: two
+// entries per warp).  A warp's first step leaves the a's in its lower half and the b's in the
+// upper one, so that the steps after it take one sum a lane.
+__device__ __forceinline__ Sum3 block_sums(const Sum3& a, const Sum3& b, Sum3* red) {
   constexpr int kWarps = kThreads / 32;
   static_assert(kWarps == 8, "the last three steps reduce eight warps");
-  a.reduce(5);
-  b.reduce(5);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float4(a.hi, a.lo, b.hi, b.lo);
+  const int lane = (int)(threadIdx.x & 31);
+  const bool up = lane >= 16;
+  Sum3 mine, t;
+  mine.hi = up ? b.hi : a.hi;
+  mine.mid = up ? b.mid : a.mid;
+  mine.lo = up ? b.lo : a.lo;
+  t.hi = __shfl_xor_sync(0xffffffffu, up ? a.hi : b.hi, 16);
+  t.mid = __shfl_xor_sync(0xffffffffu, up ? a.mid : b.mid, 16);
+  t.lo = __shfl_xor_sync(0xffffffffu, up ? a.lo : b.lo, 16);
+  mine.add(t);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) mine.add_lane(o);
+  if ((lane & 15) == 0) red[(up ? kWarps : 0) + (threadIdx.x >> 5)] = mine;
   __syncthreads();
   if (threadIdx.x < 32) {
-    const float4 v = red[threadIdx.x & (kWarps - 1)];
-    a.hi = v.x; a.lo = v.y; b.hi = v.z; b.lo = v.w;
-    a.reduce(3);
-    b.reduce(3);
+    mine = red[(up ? kWarps : 0) + (lane & (kWarps - 1))];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) mine.add_lane(o);
   }
+  return mine;
 }
 
 }  // namespace
@@ -176,7 +201,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_ssim_fwd(const LossImgs L, cons
   __shared__ __align__(16) float2 sxy[kS][kS];               // (x, y)
   __shared__ __align__(16) float2 hm[kS][kH], hq[kS][kH];    // row sums of (x, y), (x^2, y^2)
   __shared__ __align__(16) float hc[kS][kT];                 // ... of x y
-  __shared__ float4 red[kThreads / 32];
+  __shared__ Sum3 red[2 * kThreads / 32];
   const SsimItem it = decode(L, blockIdx.x);
   Taps tp;
   tp.load();
@@ -230,10 +255,11 @@ __global__ void __launch_bounds__(kThreads, 5) k_ssim_fwd(const LossImgs L, cons
   float cs[kCol];
   column_sums<true>(hm, hq, hc, r0, c, tp, m2, q2, cs);
   const int px = it.x0 + c;
-  FloatSum s_sum, l1_sum;
+  float ts[kCol], tl[kCol];  // S and |x - y| of the thread's pixels
 #pragma unroll
   for (int o = 0; o < kCol; ++o) {
     const int r = r0 + o, py = it.y0 + r;
+    ts[o] = tl[o] = 0.0f;
     if (px >= it.W || py >= it.H) continue;
     float mx, my, ex, ey;
     unpack2(m2[o], mx, my);
@@ -247,15 +273,21 @@ __global__ void __launch_bounds__(kThreads, 5) k_ssim_fwd(const LossImgs L, cons
     dmx[q] = 2.0f * my * (a2 - a1) * ib + 2.0f * mx * S * (rb2 - rb1);
     dexx[q] = -S * rb2;
     dexy[q] = 2.0f * a1 * ib;
-    s_sum.add(S);
     const float2 v = sxy[r + kR][c + kR];
-    l1_sum.add(fabsf(v.x - v.y));
+    ts[o] = S;
+    tl[o] = fabsf(v.x - v.y);
   }
-  block_sums(s_sum, l1_sum, red);
-  if (threadIdx.x == 0) {
-    atomicAdd(sums, s_sum.value());
-    atomicAdd(sums + 1, l1_sum.value());
+  Sum3 s_sum, l1_sum;
+  s_sum.hi = Sum3::two_sum(ts[0], ts[1], s_sum.mid);
+  l1_sum.hi = Sum3::two_sum(tl[0], tl[1], l1_sum.mid);
+  s_sum.lo = l1_sum.lo = 0.0f;
+#pragma unroll
+  for (int o = 2; o < kCol; ++o) {
+    s_sum.add(ts[o]);
+    l1_sum.add(tl[o]);
   }
+  const Sum3 sum = block_sums(s_sum, l1_sum, red);
+  if (threadIdx.x == 0 || threadIdx.x == 16) atomicAdd(sums + (threadIdx.x >> 4), sum.value());
 }
 
 __global__ void __launch_bounds__(kThreads, 5) k_ssim_bwd(const LossImgs L, const float* __restrict__ x,
