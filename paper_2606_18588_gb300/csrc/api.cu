@@ -218,12 +218,6 @@ ViewDev make_view(const splx_camera& c, int tile) {
   return v;
 }
 
-int bits_for(int64_t n) {
-  int b = 1;
-  while (b < 62 && (int64_t(1) << b) < n) ++b;
-  return b;
-}
-
 // A planned render of V views x K subsets.  The per-view entry points use V = 1 plans;
 // the batch API uses one plan for the whole batch.
 struct Plan {
@@ -342,7 +336,6 @@ struct Plan {
     std::memset(&b, 0, sizeof(b));
     b.V = V; b.K = K; b.sh_degree = deg; b.nc = n_sh(deg); b.N = N; b.tile = tile;
     b.n_tiles = n_tiles;
-    b.tile_bits = bits_for(n_tiles + 1);
     b.capacity = capacity;
     b.pairs = pairs_seen;
     b.eps_T = opts.eps_T; b.eps_comp = opts.eps_comp;

@@ -90,7 +90,6 @@ struct BatchDev {
   int32_t V, K, sh_degree, nc;  // nc = (deg+1)^2
   int64_t N;                    // Gaussians over all subsets
   int32_t tile;                 // tile side
-  int32_t tile_bits;            // bits of the image-tile id in a sort key
   int64_t n_tiles;              // image tiles over all (view, subset)
   int64_t capacity;             // pair capacity
   int64_t pairs;                // pairs of an earlier forward (0: none known): launch shapes only

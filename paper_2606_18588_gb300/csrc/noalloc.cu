@@ -152,9 +152,6 @@ extern "C" int splx_render_partial_noalloc(const splx_gaussians* g, const splx_c
   b.V = 1; b.K = 1; b.sh_degree = g->sh_degree; b.nc = n_sh(g->sh_degree); b.N = N;
   b.tile = tile;
   b.n_tiles = n_tiles;
-  int tb = 1;
-  while (tb < 62 && (int64_t(1) << tb) < n_tiles + 1) ++tb;
-  b.tile_bits = tb;
   b.capacity = kNoAllocMaxPairs;
   b.eps_T = o->eps_T; b.eps_comp = o->eps_comp; b.alpha_min = o->alpha_min;
   b.alpha_max = o->alpha_max;

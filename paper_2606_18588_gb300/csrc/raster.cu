@@ -180,8 +180,9 @@ template <int TS>
 constexpr int kNBFwd = TS == 8 ? 32 : 128;
 template <int TS, int PPT>
 constexpr int kRingWords = TS * TS / PPT / 32 * (kRingItems / 2) * kPairWords;  // all warps' rings
-// resident CTAs the backward's register limit is set for: 24 warps of 80 registers, as many
-// as its 9.3 KB of shared memory per warp leave room for
+// resident CTAs the backward's register limit is set for: 24 warps of 80 registers.  Six CTAs
+// of four warps and 37.2 KB fit an SM's 228 KB (1 KB of it per CTA is the system's); of 8x8
+// tiles' one-warp CTAs of 9.3 KB, 22 do
 template <int TS>
 constexpr int kMinBlocksBwd = TS == 8 ? 24 : 6;
 // above this an adjoint or a colour takes the backward's careful path
@@ -1044,12 +1045,14 @@ template <int TS>
 struct PptFwd {
   static constexpr int value = TS == 32 ? 4 : 2;
 };
-// Launches of at most this many 16x16 items take the backward's kSync form.  There one tile's
-// latency decides (a partial wave), and a Gaussian whose footprint lies inside one tile gets
-// its whole 2-D gradient by one add, so that small problems come out the same bit for bit
-// in every run; above it the tile's four warps add on their own, in any order.  Measured
-// (raster_bwd; before | warps on their own | kSync): 560 tiles 0.447 | 0.084 | 0.107 ms, 3800
-// tiles 0.523 | 0.133 | 0.179, 34.7k tiles 1.348 | 0.896 | 1.219.
+// Launches of at most this many 16x16 items take the backward's kSync form, for the sake of
+// repeatable sums: a Gaussian whose footprint lies inside one tile (or two: a sum of two adds
+// does not depend on their order) gets the same 2-D gradient bit for bit in every run, so that
+// small problems come out the same, as they did with a warp per tile.  It costs time: the
+// tile's warps wait for each other at every batch.  Larger launches leave each warp to add on
+// its own, in any order.  Measured (raster_bwd; a warp per tile | warps on their own | kSync):
+// 560 tiles 0.447 | 0.084 | 0.107 ms, 3800 tiles 0.523 | 0.133 | 0.179, 34.7k tiles 1.348 |
+// 0.896 | 1.219.
 constexpr int64_t kSyncItems = 1024;
 // Work is counted only by eager runs with a counter buffer: a captured graph launches the
 // plain variants, so replays carry no counting instructions (and keep the eager counts).
