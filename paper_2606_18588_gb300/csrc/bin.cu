@@ -631,21 +631,22 @@ void launch_seg_sort(const BatchDev& b, cudaStream_t s) {
   const int64_t items = items_of_launch(b);
   // Tiles per CTA, by the mean list: the pairs of an earlier forward where the host knows them,
   // else four fifths of the room (a batch that sizes itself leaves a quarter).  Short lists go
-  // eight to a CTA, longer ones, which its tiles take in turn as whole CTAs, two or one: 1M
-  // lists of 20 keys on average 0.42 ms at 8, 0.51 at 4, 0.74 at 2, 1.22 at 1; 170k lists of
-  // 180 keys 0.73, 0.69, 0.70, 0.77; 35k lists of 300 keys 0.28, 0.24, 0.23, 0.23; 27k lists
-  // of 440 in the middle of their views 0.234 at 2, 0.193 at 1.  Fewer where that would leave
-  // less than two CTAs of work for every resident one, and then, at one, without the exchange
-  // (kSolo), which in larger launches would have every warp look at every tile's pixels
+  // eight to a CTA, longer ones, which its tiles take in turn as whole CTAs, two: 1M lists of
+  // 20 keys on average 0.42 ms at 8, 0.51 at 4, 0.74 at 2, 1.22 at 1; 165k lists of 72 0.371,
+  // 0.355, 0.394, 0.490; 165k of 192 0.768, 0.709, 0.719, 0.761; 165k of 306 1.025, 0.970,
+  // 0.951, 0.961.  Fewer where that would leave less than two CTAs of work for every resident
+  // one.  A launch by itself (waves run beside other view groups' forwards) ends later the
+  // longer its last CTAs are: 14k lists of 116 0.066 ms at one tile per CTA, 0.076 at two; 27k
+  // of 680 0.193, 0.232; 42k of 249 0.242, 0.252, of 131 0.172 both; 54k of 269 0.305, 0.318,
+  // of 170 0.242, 0.240
   const double mean = b.pairs > 0 ? (double)b.pairs / (double)b.n_tiles
                                   : 0.8 * (double)b.capacity / (double)b.n_tiles;
-  const int want = mean < 100.0 ? kSortThreads / 32 : mean < 200.0 ? 2 : 1;
-  const int64_t fill = (int64_t)device_sm_count() * 12;
-  int group = want;
-  while (group > 1 && items < fill * group) group /= 2;
-  const bool solo = group == 1 && items < fill * 2;
+  const bool short_lists = mean < 100.0;
+  int group = short_lists ? kSortThreads / 32 : 2;
+  while (group > 1 && items < (int64_t)device_sm_count() * 12 * group) group /= 2;
+  if (!short_lists && !b.order && !b.sat && items < (mean < 200.0 ? 1 << 14 : 1 << 16)) group = 1;
   const unsigned grid = (unsigned)((items + group - 1) / group);
-  if (solo) k_seg_sort<true><<<grid, kSortThreads, 0, s>>>(b, 1);
+  if (group == 1) k_seg_sort<true><<<grid, kSortThreads, 0, s>>>(b, 1);
   else k_seg_sort<false><<<grid, kSortThreads, 0, s>>>(b, group);
   count_launch();
   // with selected prefixes no segment is left to the long-segment sort before the forward

@@ -1,5 +1,5 @@
-"""The segment sort's launch by the mean list (one tile per CTA for long lists of a large
-launch), and its test of a tile's pixels at every tile side: lists exactly as the binning
+"""The segment sort's launch by the mean list (one tile per CTA for long lists of a launch by
+itself), and its test of a tile's pixels at every tile side: lists exactly as the binning
 specification has them, and a stale saturation state's second visit equal to the waves."""
 import numpy as np
 import pytest
