@@ -11,13 +11,13 @@
 // tile's range ends before it.
 //
 // Sorting: a segment of up to 256 keys is sorted in shared memory by one warp, one of up to
-// 2048 keys by one CTA of 256 threads (8 keys per thread by a transposition network, then merge-path merges of runs).
-// Longer segments are cut into 4096-key chunks, each sorted the same way by a CTA of 512
-// threads, and then merged pairwise in rounds (run width 4096, 8192, ...) with merge-path
-// partitioning, one CTA per 4096 outputs, ping-ponging between the key buffer and its
-// twin so that the last round ends in the key buffer.  Chunk sorts and all rounds are one
-// launch (k_long_sort).  Every pair is read and written a few times instead of once per
-// 8-bit pass over 50+ key bits.
+// 2048 keys by one CTA of 256 threads (8 keys per thread by a transposition network, then
+// merge-path merges of runs).  Longer segments are cut into 4096-key chunks, each sorted the
+// same way by a CTA of 512 threads, and then merged pairwise in rounds (run width 4096, 8192,
+// ...) with merge-path partitioning, one CTA per 4096 outputs, ping-ponging between the key
+// buffer and its twin so that the last round ends in the key buffer.  Chunk sorts and all
+// rounds are one launch (k_long_sort).  Every pair is read and written a few times instead of
+// once per 8-bit pass over 50+ key bits.
 #include "common.cuh"
 #include "spec.cuh"
 #include "walk.cuh"

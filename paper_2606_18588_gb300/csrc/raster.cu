@@ -193,7 +193,7 @@ constexpr float kWild = 1e18f;
 // warp-entries of the 2M-Gaussian, 4-view step), and it takes them two at a time with the
 // exponents of both in packed FP32 instructions, without a branch per pixel.  Measured on
 // that step (8 subsets, no skipping, 16x16 tiles): 2.89 -> 2.12 ms, 3.07e9 -> 2.06e9 warp
-// instructions; 8x8 tiles 3.39 -> 1.96 ms, 32x32 4.14 -> 3.78 ms; the 10M step 58.4
+// instructions; 8x8 tiles 3.39 -> 1.94 ms, 32x32 4.14 -> 3.65 ms; the 10M step 58.4
 // -> 55.5 ms.  Packing the colours too (channel pairs, with w moved into both halves) took
 // 2.37 ms, a branch per stopping pair 2.46 ms, 10 CTAs per SM at 48 registers (spilling)
 // and 7 at 72 1-2 % more than 8 at 64.
@@ -360,7 +360,7 @@ __device__ __forceinline__ void fwd_item(const BatchDev& b, const int64_t id, co
     head += 2;
     if (kCount && lane == 0) n_eval += 2u;
     // a column of blocks (two slots) at a time; of a 16 x 8 region's two, those that the pair's
-    // rectangles meet (a small Gaussian meets one: 32x32 tiles, the 2M step 3.99 -> 3.78 ms,
+    // rectangles meet (a small Gaussian meets one: 32x32 tiles, the 2M step 3.91 -> 3.65 ms,
     // 3M Gaussians of a pixel or less 2.15 -> 1.96; a test per slot spilled and took 5.4)
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -599,10 +599,10 @@ struct BwdShared {
 // eight items at once (18 for a group) and no atomics but three per item and block.  Before,
 // one warp held a whole 16x16 tile, 8 pixels a lane, branched per 8 x 4 block and reduced
 // nine sums over its 32 lanes for every entry (some 50 instructions) or let up to 20 lanes
-// add their own.  2M Gaussians, 4 views, 8 subsets: 2.75 -> 2.15 ms at 16x16 tiles, 2.90 ->
-// 2.13 at 8x8, 4.55 -> 2.45 at 32x32; the 10M step's 17.5 -> 13.45 ms, the city's 3.6 ->
-// 2.42 ms.  Measured beside it: the one-warp tile with the packed arithmetic and box tests
-// alone 2.51 ms; one-warp CTAs 2.21 ms (the city 3.66: siblings share records in L1); the
+// add their own.  2M Gaussians, 4 views, 8 subsets: 2.75 -> 2.08 ms at 16x16 tiles, 2.90 ->
+// 2.12 at 8x8, 4.55 -> 2.34 at 32x32; the 10M step's 17.5 -> 13.0 ms, the city's 3.6 ->
+// 2.32 ms.  Measured beside it, when it took 2.15 ms: the one-warp tile with the packed
+// arithmetic and box tests alone 2.51 ms; one-warp CTAs 2.21 ms (the city 3.66: siblings share records in L1); the
 // group's four pairs not unrolled 2.22 ms; one warp taking a tile's four blocks in turn,
 // batch by batch, 2.41 ms (0.211 ms on 560 tiles).
 // kSync: the tile's warps take the batches of 32 entries together and leave their sums per

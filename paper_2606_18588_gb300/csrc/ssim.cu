@@ -19,9 +19,9 @@
 // image), a thread makes four outputs of a row and then four of a column, so that each staged
 // value is loaded once for four, tap sums run in registers with two statistics to a packed
 // instruction ((x, y) and (E[x^2], E[y^2]) sit side by side in shared memory for that), and
-// the loss is summed in FP32 parts (Sum3) up to one FP64 add per CTA.  1920x1080x3: forward 128 ->
-// 67 us, backward 102 -> 49 us (cold), the call 241 -> 126 us; the forward now issues on 79 %
-// of the slots.
+// the loss is summed in FP32 parts (Sum3) up to one FP64 add per CTA.  1920x1080x3: forward
+// 128 -> 67 us, backward 102 -> 49 us (cold; with sums in two parts), the call 241 -> 128 us;
+// the forward now issues on 79 % of the slots.
 #include <cmath>
 #include <cstring>
 
