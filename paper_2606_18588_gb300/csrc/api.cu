@@ -239,10 +239,11 @@ struct Plan {
   uint32_t* seg_done = nullptr;
   uint2* chunks = nullptr;
   // [kGroups][K][kSortCounts]: the sort counters of each view group's waves (the first ones
-  // serve launches without waves)
+  // serve launches without waves), and behind them the plan's own status word; cleared before
+  // every forward
   unsigned* sort_counts = nullptr;
+  bool own_status = false;  // kernels report to that word (server launches), not the context's
   uint2* ranges = nullptr;
-  int* status = nullptr;  // the plan's own status word (server launches), else the context's
   float4* grad2d = nullptr;
   uint8_t* defer = nullptr;  // [ceil(N / 128)]: blocks left to the zero-gradient Adam pass
   float* scales = nullptr;   // [8]: the update step's bias-corrected rates
@@ -346,7 +347,7 @@ struct Plan {
     b.keys = keys; b.keys_alt = keys_alt; b.chunks = chunks;
     b.seg_done = seg_done; set_sort_counts(b, sort_counts);
     b.ranges = ranges; b.grad2d = grad2d;
-    b.status = status ? status : ctx->d_status;
+    b.status = own_status ? status_word() : ctx->d_status;
     b.wait_polls = ctx->wait_polls.load(std::memory_order_relaxed);
     b.counters = counters;
     b.persist_grid = persist_grid;
@@ -393,7 +394,7 @@ struct Plan {
     void** ps[] = {(void**)&subsets_d, (void**)&views_d, (void**)&imgs_d, (void**)&rec,
                    (void**)&counts, (void**)&tile_cnt, (void**)&tile_start, (void**)&keys,
                    (void**)&keys_alt, (void**)&seg_done, (void**)&sort_counts, (void**)&chunks,
-                   (void**)&ranges, (void**)&status,
+                   (void**)&ranges,
                    (void**)&grad2d, (void**)&defer, (void**)&scales, (void**)&scan_temp, (void**)&counters, (void**)&work_ctr,
                    (void**)&order_d, (void**)&rank_d, (void**)&sat_d, (void**)&tpre,
                    (void**)&omega, (void**)&cells_d,
@@ -414,9 +415,9 @@ struct Plan {
     wev.clear();
   }
 
-  size_t sort_counts_bytes() const {
-    return sizeof(unsigned) * kSortCounts * kGroups * (size_t)std::max(K, 1);
-  }
+  size_t sort_counts_n() const { return (size_t)kSortCounts * kGroups * std::max(K, 1); }
+  size_t sort_counts_bytes() const { return sizeof(unsigned) * (sort_counts_n() + 1); }
+  int* status_word() const { return reinterpret_cast<int*>(sort_counts + sort_counts_n()); }
 
   // Project (counting pairs per tile) and scan the counts into segment starts.
   int project_and_count(cudaStream_t s) {
@@ -1781,9 +1782,7 @@ int srv_start(splx_server_s* S, SrvLaunch& L) {
   if ((r = P.alloc_common(L.s))) return r;
   if ((r = ctx_alloc_t(S->ctx, &P.omega, (size_t)4 * V * K, L.s))) return r;
   P.visibility = true;
-  // a status word of the launch's own: a wait that gave up fails its requests, not others'
-  if ((r = ctx_alloc_t(S->ctx, &P.status, 1, L.s))) return r;
-  CK(cudaMemsetAsync(P.status, 0, sizeof(int), L.s));
+  P.own_status = true;  // a wait that gave up fails this launch's requests, not others'
   bool ordered = true;
   for (const SrvReq& q : L.reqs) ordered = ordered && q.has_order;
   if (ordered) {  // saturation skipping for the launch: per-view orders, prefix buffer
@@ -1827,7 +1826,7 @@ int srv_render(splx_server_s* S, SrvLaunch& L, uint64_t total) {
     CK(cudaMemcpyAsync(L.reqs[v].out, L.out_cat + 3 * P.pix_off[v], bytes,
                        cudaMemcpyDeviceToDevice, L.s));
   }
-  CK(cudaMemcpyAsync(L.total_h + 1, P.status, sizeof(int), cudaMemcpyDeviceToHost, L.s));
+  CK(cudaMemcpyAsync(L.total_h + 1, P.status_word(), sizeof(int), cudaMemcpyDeviceToHost, L.s));
   CK(cudaEventRecord(L.t_end, L.s));
   CK(cudaEventRecord(L.ev, L.s));
   L.phase = 2;
