@@ -15,8 +15,11 @@
 // The thread per pixel stays where it is the better form.  One subset has no order (1M
 // Gaussians, 2 views 1600x1064: composite 24 us, adjoint 23; a patch 24 and 42).  More than
 // 16 subsets without regions go through local memory: 24 partials of 1600x1064, every pixel
-// covered, 0.90 ms, against 1.05 ms by the patches' array form, which stays for tiles with
-// more than 8 subsets of a launch with regions (K = 24, every tile with all: 1.08 ms).
+// covered, 0.74 ms (0.88 by the patches' array form, which is the one for tiles with more
+// than 8 subsets of a launch with regions: K = 24, all in every tile, two views 0.95 ms,
+// adjoint 1.39; 1.15 and 1.58 before the patches).  Both are bound by the insertion's moves
+// in local memory, which is why the order is a byte per subset (as ints, which leave L1:
+// 0.90 ms, and 1.08 and 1.67).
 //
 // Order: subsets sorted per pixel by the normalised depth D^m / (1 - T^m), a convex
 // combination of the subset's contributor depths (Eq. 4 read as D = sum d alpha T);
@@ -276,15 +279,18 @@ __device__ __forceinline__ void composite_bwd_patch(const BatchDev& b, const Pat
 }
 
 // More inside subsets than the register forms hold: the same, through arrays indexed at run
-// time (local memory).  All lanes run along (the planes' pointers come by shuffles).
+// time (local memory; kept small, a key and a byte per subset, so that they stay in L1: the
+// transmittances are read again where they are used).  All lanes run along (the planes'
+// pointers come by shuffles).
 struct PixOrderAny {
-  float T[kMaxK], key[kMaxK];
-  int ord[kMaxK];
+  float key[kMaxK];  // by subset
+  uint8_t ord[kMaxK];
+  Planes<true> pt;
 
   // kLoads: subsets whose planes are in flight together
   template <int kLoads>
   __device__ __forceinline__ int load(const BatchDev& b, const Patch& q) {
-    Planes<true> pt, pd;
+    Planes<true> pd;
     const ImgDev *a = lane_img(b, q, 0), *c = lane_img(b, q, 1);
     pt.set(a->T, c->T);
     pd.set(a->D, c->D);
@@ -306,14 +312,10 @@ struct PixOrderAny {
       for (int i = 0; i < kLoads; ++i) {
         if (m[i] < 0) continue;
         const float km = t[i] < 1.0f ? d[i] / (1.0f - t[i]) : __int_as_float(0x7f800000);
-        T[m[i]] = t[i];
         key[m[i]] = km;
         int j = n++;
-        while (j > 0 && key[ord[j - 1]] > km) {
-          ord[j] = ord[j - 1];
-          --j;
-        }
-        ord[j] = m[i];
+        for (int o; j > 0 && key[o = ord[j - 1]] > km; --j) ord[j] = (uint8_t)o;
+        ord[j] = (uint8_t)m[i];
       }
     }
     return n;
@@ -327,28 +329,33 @@ __device__ __noinline__ void composite_any(const BatchDev& b, const Patch& q) {
   pr.set(lane_img(b, q, 0)->rgb, lane_img(b, q, 1)->rgb);
   float P = 1.0f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
   for (int j0 = 0; j0 < n; j0 += kAhead) {
-    if (__all_sync(0xffffffffu, P < b.eps_comp)) break;
-    float r[kAhead], g[kAhead], bl[kAhead], w[kAhead];
+    const bool open = !(P < b.eps_comp);
+    if (!__any_sync(0xffffffffu, open)) break;
+    float r[kAhead], g[kAhead], bl[kAhead], t[kAhead];
 #pragma unroll
     for (int i = 0; i < kAhead; ++i) {
-      r[i] = g[i] = bl[i] = w[i] = 0.0f;
+      r[i] = g[i] = bl[i] = 0.0f;
+      t[i] = 1.0f;
       if (j0 + i < n) {
         const int m = po.ord[j0 + i];
         const float* rgb = pr.get<const float*>(m);
-        if (!(P < b.eps_comp)) {
+        const float* Tm = po.pt.get<const float*>(m);
+        if (open) {
           r[i] = rgb[q.p];
           g[i] = rgb[q.HW + q.p];
           bl[i] = rgb[2 * q.HW + q.p];
-          w[i] = P;
-          P *= po.T[m];
+          t[i] = Tm[q.p];
         }
       }
     }
 #pragma unroll
     for (int i = 0; i < kAhead; ++i) {
-      c0 = fmaf(r[i], w[i], c0);
-      c1 = fmaf(g[i], w[i], c1);
-      c2 = fmaf(bl[i], w[i], c2);
+      if (j0 + i < n && !(P < b.eps_comp)) {
+        c0 = fmaf(r[i], P, c0);
+        c1 = fmaf(g[i], P, c1);
+        c2 = fmaf(bl[i], P, c2);
+        P *= t[i];
+      }
     }
   }
   if (!q.in) return;
@@ -369,35 +376,49 @@ __device__ __noinline__ void composite_bwd_any(const BatchDev& b, const Patch& q
   // key[m] becomes the prefix P of the subsets before the cut, the first L in the order
   float P = 1.0f;
   int L = 0;
-  for (int j = 0; j < n; ++j) {
-    if (P < b.eps_comp) break;
-    const int m = po.ord[j];
-    po.key[m] = P;
-    P *= po.T[m];
-    ++L;
+  for (int j0 = 0; j0 < n; j0 += kAhead) {
+    if (!__any_sync(0xffffffffu, !(P < b.eps_comp))) break;
+    float t[kAhead];
+    int m[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      m[i] = j0 + i < n ? po.ord[j0 + i] : 0;
+      const float* Tm = po.pt.get<const float*>(m[i]);
+      t[i] = j0 + i < n ? Tm[q.p] : 1.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      if (j0 + i < n && !(P < b.eps_comp)) {
+        po.key[m[i]] = P;
+        P *= t[i];
+        ++L;
+      }
+    }
   }
   const float* dl = b.dL_drgb + 3 * b.pix_off[q.v];
   const float g0 = dl[q.p], g1 = dl[q.HW + q.p], g2 = dl[2 * q.HW + q.p];
   const float gT = b.dL_dT ? b.dL_dT[b.pix_off[q.v] + q.p] : 0.0f;
   float S0 = b.bg[0], S1 = b.bg[1], S2 = b.bg[2], Rt = 1.0f;
   for (int j1 = n - 1; j1 >= 0; j1 -= kAhead) {
-    float r[kAhead], g[kAhead], bl[kAhead];
+    float r[kAhead], g[kAhead], bl[kAhead], t[kAhead];
     float4* out[kAhead];
     int m[kAhead];
 #pragma unroll
     for (int i = 0; i < kAhead; ++i) {
       const int j = j1 - i;
-      r[i] = g[i] = bl[i] = 0.0f;
+      r[i] = g[i] = bl[i] = t[i] = 0.0f;
       m[i] = 0;
       out[i] = nullptr;
       if (j >= 0) {
         m[i] = po.ord[j];
         const float* rgb = pr.get<const float*>(m[i]);
+        const float* Tm = po.pt.get<const float*>(m[i]);
         out[i] = pg.get<float4*>(m[i]) + q.p;
         if (j < L) {
           r[i] = rgb[q.p];
           g[i] = rgb[q.HW + q.p];
           bl[i] = rgb[2 * q.HW + q.p];
+          t[i] = Tm[q.p];
         }
       }
     }
@@ -407,13 +428,13 @@ __device__ __noinline__ void composite_bwd_any(const BatchDev& b, const Patch& q
       if (j < 0) continue;
       float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
       if (j < L) {
-        const float Pm = po.key[m[i]], Tm = po.T[m[i]];
+        const float Pm = po.key[m[i]];
         const float gTm = (g0 * S0 + g1 * S1 + g2 * S2) * Pm + gT * Pm * Rt;
         o = make_float4(g0 * Pm, g1 * Pm, g2 * Pm, gTm);
-        S0 = fmaf(Tm, S0, r[i]);
-        S1 = fmaf(Tm, S1, g[i]);
-        S2 = fmaf(Tm, S2, bl[i]);
-        Rt *= Tm;
+        S0 = fmaf(t[i], S0, r[i]);
+        S1 = fmaf(t[i], S1, g[i]);
+        S2 = fmaf(t[i], S2, bl[i]);
+        Rt *= t[i];
       }
       if (q.in) *out[i] = o;
     }
@@ -461,7 +482,7 @@ __global__ void __launch_bounds__(256, kCompositeCtas<MK, kAny, kBwd>) k_composi
 template <int MK>
 struct PixOrderMany {
   float T[MK], key[MK];
-  int ord[MK];
+  uint8_t ord[MK];
 
   __device__ __forceinline__ void load(const BatchDev& b, int v, int64_t p) {
 #pragma unroll
@@ -481,7 +502,7 @@ struct PixOrderMany {
         ord[j] = ord[j - 1];
         --j;
       }
-      ord[j] = m;
+      ord[j] = (uint8_t)m;
     }
   }
 };
